@@ -75,24 +75,73 @@ __device__ __forceinline__ int kkt_comp(const KktArgs& a, int64_t s) {
 
 // Values: the KKT is cut into regions of uniform layout (the X rows of the nodes, the U rows,
 // the tf row, the boundary rows, the defect rows of each component), each with its own range
-// of blocks.  In the row regions a block takes KKT_ROWS consecutive periods (nodes or defect rows)
-// and its threads walk the block's output slots in order, so loads and stores are
-// coalesced; the period of a slot comes from a single-precision product (exact for the
-// block-local indices, see kkt_div) instead of an integer division, and the X / U templates
-// sit in shared memory.  Moved values are copied bit for bit; the (1,1) diagonal gets
-// sigma_x + delta_w, the constraint diagonal is -delta_c.
-constexpr int KKT_ROWS = 1024;
-constexpr int KKT_BATCH = 4;
+// of blocks.  A block takes KKT_SLOTS consecutive output slots of its region, whatever their
+// rows: every region, the tf row's (tx + tu)(N + 1) copied entries too, splits into blocks of
+// the same work, so that a mid-sized problem still fills the SMs.  (By 1024 periods of a row
+// region, or 262144 slots of the others, per block, the Goddard matrix at N = 1e5 put the tf row's 4e5
+// slots on two blocks: 475 us for 4.4e6 entries, and the quadrotor's at N = 33333 took 38 us in
+// 480 uneven blocks.)  Each thread issues the loads of all its KKT_PER slots before the
+// first store: the gather is latency-bound otherwise.  Loads and stores are coalesced; the period of a
+// slot comes from a single-precision product (see kkt_div) instead of an integer division, and
+// the X / U templates sit in shared memory.  Moved values are copied bit for bit; the (1,1)
+// diagonal gets sigma_x + delta_w, the constraint diagonal is -delta_c.
+constexpr int KKT_THREADS = 256, KKT_PER = 8;
+constexpr uint32_t KKT_SLOTS = KKT_THREADS * KKT_PER;
 enum { KR_X = 0, KR_U = 1, KR_TF = 2, KR_BND = 3, KR_DEF = 4, KR_XN = 5 };
 
-// floor(i / P) for block-local i < KKT_ROWS * P, P <= 1024: (i + 1/2) / P lies at least 1/(2P) >=
-// 2^-11 from an integer; its single-precision value (below KKT_ROWS = 2^10, computed from
-// 1/P rounded to nearest and a product rounded toward zero) is off by less than 2^-12.
+// floor(i / P) for block-local i < KKT_SLOTS + P, P <= 1024: (i + 1/2) / P lies at least 1/(2P) from
+// an integer; its single-precision value (1/P rounded to nearest, a product rounded toward
+// zero) is off by less than (i + 1/2) / P 2^-22 < 2^-10 / P.
 __device__ __forceinline__ uint32_t kkt_div(uint32_t i, float invP) {
   return (uint32_t)__fmul_rz((float)i + 0.5f, invP);
 }
 
-__global__ void __launch_bounds__(256) k_kkt_values(const __grid_constant__ KktArgs a) {
+template <int KIND>
+__device__ __forceinline__ void kkt_block(const KktArgs& a, const KRegion& R, uint32_t s0, const int16_t* s_src,
+                                          const int16_t* s_a, const uint8_t* s_diag) {
+  constexpr bool ROWS = KIND == KR_X || KIND == KR_U || KIND == KR_DEF;
+  const uint32_t n = min(KKT_SLOTS, R.len - s0);
+  const uint32_t P = R.period;
+  const uint32_t j0 = ROWS ? s0 / P : 0u, o0 = ROWS ? s0 - j0 * P : 0u;   // first period, offset in it
+  const float invP = 1.0f / (float)P;
+  // (the output never aliases the inputs: the loads of later slots may be issued before stores)
+  const double* __restrict__ src = ((KIND == KR_DEF || KIND == KR_BND) ? a.jv : a.hv) + R.src + (int64_t)j0 * R.stride;
+  double* __restrict__ out = a.out + R.out + s0;
+  double v[KKT_PER];
+#pragma unroll
+  for (int q = 0; q < KKT_PER; ++q) {
+    const uint32_t i = threadIdx.x + q * KKT_THREADS;
+    v[q] = 0.0;
+    if (i >= n) continue;
+    if constexpr (KIND == KR_DEF) {
+      const uint32_t u = i + o0, jl = kkt_div(u, invP);
+      v[q] = (u - jl * P + 1 == P) ? -a.dc : __ldg(src + (u - jl));   // u - jl: the diagonals before this slot
+    } else if constexpr (ROWS) {
+      const uint32_t u = i + o0, jl = kkt_div(u, invP), e = u - jl * P;
+      const int sp = s_src[e];
+      if (sp >= 0) v[q] = __ldg(src + (int64_t)R.stride * jl + sp);
+      if (s_diag[e]) {
+        const int64_t j = (int64_t)j0 + jl;
+        const int64_t row = (KIND == KR_X) ? (int64_t)a.nx * j + s_a[e] : a.uoff + (int64_t)a.nu * j + (s_a[e] - a.nx);
+        v[q] = v[q] + ((a.sx ? __ldg(a.sx + row) : 0.0) + a.dw);
+      }
+    } else if constexpr (KIND == KR_TF) {   // H's tf row, then its diagonal
+      if (s0 + i + 1 < R.len) v[q] = __ldg(src + s0 + i);
+      else v[q] = (a.sx ? __ldg(a.sx + a.n - 1) : 0.0) + a.dw;
+    } else if constexpr (KIND == KR_XN) {   // Euler: the X rows of node N hold only their diagonal
+      v[q] = (a.sx ? __ldg(a.sx + (int64_t)a.nx * a.N + s0 + i) : 0.0) + a.dw;
+    } else {                                // boundary rows: the unit entry, then the diagonal
+      v[q] = ((s0 + i) & 1) ? -a.dc : __ldg(src + ((s0 + i) >> 1));
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < KKT_PER; ++q) {
+    const uint32_t i = threadIdx.x + q * KKT_THREADS;
+    if (i < n) out[i] = v[q];
+  }
+}
+
+__global__ void __launch_bounds__(KKT_THREADS) k_kkt_values(const __grid_constant__ KktArgs a) {
   __shared__ int16_t s_src[KKT_TMAX], s_a[KKT_TMAX];
   __shared__ uint8_t s_diag[KKT_TMAX];
   // the region of this block: the last one whose first block is <= blockIdx.x
@@ -102,67 +151,23 @@ __global__ void __launch_bounds__(256) k_kkt_values(const __grid_constant__ KktA
     if (a.reg[mid].block0 <= blockIdx.x) lo = mid; else hi = mid - 1;
   }
   const KRegion R = a.reg[lo];
-  const uint32_t chunk = blockIdx.x - R.block0;
-  if (R.kind == KR_TF || R.kind == KR_BND || R.kind == KR_XN) {  // short regions: slot by slot
-    const uint32_t i1 = min(R.len, (chunk + 1) * 256u * KKT_ROWS);
-    for (uint32_t i = chunk * 256u * KKT_ROWS + threadIdx.x; i < i1; i += blockDim.x) {
-      double v;
-      if (R.kind == KR_TF) {
-        if (i + 1 < R.len) v = __ldg(a.hv + R.src + i);
-        else v = (a.sx ? __ldg(a.sx + a.n - 1) : 0.0) + a.dw;
-      } else if (R.kind == KR_XN) {  // Euler: the X rows of node N hold only their diagonal
-        v = (a.sx ? __ldg(a.sx + (int64_t)a.nx * a.N + i) : 0.0) + a.dw;
-      } else {
-        v = (i & 1) ? -a.dc : __ldg(a.jv + (i >> 1));
-      }
-      a.out[R.out + i] = v;
-    }
-    return;
-  }
-  const uint32_t P = R.period;
-  if (R.kind != KR_DEF) {  // the node template of the X or U rows
+  const uint32_t s0 = (blockIdx.x - R.block0) * KKT_SLOTS;
+  if (R.kind == KR_X || R.kind == KR_U) {  // the node template of the X or U rows
     const int toff = (R.kind == KR_U) ? KKT_TMAX : 0;
-    for (uint32_t p = threadIdx.x; p < P; p += blockDim.x) {
+    for (uint32_t p = threadIdx.x; p < R.period; p += KKT_THREADS) {
       s_src[p] = a.ksrc[toff + p];
       s_a[p] = a.ka[toff + p];
       s_diag[p] = a.ka[toff + p] == a.kb[toff + p];
     }
     __syncthreads();
   }
-  const float invP = 1.0f / (float)P;
-  const uint32_t nper = R.len / P;   // nodes or defect rows of the region
-  const uint32_t c0 = chunk * KKT_ROWS;
-  const uint32_t nloc = min((uint32_t)KKT_ROWS, nper - c0) * P;
-  // (the output never aliases the inputs: loads of later slots may be issued before stores)
-  const double* __restrict__ src0 = ((R.kind == KR_DEF) ? a.jv : a.hv) + R.src + (int64_t)c0 * R.stride;
-  double* __restrict__ out0 = a.out + R.out + (int64_t)c0 * P;
-  // KKT_BATCH slots per thread per pass: their loads are issued before any store
-  for (uint32_t i0 = threadIdx.x; i0 < nloc; i0 += KKT_BATCH * 256u) {
-    double v[KKT_BATCH];
-#pragma unroll
-    for (int q = 0; q < KKT_BATCH; ++q) {
-      const uint32_t i = i0 + q * 256u;
-      v[q] = 0.0;
-      if (i >= nloc) continue;
-      const uint32_t jl = kkt_div(i, invP);
-      const uint32_t e = i - jl * P;
-      if (R.kind == KR_DEF) {
-        v[q] = (e + 1 == P) ? -a.dc : __ldg(src0 + (i - jl));   // i - jl: the diagonals before this slot
-      } else {
-        const int sp = s_src[e];
-        v[q] = (sp >= 0) ? __ldg(src0 + (int64_t)R.stride * jl + sp) : 0.0;
-        if (s_diag[e]) {
-          const int64_t j = (int64_t)c0 + jl;
-          const int64_t row = (R.kind == KR_X) ? (int64_t)a.nx * j + s_a[e] : a.uoff + (int64_t)a.nu * j + (s_a[e] - a.nx);
-          v[q] = v[q] + ((a.sx ? __ldg(a.sx + row) : 0.0) + a.dw);
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < KKT_BATCH; ++q) {
-      const uint32_t i = i0 + q * 256u;
-      if (i < nloc) out0[i] = v[q];
-    }
+  switch (R.kind) {  // (CTA-uniform)
+    case KR_X: kkt_block<KR_X>(a, R, s0, s_src, s_a, s_diag); break;
+    case KR_U: kkt_block<KR_U>(a, R, s0, s_src, s_a, s_diag); break;
+    case KR_DEF: kkt_block<KR_DEF>(a, R, s0, s_src, s_a, s_diag); break;
+    case KR_TF: kkt_block<KR_TF>(a, R, s0, s_src, s_a, s_diag); break;
+    case KR_XN: kkt_block<KR_XN>(a, R, s0, s_src, s_a, s_diag); break;
+    default: kkt_block<KR_BND>(a, R, s0, s_src, s_a, s_diag); break;
   }
 }
 
@@ -276,7 +281,7 @@ static ocp_status kkt_fill(const ocp* h, KktArgs& a) {
   add(KR_XN, a.kb_xn, P.kb_u - a.kb_xn, 1, 0, 1);
   add(KR_U, P.kb_u, P.kb_t - P.kb_u, (uint32_t)a.ku, P.hbase_u, (uint32_t)P.hu);
   add(KR_TF, P.kb_t, P.kb_c - P.kb_t, 1, P.hbase_t, 1);
-  add(KR_BND, P.kb_c, 2 * P.nb, 2, 0, 1);
+  add(KR_BND, P.kb_c, 2 * P.nb, 1, 0, 1);
   for (int k = 0; k < h->nx; ++k)
     add(KR_DEF, P.kcbase[k], P.kcbase[k + 1] - P.kcbase[k], (uint32_t)(P.row_count(k) + 1), P.jbase[k],
         (uint32_t)P.row_count(k));
@@ -286,17 +291,13 @@ static ocp_status kkt_fill(const ocp* h, KktArgs& a) {
   for (int q = 0; q < P.nbin; ++q)  // boundary-inequality rows: one row each (entries, then the diagonal)
     add(KR_DEF, P.kbbase[q], P.kbbase[q + 1] - P.kbbase[q], (uint32_t)(P.bsupp[q].size() + 1), P.jbbase[q],
         (uint32_t)P.bsupp[q].size());
-  // blocks of the values kernel: KKT_ROWS periods of a row region per block, or
-  // blockDim * KKT_ROWS slots of a short region
+  // blocks of the values kernel: KKT_SLOTS slots of a region per block
   uint32_t b = 0;
   for (int r = 0; r < a.nreg; ++r) {
     KRegion& R = a.reg[r];
     if (R.period > 1024) return OCP_EDIM;  // kkt_div's exactness bound
     R.block0 = b;
-    const bool short_r = R.kind == KR_TF || R.kind == KR_BND || R.kind == KR_XN;
-    const int64_t nb = short_r ? ((int64_t)R.len + 256 * KKT_ROWS - 1) / (256 * KKT_ROWS)
-                                                              : ((int64_t)(R.len / R.period) + KKT_ROWS - 1) / KKT_ROWS;
-    b += (uint32_t)nb;
+    b += (R.len + KKT_SLOTS - 1) / KKT_SLOTS;
   }
   a.nblocks = b;
   return OCP_OK;
@@ -345,7 +346,7 @@ ocp_status ocp_kkt_values(ocp_t* h, const double* hvals, const double* jvals, co
   KktArgs a;
   if (kkt_fill(h, a) != OCP_OK) return set_err(h, OCP_EDIM, "KKT matrix too large for the int32 interface");
   a.hv = hvals; a.jv = jvals; a.sx = sigma_x; a.out = kvals; a.dw = delta_w; a.dc = delta_c;
-  k_kkt_values<<<a.nblocks, 256, 0, (cudaStream_t)stream>>>(a);
+  k_kkt_values<<<a.nblocks, KKT_THREADS, 0, (cudaStream_t)stream>>>(a);
   return cuda_err(h, cudaGetLastError(), "KKT values launch");
 }
 
