@@ -377,15 +377,11 @@ static ocp_status model_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream
   return set_err(h, OCP_EMODEL, "unknown model");
 }
 
-// The model's kernel, then (same stream) the path rows, then the boundary inequalities, with
-// their updates.
+// The model's kernel, then (same stream) the path and boundary terms.
 ocp_status ocpg::dispatch_eval(ocp* h, unsigned out, const EvalCall& c, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   ocp_status st = model_eval(h, out, c, s);
-  if (st == OCP_OK && h->pat.npath > 0) st = path_eval(h, out, c, s);
-  if (st == OCP_OK && h->pat.nbin > 0) st = bin_eval(h, out, c, s);
-  if (st == OCP_OK && h->has_bol) st = bol_eval(h, c, s);
-  return st;
+  return st == OCP_OK ? extra_eval(h, c, s) : st;
 }
 
 static ocp_status model_prod(ocp* h, const ProdCall& c, cudaStream_t s) {
@@ -403,10 +399,7 @@ static ocp_status model_prod(ocp* h, const ProdCall& c, cudaStream_t s) {
 static ocp_status dispatch_prod(ocp* h, const ProdCall& c, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   ocp_status st = model_prod(h, c, s);
-  if (st == OCP_OK && h->pat.npath > 0) st = path_prod(h, c, s);
-  if (st == OCP_OK && h->pat.nbin > 0) st = bin_prod(h, c, s);
-  if (st == OCP_OK && h->has_bol) st = bol_prod(h, c, s);
-  return st;
+  return st == OCP_OK ? extra_prod(h, c, s) : st;
 }
 
 static ocp_status need(ocp* h, const void* p, const char* name) {
@@ -556,8 +549,8 @@ ocp_status ocp_eval_step(ocp_t* h, const double* x, const double* y, double sigm
   NEED(Jv); NEED(Jtv); NEED(Hv);
   if (h->model == OCP_MODEL_HEAT1D) {
     // the heat model runs two kernels in sequence: the evaluation, and Jv, J^T w and H v in one
-    // launch; then each product's path, boundary-inequality and boundary-cost terms as in the
-    // separate calls (each array's own operations in the same order: the same bits)
+    // launch; then the products' path and boundary terms in one launch (each array's own
+    // operations in the order of the separate calls: the same bits)
     ocp_status st = ocp_eval_all(h, x, y, sigma, f, cv, g, jvals, hvals, stream);
     ProdCall a, b, c;
     a.kind = P_JPROD; a.x = x; a.v = vn; a.out = Jv;
@@ -565,12 +558,7 @@ ocp_status ocp_eval_step(ocp_t* h, const double* x, const double* y, double sigm
     c.kind = P_HPROD; c.x = x; c.y = y; c.sigma = sigma; c.v = vn; c.out = Hv;
     cudaStream_t s = (cudaStream_t)stream;
     if (st == OCP_OK) st = heat_prod2(h, a, b, &c, s);
-    for (const ProdCall* pc : {&a, &b, &c}) {
-      if (st == OCP_OK && h->pat.npath > 0) st = path_prod(h, *pc, s);
-      if (st == OCP_OK && h->pat.nbin > 0) st = bin_prod(h, *pc, s);
-      if (st == OCP_OK && h->has_bol) st = bol_prod(h, *pc, s);
-    }
-    return st;
+    return st == OCP_OK ? extra_prod3(h, a, b, c, s) : st;
   }
   EvalCall c = full_call(h);
   c.x = x; c.y = y; c.sigma = sigma; c.f = f; c.c = cv; c.g = g; c.jv = jvals; c.hv = hvals;

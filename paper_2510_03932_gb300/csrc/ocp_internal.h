@@ -124,10 +124,12 @@ struct ocp {
   // pv, coefficients pa, pb, pl; pr[p]; and the supports for the structure kernels
   int32_t* d_poff = nullptr;
   int32_t* d_pv = nullptr;
-  double* d_pcoef = nullptr;     // pa, pb, pl of every term (3 per term), then pr (npath)
+  double* d_pcoef = nullptr;     // a, b, l, 2a of every term (4 per term), then r (npath)
   int64_t* d_pbase = nullptr;    // jpbase (npath + 1) then kpbase (npath + 1)
   // boundary inequalities on the device: row q's terms boff[q]..boff[q+1]-1 with variable bv
-  // (local index of z = (X_0, X_N)) and coefficients a, b, l; then r (nbin)
+  // (local index of z = (X_0, X_N)) and coefficients a, b, l, 2a; then r (nbin) and, if set, the
+  // boundary cost's a, b, l (2 nx each).  After boff, by variable: offsets (2 nx + 1) and (row, term)
+  // pairs (with boundary inequalities only)
   int32_t* d_boff = nullptr;
   int32_t* d_bv = nullptr;
   double* d_bcoef = nullptr;
@@ -235,19 +237,14 @@ void model_hess_max_template(int model, int nx, std::vector<std::pair<int, int>>
 ocp_status obj_launch(ocp* h, bool hvp, const double* x, const double* s, const double* v, double* out,
                       double* dot, cudaStream_t st);
 
-// Path inequalities: rows, Jacobian entries and the updates of H, J^T w and H v that belong
-// to them, after the model's own kernel on the same stream (see path_kernels.cu).
-ocp_status path_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s);
-ocp_status path_prod(ocp* h, const ProdCall& c, cudaStream_t s);
+// Path inequalities, boundary inequalities and the boundary cost: their rows, Jacobian entries and
+// the updates of f, the gradient, H, J^T w and H v that belong to them, in one launch after the
+// model's own kernel on the same stream (see extra_kernels.cu).
+ocp_status extra_eval(ocp* h, const EvalCall& c, cudaStream_t s);
+ocp_status extra_prod(ocp* h, const ProdCall& c, cudaStream_t s);
+ocp_status extra_prod3(ocp* h, const ProdCall& jp, const ProdCall& jt, const ProdCall& hp, cudaStream_t s);
 ocp_status path_upload(ocp* h);
-// Boundary inequalities: their rows, Jacobian entries and the updates of H (nodes 0 and N),
-// J^T w and H v, after the path rows' kernel on the same stream (see bineq_kernels.cu).
-ocp_status bin_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s);
-ocp_status bin_prod(ocp* h, const ProdCall& c, cudaStream_t s);
 ocp_status bin_upload(ocp* h);
-// The boundary cost: its value, gradient and Hessian terms after the other kernels.
-ocp_status bol_eval(ocp* h, const EvalCall& c, cudaStream_t s);
-ocp_status bol_prod(ocp* h, const ProdCall& c, cudaStream_t s);
 // Releases the scatter map (called on every pattern rebuild and by ocp_destroy).
 void scatter_map_free(ocp* h);
 // Releases what ocp_eval_step_host allocated (called by ocp_destroy).
