@@ -109,8 +109,8 @@ KERNEL_SOURCES = {
     "heat64": _COMMON + ["heat_kernels.cu"],
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
-FP64_OPS_SRC = {"vdp": "76d84f0080b4", "vdp:euler": "76d84f0080b4", "cartpole": "810d82f3b0b7",
-                "quadrotor": "d9efc5bf84c0", "goddard": "5f8786230bfe", "heat64": "6e2d20e68d84"}
+FP64_OPS_SRC = {"vdp": "a6750866746d", "vdp:euler": "a6750866746d", "cartpole": "ad78faee0ec2",
+                "quadrotor": "6133431e199d", "goddard": "43beedec8173", "heat64": "13efe9b33e11"}
 
 
 def kernel_source_tag(key):
@@ -159,7 +159,7 @@ def named_workload(name):
 # DRAM bytes (read + write) of one launch at a workload, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; writes still dirty in L2 when the kernel ends
 # are not counted), with the source tag of the kernel it was captured on (see traffic()).
-TRAFFIC = {("vdp_mu_n1e6", "step"): (227.69e6, "76d84f0080b4")}
+TRAFFIC = {("vdp_mu_n1e6", "step"): (227.69e6, "a6750866746d")}
 # Each SM's FP64 pipe completes 2 FP64 instructions (one lane each) per clock: the recipe's
 # nominal 1.25 TFLOP/s FP64 of GB300 is 6.25e11 FMA/s = 1.99 per clock per SM at 152 SMs and
 # 2070 MHz.  bench.py measures the rate live (measure_fp64_rate) and reports it beside the peak.

@@ -48,6 +48,7 @@ struct GodArgs {
   const double* p_dev;             // G_PAR: (Cd, beta, Tmax, b) read from the device
   double* dpar;                    // G_DP: (dc/dp)^T w, 4 doubles
   int64_t N, nb, uoff, tau, ntiles;  // tau: index of tf in x (n - 1)
+  int64_t tile0;                     // first tile of the launch
   int64_t jbase[3];                  // first slot of the defect rows of each component
   int64_t hbase_u, hbase_t;          // Hessian slots: U block, tf row
   int hu, hpos_um;                   // U block entries per node; position of (u, m) in it
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
   constexpr bool WF = OUT & O_F, WC = OUT & O_C, WG = OUT & O_G, WJ = OUT & O_J, WH = OUT & O_H;
   constexpr bool WJV = OUT & O_JV, WJTV = OUT & O_JTV, WHV = OUT & O_HV;
   constexpr bool NEEDD = WJ || WH || WJV || WJTV || WHV;   // first derivatives of f
+  constexpr bool NEEDF = WC || NEEDD;                      // the dynamics at all
   constexpr bool RED = FREE && (WJTV || WHV);              // tf components of the products
   constexpr bool DP = WJTV && (OUT & G_DP);                // (dc/dp)^T w
   constexpr bool PAR = OUT & G_PAR;
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
   double vt = 0.0;  // tf component of the direction
   if (FREE && (WJV || WHV)) vt = __ldg(a.vn + a.tau);
 
-  for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
+  for (int64_t tile = a.tile0 + blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
     const int64_t r0 = tile * R;
     const int64_t own_end = min(r0 + R, N + 1);
     const int64_t row_end = min(own_end, N);
@@ -149,6 +151,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
     if (act) {
       const double r = __ldg(a.x + 3 * j), v = __ldg(a.x + 3 * j + 1), m = __ldg(a.x + 3 * j + 2);
       const double u = __ldg(a.x + a.uoff + j);
+      if constexpr (NEEDF) {
       const double E = exp_tab(fma(-beta, r, beta), a.one, a.mz);  // exp(-beta (r - 1))
       const double im = recip(a.one, m), ir = recip(a.one, r);
       const double ir2 = gmul(a, ir, ir);
@@ -306,6 +309,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
           }
         }
       }
+      }
       if (own) {
         const double zx[3] = {r, v, m};
         if (sG) {  // the terminal cost is the only objective term
@@ -448,7 +452,8 @@ template <unsigned OUT, bool FREE>
 static cudaError_t god_launch(const GodArgs& a, cudaStream_t s) {
   constexpr int F1 = FREE ? 1 : 0;
   const size_t smem = (OUT & O_J) ? sizeof(double) * (size_t)(16 + 3 * F1) * (GT - 1) : 0;
-  const int grid = (int)(a.ntiles < 0x7fffffff ? a.ntiles : 0x7fffffff);
+  const int64_t tiles = a.ntiles - a.tile0;
+  const int grid = (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff);
   k_god<OUT, FREE><<<grid, GT, smem, s>>>(a);  // (G_DP, G_PAR bits in OUT)
   return cudaGetLastError();
 }
@@ -469,9 +474,17 @@ ocp_status goddard_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s)
   cudaError_t e;
   if (a.p_dev) {  // device parameters: the constraints alone
     if (out != O_C) return set_err(h, OCP_EMODEL, "device parameters: the constraints only");
-    return cuda_err(h, god_launch_tf<O_ALL | G_PAR>(h, a, s), "Goddard kernel launch");
+    return cuda_err(h, god_launch_tf<O_C | G_PAR>(h, a, s), "Goddard kernel launch");
   }
   switch (out) {
+    case O_F:   // the terminal cost alone: the last tile
+      a.tile0 = a.ntiles - 1;
+      e = god_launch_tf<O_F>(h, a, s);
+      break;
+    case O_C: e = god_launch_tf<O_C>(h, a, s); break;
+    case O_G: e = god_launch_tf<O_G>(h, a, s); break;
+    case O_J: e = god_launch_tf<O_J>(h, a, s); break;
+    case O_H: e = god_launch_tf<O_H>(h, a, s); break;
     case O_STEP: e = god_launch_tf<O_STEP>(h, a, s); break;
     case O_J | O_H: e = god_launch_tf<O_J | O_H>(h, a, s); break;
     default: e = god_launch_tf<O_ALL>(h, a, s); break;  // subsets: NULL outputs are skipped

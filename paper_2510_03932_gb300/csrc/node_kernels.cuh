@@ -444,7 +444,8 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
         load_ybar<M>(a, K, a.y, j, yb);
         node_cq<M>(a, endp, cqd);
       }
-      M::template eval<WC, NEEDJ, NEEDH>(K, z, yb, cqd, pa[q], pb[q], mjx, mju, hd);
+      // (skipped, not left to dead-code elimination: the models' warp votes would keep parts of it)
+      if constexpr (WC || NEEDJ || NEEDH) M::template eval<WC, NEEDJ, NEEDH>(K, z, yb, cqd, pa[q], pb[q], mjx, mju, hd);
       if (WJV || WHV) load_vz<M>(a, a.v, j, vz);
       if (WJV) {
         double mdp[NX];
@@ -952,7 +953,7 @@ __global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs
         for (int k = 0; k < NX; ++k) yb[k] = (doH && M::HK(k)) ? __ldg(a.y + a.nb + (int64_t)k * N + j) : 0.0;
         node_cq<M>(a, false, cqd);
       }
-      M::template eval<WC, NEEDJ, NEEDH>(K, z, yb, cqd, pa, pb, mjx, mju, hd);
+      if constexpr (WC || NEEDJ || NEEDH) M::template eval<WC, NEEDJ, NEEDH>(K, z, yb, cqd, pa, pb, mjx, mju, hd);
       if (sC) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) a.c[a.nb + (int64_t)k * N + j] = fsub(K, __ldg(a.x + NX * (j + 1) + k), pa[k]);
@@ -1099,8 +1100,7 @@ ocp_status launch_euler_k(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
 
 template <class M, int TILE, unsigned OUT>
 ocp_status launch_euler_t(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
-  // (under forward Euler the constraints alone run through the O_ALL kernel, null outputs skipped)
-  if constexpr (M::HAS_DPARAM || (M::NP > 0 && OUT == O_ALL)) {
+  if constexpr (M::HAS_DPARAM || (M::NP > 0 && OUT == O_C)) {
     if (a.p0_dev) return launch_euler_k<M, TILE, OUT, true>(h, a, s);
   } else {
     if (a.p0_dev) return set_err(h, OCP_EMODEL, "device parameters are not provided for this output set");
@@ -1123,7 +1123,15 @@ ocp_status euler_eval_dispatch(ocp* h, unsigned out, const EvalCall& c, cudaStre
   fill_euler_args<M>(h, c.sigma, a);
   a.x = c.x; a.y = c.y; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
   a.v = c.vn; a.wv = c.vm; a.ojv = c.ojv; a.ojtv = c.ojtv; a.ohv = c.ohv;
+  // a solver's callbacks ask for one output each: a kernel each (the cart-pole's five at N = 250001
+  // took 40 to 49 us apiece through the kernel of all outputs, its evaluation and its
+  // staged rows included)
   switch (out) {
+    case O_F: return launch_euler_t<M, TILE, O_F>(h, a, s);
+    case O_C: return launch_euler_t<M, TILE, O_C>(h, a, s);
+    case O_G: return launch_euler_t<M, TILE, O_G>(h, a, s);
+    case O_J: return launch_euler_t<M, TILE, O_J>(h, a, s);
+    case O_H: return launch_euler_t<M, TILE, O_H>(h, a, s);
     case O_STEP: return launch_euler_t<M, TILE, O_STEP>(h, a, s);
     case O_J | O_H: return launch_euler_t<M, TILE, O_J | O_H>(h, a, s);
     default: return launch_euler_t<M, TILE, O_ALL>(h, a, s);  // subsets: NULL outputs are skipped
