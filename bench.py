@@ -82,16 +82,16 @@ def _counts(w):
 # Goddard) and 1e6 (Van der Pol).  Each model's counts hold for the kernel sources whose tag
 # (kernel_source_tag) is in FP64_OPS_SRC; when the sources change the counts are stale and the
 # bench reports no FP64 fraction for that model until they are measured again.
-FP64_OPS_PER_NODE = {("vdp", "eval_all"): 26.6, ("vdp", "jh"): 10.0, ("vdp", "jprod"): 13.0,
-                     ("vdp", "jtprod"): 12.0, ("vdp", "hprod"): 11.0, ("vdp", "step"): 50.6,
-                     ("cartpole", "eval_all"): 109.7, ("cartpole", "jh"): 87.7, ("cartpole", "jprod"): 74.6,
-                     ("cartpole", "jtprod"): 71.0, ("cartpole", "hprod"): 89.0, ("cartpole", "step"): 156.9,
-                     ("quadrotor", "eval_all"): 235.5, ("quadrotor", "jh"): 163.3, ("quadrotor", "jprod"): 151.2,
-                     ("quadrotor", "jtprod"): 143.0, ("quadrotor", "hprod"): 186.0, ("quadrotor", "step"): 382.8,
-                     ("goddard", "eval_all"): 94.2, ("goddard", "jh"): 85.2, ("goddard", "jprod"): 62.3,
-                     ("goddard", "jtprod"): 62.1, ("goddard", "hprod"): 89.1, ("goddard", "step"): 149.3,
-                     ("vdp:euler", "eval_all"): 21.5, ("vdp:euler", "jh"): 8.0, ("vdp:euler", "jprod"): 11.0,
-                     ("vdp:euler", "jtprod"): 10.0, ("vdp:euler", "hprod"): 10.0, ("vdp:euler", "step"): 41.5,
+FP64_OPS_PER_NODE = {("vdp", "eval_all"): 18.6, ("vdp", "jh"): 10.0, ("vdp", "jprod"): 10.0,
+                     ("vdp", "jtprod"): 9.0, ("vdp", "hprod"): 6.0, ("vdp", "step"): 35.6,
+                     ("cartpole", "eval_all"): 66.5, ("cartpole", "jh"): 48.4, ("cartpole", "jprod"): 46.3,
+                     ("cartpole", "jtprod"): 45.0, ("cartpole", "hprod"): 50.0, ("cartpole", "step"): 101.6,
+                     ("quadrotor", "eval_all"): 232.4, ("quadrotor", "jh"): 160.2, ("quadrotor", "jprod"): 95.3,
+                     ("quadrotor", "jtprod"): 90.0, ("quadrotor", "hprod"): 104.0, ("quadrotor", "step"): 385.8,
+                     ("goddard", "eval_all"): 52.2, ("goddard", "jh"): 44.2, ("goddard", "jprod"): 41.2,
+                     ("goddard", "jtprod"): 42.2, ("goddard", "hprod"): 51.2, ("goddard", "step"): 97.3,
+                     ("vdp:euler", "eval_all"): 13.5, ("vdp:euler", "jh"): 8.0, ("vdp:euler", "jprod"): 8.0,
+                     ("vdp:euler", "jtprod"): 7.0, ("vdp:euler", "hprod"): 5.0, ("vdp:euler", "step"): 26.5,
                      # heat, 64 cells: the step is its evaluation and one launch of Jv, J^T w and H v
                      ("heat64", "eval_all"): 1122.8, ("heat64", "jh"): 390.4, ("heat64", "jprod"): 523.4,
                      ("heat64", "jtprod"): 463.0, ("heat64", "hprod"): 257.0, ("heat64", "step"): 2366.2}
@@ -99,7 +99,7 @@ FP64_OPS_PER_NODE = {("vdp", "eval_all"): 26.6, ("vdp", "jh"): 10.0, ("vdp", "jp
 # The kernel sources of each model key (paths under the package's csrc/): the tile body and
 # the helpers it includes, the model's device functor, the translation unit that instantiates
 # its kernels.
-_COMMON = ["node_kernels.cuh", "model_base.cuh", "kernel_config.h"]
+_COMMON = ["node_kernels.cuh", "model_base.cuh", "soft_mul.cuh", "kernel_config.h"]
 KERNEL_SOURCES = {
     "vdp": _COMMON + ["model_vdp.cuh", "node_vdp.cu"],
     "vdp:euler": _COMMON + ["model_vdp.cuh", "node_vdp.cu"],
@@ -109,8 +109,8 @@ KERNEL_SOURCES = {
     "heat64": _COMMON + ["heat_kernels.cu"],
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
-FP64_OPS_SRC = {"vdp": "a6750866746d", "vdp:euler": "a6750866746d", "cartpole": "ad78faee0ec2",
-                "quadrotor": "6133431e199d", "goddard": "43beedec8173", "heat64": "13efe9b33e11"}
+FP64_OPS_SRC = {"vdp": "3dcd0c729ec8", "vdp:euler": "3dcd0c729ec8", "cartpole": "b47378fa5ab4",
+                "quadrotor": "ea70b7578567", "goddard": "861bebe22adc", "heat64": "b90b5bc0c26d"}
 
 
 def kernel_source_tag(key):
@@ -159,7 +159,7 @@ def named_workload(name):
 # DRAM bytes (read + write) of one launch at a workload, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; writes still dirty in L2 when the kernel ends
 # are not counted), with the source tag of the kernel it was captured on (see traffic()).
-TRAFFIC = {("vdp_mu_n1e6", "step"): (227.69e6, "a6750866746d")}
+TRAFFIC = {("vdp_mu_n1e6", "step"): (226.65e6, "3dcd0c729ec8")}
 # Each SM's FP64 pipe completes 2 FP64 instructions (one lane each) per clock: the recipe's
 # nominal 1.25 TFLOP/s FP64 of GB300 is 6.25e11 FMA/s = 1.99 per clock per SM at 152 SMs and
 # 2070 MHz.  bench.py measures the rate live (measure_fp64_rate) and reports it beside the peak.

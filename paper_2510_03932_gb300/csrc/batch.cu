@@ -58,8 +58,13 @@ struct BatchArgs {
   int count;
 };
 
-template <class M, int TILE, int NPT>
-__global__ void __launch_bounds__(TILE) k_batch_eval(const __grid_constant__ BatchArgs<M> b) {
+// Resident CTAs that the registers are capped for: as many threads as the plain evaluation's (the
+// cart-pole batch of 6.5e6 nodes 1042 us at 72 registers, 1433 at the allocator's 126).
+template <class M, int TILE, bool IP>
+constexpr int batch_ctas() { return soft_kernel<M, O_ALL, IP>() ? M::template CTAS<O_ALL> * M::EVAL_TILE / TILE : 0; }
+
+template <class M, int TILE, int NPT, bool IP>
+__global__ void __launch_bounds__(TILE, batch_ctas<M, TILE, IP>()) k_batch_eval(const __grid_constant__ BatchArgs<M> b) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double sEdge[2 * (TILE / 32 + 1) * M::NX];
   __shared__ NodeArgs<M> sa;
@@ -102,9 +107,9 @@ __global__ void __launch_bounds__(TILE) k_batch_eval(const __grid_constant__ Bat
       }
     }
     __syncthreads();
-    const ModelConst K = sa.K;
+    const ModelConst& K = sa.K;
     const int64_t t0 = __ldg(b.tileoff + i), t1 = __ldg(b.tileoff + i + 1);
-    node_eval_tile<M, TILE, NPT, O_ALL>(sa, K, gt - t0, sm, sEdge, b.partials + gt);
+    node_eval_tile<M, TILE, NPT, O_ALL, IP>(sa, K, gt - t0, sm, sEdge, b.partials + gt);
     if (b.f) {
       // the CTA that completes an instance's last tile sums its tile terms in tile order
       if (threadIdx.x == 0) {
@@ -148,22 +153,25 @@ static const BatchConfig kConfigs[] = {{64, 1}, {128, 1}, {256, 1}, {64, 2}, {12
 template <class M>
 constexpr int batch_max_nodes() { return jrow_total<M>() > 32 ? 128 : 512; }
 
+// (integer products with one node per thread, in batches that soft_launch names large)
 template <class M, int TILE, int NPT>
-static const void* batch_kernel() {
-  if constexpr (TILE * NPT <= batch_max_nodes<M>()) return (const void*)k_batch_eval<M, TILE, NPT>;
-  else return nullptr;
+static const void* batch_kernel(bool many) {
+  if constexpr (TILE * NPT > batch_max_nodes<M>()) return nullptr;
+  else if constexpr (NPT == 1 && M::template SOFT<O_ALL> != 0)
+    return many ? (const void*)k_batch_eval<M, TILE, NPT, true> : (const void*)k_batch_eval<M, TILE, NPT, false>;
+  else return (const void*)k_batch_eval<M, TILE, NPT, false>;
 }
 
 template <class M>
-static const void* kernel_for(int threads, int npt) {
+static const void* kernel_for(int threads, int npt, bool many) {
   if (npt == 1) {
-    if (threads == 64) return batch_kernel<M, 64, 1>();
-    if (threads == 128) return batch_kernel<M, 128, 1>();
-    if (threads == 256) return batch_kernel<M, 256, 1>();
+    if (threads == 64) return batch_kernel<M, 64, 1>(many);
+    if (threads == 128) return batch_kernel<M, 128, 1>(many);
+    if (threads == 256) return batch_kernel<M, 256, 1>(many);
   } else {
-    if (threads == 64) return batch_kernel<M, 64, 2>();
-    if (threads == 128) return batch_kernel<M, 128, 2>();
-    if (threads == 256) return batch_kernel<M, 256, 2>();
+    if (threads == 64) return batch_kernel<M, 64, 2>(many);
+    if (threads == 128) return batch_kernel<M, 128, 2>(many);
+    if (threads == 256) return batch_kernel<M, 256, 2>(many);
   }
   return nullptr;
 }
@@ -180,6 +188,7 @@ struct ocp_batch_impl {
   std::vector<ocp*> items;
   std::vector<int64_t> xoff, coff, joff, hoff, tileoff;
   int threads = 128, npt = 1, ctas_per_sm = 0;
+  bool many = false;   // soft_launch of the whole batch
   int64_t ntiles = 0;
   void* d_inst = nullptr;
   int64_t *d_tileoff = nullptr, *d_xoff = nullptr, *d_coff = nullptr, *d_joff = nullptr, *d_hoff = nullptr;
@@ -254,6 +263,8 @@ static ocp_status batch_upload_inst(ocp_batch* b) {
   std::vector<NodeArgs<M>> inst(b->count);
   for (int i = 0; i < b->count; ++i) {
     fill_args<M>(b->items[i], 1.0, inst[i]);
+    inst[i].K.many = b->many;   // (the instances share one launch)
+    inst[i].K.soft = inst[i].K.many && soft_consts(inst[i].K, M::NC);
     inst[i].B = 0;
     inst[i].E = b->items[i]->N + 1;
     inst[i].p0_dev = nullptr;
@@ -264,8 +275,8 @@ static ocp_status batch_upload_inst(ocp_batch* b) {
   if (e != cudaSuccess) return berr(b, OCP_ECUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));
   // allow the largest shared-memory request of every configuration once
   for (const auto& cf : kConfigs) {
-    if (!kernel_for<M>(cf.threads, cf.npt)) continue;   // not provided for this model
-    e = cudaFuncSetAttribute(kernel_for<M>(cf.threads, cf.npt), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (!kernel_for<M>(cf.threads, cf.npt, b->many)) continue;   // not provided for this model
+    e = cudaFuncSetAttribute(kernel_for<M>(cf.threads, cf.npt, b->many), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem_bytes<M>(cf.threads, cf.npt));
     if (e != cudaSuccess) return berr(b, OCP_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));
   }
@@ -290,7 +301,7 @@ static ocp_status batch_tiles(ocp_batch* b) {
 template <class M>
 static int max_ctas_per_sm(const ocp_batch* b) {
   int per = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_for<M>(b->threads, b->npt), b->threads,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_for<M>(b->threads, b->npt, b->many), b->threads,
                                                     smem_bytes<M>(b->threads, b->npt)) != cudaSuccess || per < 1)
     per = 1;
   return per;
@@ -313,22 +324,10 @@ static ocp_status batch_launch(ocp_batch* b, const double* x, const double* y, d
   const int per = b->ctas_per_sm > 0 ? std::min(b->ctas_per_sm, max_ctas_per_sm<M>(b)) : max_ctas_per_sm<M>(b);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(b->ntiles, (int64_t)per * b->num_sms));
   const size_t sm = smem_bytes<M>(b->threads, b->npt);
-  const int T = b->threads;
-  auto go = [&](auto tt, auto pp) {
-    constexpr int TT = decltype(tt)::value, PP = decltype(pp)::value;
-    if constexpr (TT * PP <= batch_max_nodes<M>()) k_batch_eval<M, TT, PP><<<grid, TT, sm, s>>>(a);
-  };
-  using I64 = std::integral_constant<int, 64>;
-  using I128 = std::integral_constant<int, 128>;
-  using I256 = std::integral_constant<int, 256>;
-  using P1 = std::integral_constant<int, 1>;
-  using P2 = std::integral_constant<int, 2>;
-  if (!kernel_for<M>(T, b->npt)) return berr(b, OCP_EINVAL, "configuration not provided for this model");
-  if (b->npt == 1) {
-    if (T == 64) go(I64{}, P1{}); else if (T == 128) go(I128{}, P1{}); else go(I256{}, P1{});
-  } else {
-    if (T == 64) go(I64{}, P2{}); else if (T == 128) go(I128{}, P2{}); else go(I256{}, P2{});
-  }
+  const void* kern = kernel_for<M>(b->threads, b->npt, b->many);
+  if (!kern) return berr(b, OCP_EINVAL, "configuration not provided for this model");
+  void* args[] = {&a};
+  cudaLaunchKernel(kern, dim3(grid), dim3(b->threads), args, sm, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return berr(b, OCP_ECUDA, std::string("batch launch: ") + cudaGetErrorString(e));
   return OCP_OK;
@@ -353,7 +352,7 @@ static ocp_status dispatch_batch(ocp_batch* b, const double* x, const double* y,
 }
 
 static bool config_provided(const ocp_batch* b, int threads, int npt) {
-  return with_model(b->model, [&](auto m) { return kernel_for<decltype(m)>(threads, npt) != nullptr; });
+  return with_model(b->model, [&](auto m) { return kernel_for<decltype(m)>(threads, npt, b->many) != nullptr; });
 }
 
 static void batch_free(ocp_batch* b) {
@@ -389,6 +388,9 @@ ocp_status ocp_batch_create(ocp_t* const* items, int count, ocp_batch_t** out) {
   ocp_batch* b = new (std::nothrow) ocp_batch();
   if (!b) return set_err(nullptr, OCP_ENOMEM, "host allocation failed");
   b->model = model; b->count = count; b->device = items[0]->device; b->num_sms = items[0]->num_sms;
+  int64_t nodes = 0;
+  for (int i = 0; i < count; ++i) nodes += items[i]->N + 1;
+  b->many = soft_launch(nodes, b->num_sms);
   b->items.assign(items, items + count);
   b->xoff.assign(count + 1, 0); b->coff.assign(count + 1, 0); b->joff.assign(count + 1, 0); b->hoff.assign(count + 1, 0);
   int64_t cap = 0;

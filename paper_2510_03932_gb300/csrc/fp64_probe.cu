@@ -81,9 +81,10 @@ __global__ void k_probe_sincos_tab(const double* x, double* s, double* c, double
 }
 
 // The table-driven exponential (exp_tab) and the library's on the same arguments.
-__global__ void k_probe_exp(const double* x, double* e, double* el, int64_t n) {
+__global__ void k_probe_exp(const double* x, double* e, double* el, int64_t n,
+                            const __grid_constant__ ocpg::ModelConst K) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    e[i] = ocpg::exp_tab(x[i], 1.0, -0.0);
+    e[i] = ocpg::exp_tab(K, x[i]);
     el[i] = exp(x[i]);
   }
 }
@@ -98,7 +99,11 @@ extern "C" ocp_status ocp_probe_exp_table(const double* x, double* e, double* e_
   if (n < 0) return ocpg::set_err(nullptr, OCP_EINVAL, "ocp_probe_exp_table: n < 0");
   if (n == 0) return OCP_OK;
   const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  k_probe_exp<<<grid, 256, 0, (cudaStream_t)stream>>>(x, e, e_lib, n);
+  ocpg::ModelConst K;
+  memset(&K, 0, sizeof(K));
+  K.one = 1.0;
+  K.mz = -0.0;
+  k_probe_exp<<<grid, 256, 0, (cudaStream_t)stream>>>(x, e, e_lib, n, K);
   return ocpg::cuda_err(nullptr, cudaGetLastError(), "ocp_probe_exp_table launch");
 }
 

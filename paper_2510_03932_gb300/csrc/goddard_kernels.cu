@@ -58,12 +58,25 @@ struct GodArgs {
   double mayer[3];
   int finpos[3];                     // row of X_{N,k} among the final rows, or -1
   double one, mz;                    // 1.0 and -0.0 at run time (sums and products as FMAs)
+  int many;                          // soft_launch
 };
 
-// a + b, a - b, a * b issued as FMAs (same rounding; see fadd in models.cuh)
-__device__ __forceinline__ double gadd(const GodArgs& a, double p, double q) { return fma(p, a.one, q); }
-__device__ __forceinline__ double gsub(const GodArgs& a, double p, double q) { return fma(-q, a.one, p); }
-__device__ __forceinline__ double gmul(const GodArgs& a, double p, double q) { return fma(p, q, a.mz); }
+// The inputs of node j's work that its products multiply (see soft_mul.cuh).
+template <bool Y, bool YALL, bool V, bool W>
+__device__ __forceinline__ bool soft_god(const GodArgs& a, int64_t j) {
+  const int64_t jl = max(j - 1, (int64_t)0), jr = min(j, a.N - 1);   // (as in soft_node)
+  bool ok = soft_input(a.x + a.uoff + j);
+  if (V) ok &= soft_input(a.vn + a.uoff + j);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    ok &= soft_input(a.x + 3 * j + k);
+    if (V) ok &= soft_input(a.vn + 3 * j + k);
+    const int64_t row = a.nb + (int64_t)k * a.N;
+    if (Y && (YALL || k == 1)) ok &= soft_input(a.y + row + jl) & soft_input(a.y + row + jr);
+    if (W) ok &= soft_input(a.vm + row + jl) & soft_input(a.vm + row + jr);
+  }
+  return ok;
+}
 
 // Variant bits of k_god beside the outputs: G_DP adds (dc/dp)^T w to J^T w, G_PAR reads the
 // parameters from the device.
@@ -95,8 +108,13 @@ __device__ __forceinline__ void finish_sums(const double* partials, int64_t ntil
   if (threadIdx.x == 0) *counter = 0u;
 }
 
-template <unsigned OUT, bool FREE>
-__global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
+// Resident CTAs per SM that the registers are capped for (0: the allocator's choice): the step at 80
+// (241.6 us at N = 1e6; 255.9 uncapped), the evaluation at 64 (136 us; 156).
+template <unsigned OUT, bool IP>
+constexpr int god_ctas() { return !IP ? 0 : OUT == O_STEP ? 3 : OUT == O_ALL ? 4 : 0; }
+
+template <unsigned OUT, bool FREE, bool IP>
+__global__ void __launch_bounds__(GT, god_ctas<OUT, IP>()) k_god(const __grid_constant__ GodArgs a) {
   constexpr bool WF = OUT & O_F, WC = OUT & O_C, WG = OUT & O_G, WJ = OUT & O_J, WH = OUT & O_H;
   constexpr bool WJV = OUT & O_JV, WJTV = OUT & O_JTV, WHV = OUT & O_HV;
   constexpr bool NEEDD = WJ || WH || WJV || WJTV || WHV;   // first derivatives of f
@@ -104,6 +122,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
   constexpr bool RED = FREE && (WJTV || WHV);              // tf components of the products
   constexpr bool DP = WJTV && (OUT & G_DP);                // (dc/dp)^T w
   constexpr bool PAR = OUT & G_PAR;
+  constexpr unsigned SOFT = IP ? MUL_ALL : 0u;             // products on the integer pipes (soft_mul.cuh)
   constexpr int F1 = FREE ? 1 : 0;
   constexpr int CR = 4 + F1, CV = 8 + F1, CM = 4 + F1;     // entries per defect row of r, v, m
   constexpr int R = GT - 1;
@@ -128,7 +147,11 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
   // the parameters: kernel arguments, or device memory with PAR (bT = b Tmax as on the host)
   const double Cd = PAR ? __ldg(a.p_dev) : a.Cd, beta = PAR ? __ldg(a.p_dev + 1) : a.beta;
   const double Tmax = PAR ? __ldg(a.p_dev + 2) : a.Tmax, bpar = PAR ? __ldg(a.p_dev + 3) : a.b;
-  const double bT = PAR ? gmul(a, bpar, Tmax) : a.bT;
+  const double bT = PAR ? fma(bpar, Tmax, a.mz) : a.bT;
+  ModelConst K0;
+  K0.one = a.one; K0.mz = a.mz; K0.hh = hh;
+  K0.c[0] = Cd; K0.c[1] = beta; K0.c[2] = Tmax; K0.c[3] = bpar; K0.c[4] = bT; K0.c[5] = a.kappa;
+  K0.soft = SOFT != 0 ? soft_consts(K0, 6) : 0;
   double vt = 0.0;  // tf component of the direction
   if (FREE && (WJV || WHV)) vt = __ldg(a.vn + a.tau);
 
@@ -148,33 +171,37 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
     double jA[3] = {0.0, 0.0, 0.0}, jB[3] = {0.0, 0.0, 0.0}, fk[3] = {0.0, 0.0, 0.0};
     double accJ = 0.0, accH = 0.0;
     double accP[4] = {0.0, 0.0, 0.0, 0.0};
-    if (act) {
+    bool ok = false;
+    if constexpr (SOFT != 0) {
+      if (K0.soft && act) ok = soft_god<(WH || WHV), FREE, (WJV || WHV), WJTV>(a, j);
+    }
+    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
       const double r = __ldg(a.x + 3 * j), v = __ldg(a.x + 3 * j + 1), m = __ldg(a.x + 3 * j + 2);
       const double u = __ldg(a.x + a.uoff + j);
       if constexpr (NEEDF) {
-      const double E = exp_tab(fma(-beta, r, beta), a.one, a.mz);  // exp(-beta (r - 1))
-      const double im = recip(a.one, m), ir = recip(a.one, r);
-      const double ir2 = gmul(a, ir, ir);
-      const double q1 = gmul(a, gmul(a, Cd, E), im);        // Cd E / m
-      const double D = gmul(a, gmul(a, q1, v), v);
-      const double aU = gmul(a, Tmax, im);                  // dv'/du = Tmax / m
-      const double fv = fma(u, aU, -gadd(a, D, ir2));
-      const double fm = gmul(a, -bT, u);
+      const double E = exp_tab(K, fma(-beta, r, beta));  // exp(-beta (r - 1))
+      const double im = recip(K, m), ir = recip(K, r);
+      const double ir2 = fmul(K, ir, ir);
+      const double q1 = fmul(K, fmul(K, Cd, E), im);        // Cd E / m
+      const double D = fmul(K, fmul(K, q1, v), v);
+      const double aU = fmul(K, Tmax, im);                  // dv'/du = Tmax / m
+      const double fv = fma(u, aU, -fadd(K, D, ir2));
+      const double fm = fmul(K, -bT, u);
       pa[0] = fma(hh, v, r);  pb[0] = fma(mhh, v, r);
       pa[1] = fma(hh, fv, v); pb[1] = fma(mhh, fv, v);
       pa[2] = fma(hh, fm, m); pb[2] = fma(mhh, fm, m);
       if (FREE && (WJ || WJV || WJTV)) {
-        fk[0] = gmul(a, mk, v);
-        fk[1] = gmul(a, mk, fv);
-        fk[2] = gmul(a, mk, fm);
+        fk[0] = fmul(K, mk, v);
+        fk[1] = fmul(K, mk, fv);
+        fk[2] = fmul(K, mk, fm);
       }
       if (NEEDD) {
-        const double ar = fma(beta, D, gmul(a, 2.0, gmul(a, ir2, ir)));   // beta D + 2/r^3
-        const double av = gmul(a, -2.0, gmul(a, q1, v));                     // -2 Cd v E / m
-        const double am = gmul(a, gsub(a, D, gmul(a, u, aU)), im);          // (D - u Tmax/m) / m
+        const double ar = fma(beta, D, fmul(K, 2.0, fmul(K, ir2, ir)));   // beta D + 2/r^3
+        const double av = fmul(K, -2.0, fmul(K, q1, v));                     // -2 Cd v E / m
+        const double am = fmul(K, fsub(K, D, fmul(K, u, aU)), im);          // (D - u Tmax/m) / m
         // Jacobian values without the identity: -hh df/dz
-        const double jr = gmul(a, mhh, ar), jvv = gmul(a, mhh, av), jm = gmul(a, mhh, am);
-        const double ju = gmul(a, mhh, aU), jmu = gmul(a, hh, bT);
+        const double jr = fmul<MUL_J>(K, mhh, ar), jvv = fmul<MUL_J>(K, mhh, av), jm = fmul<MUL_J>(K, mhh, am);
+        const double ju = fmul<MUL_J>(K, mhh, aU), jmu = fmul<MUL_J>(K, hh, bT);
         if (sJ) {  // left part of row t, right part of row t-1
           if (t < nrows) {
             double* rr = sm + t * CR;
@@ -199,13 +226,13 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
           vz[3] = __ldg(a.vn + a.uoff + j);
         }
         if (WJV) {  // node shares of rows (k, j-1) and (k, j): p_k +- v_{X_j,k}
-          double p0 = gmul(a, mhh, vz[1]);
-          double p1 = fma(jr, vz[0], fma(jvv, vz[1], fma(jm, vz[2], gmul(a, ju, vz[3]))));
-          double p2 = gmul(a, jmu, vz[3]);
+          double p0 = fmul<MUL_V>(K, mhh, vz[1]);
+          double p1 = fma(jr, vz[0], fma(jvv, vz[1], fma(jm, vz[2], fmul<MUL_V>(K, ju, vz[3]))));
+          double p2 = fmul<MUL_V>(K, jmu, vz[3]);
           if (FREE) { p0 = fma(fk[0], vt, p0); p1 = fma(fk[1], vt, p1); p2 = fma(fk[2], vt, p2); }
           const double p[3] = {p0, p1, p2};
 #pragma unroll
-          for (int k = 0; k < 3; ++k) { jA[k] = gadd(a, p[k], vz[k]); jB[k] = gsub(a, p[k], vz[k]); }
+          for (int k = 0; k < 3; ++k) { jA[k] = fadd(K, p[k], vz[k]); jB[k] = fsub(K, p[k], vz[k]); }
           if (own && j == 0) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) a.ojv[k] = vz[k];
@@ -223,33 +250,33 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
             const double* row = a.vm + a.nb + (int64_t)k * N;
             wl[k] = (j >= 1) ? __ldg(row + j - 1) : 0.0;
             wr[k] = (j < N) ? __ldg(row + j) : 0.0;
-            wb[k] = gadd(a, wl[k], wr[k]);
+            wb[k] = fadd(K, wl[k], wr[k]);
           }
           double o[4];
-          o[0] = fma(wb[1], jr, gsub(a, wl[0], wr[0]));
-          o[1] = fma(wb[1], jvv, fma(wb[0], mhh, gsub(a, wl[1], wr[1])));
-          o[2] = fma(wb[1], jm, gsub(a, wl[2], wr[2]));
-          o[3] = fma(wb[2], jmu, gmul(a, wb[1], ju));
+          o[0] = fma(wb[1], jr, fsub(K, wl[0], wr[0]));
+          o[1] = fma(wb[1], jvv, fma(wb[0], mhh, fsub(K, wl[1], wr[1])));
+          o[2] = fma(wb[1], jm, fsub(K, wl[2], wr[2]));
+          o[3] = fma(wb[2], jmu, fmul<MUL_V>(K, wb[1], ju));
           if (bnd) {
             if (j == 0) {
 #pragma unroll
-              for (int k = 0; k < 3; ++k) o[k] = gadd(a, o[k], __ldg(a.vm + k));
+              for (int k = 0; k < 3; ++k) o[k] = fadd(K, o[k], __ldg(a.vm + k));
             }
             if (j == N) {
 #pragma unroll
               for (int k = 0; k < 3; ++k)
-                if (a.finpos[k] >= 0) o[k] = gadd(a, o[k], __ldg(a.vm + 3 + a.finpos[k]));
+                if (a.finpos[k] >= 0) o[k] = fadd(K, o[k], __ldg(a.vm + 3 + a.finpos[k]));
             }
           }
           a.ojtv[3 * j] = o[0]; a.ojtv[3 * j + 1] = o[1]; a.ojtv[3 * j + 2] = o[2];
           a.ojtv[a.uoff + j] = o[3];
-          if (FREE) accJ = fma(wb[0], fk[0], fma(wb[1], fk[1], gmul(a, wb[2], fk[2])));
+          if (FREE) accJ = fma(wb[0], fk[0], fma(wb[1], fk[1], fmul<MUL_V>(K, wb[2], fk[2])));
           if (DP) {  // sum_k wbar_k (-hh df_k/dp_i)
-            const double vEm = gmul(a, gmul(a, gmul(a, E, im), v), v);        // v^2 E / m
-            accP[0] = gmul(a, wb[1], gmul(a, hh, vEm));
-            accP[1] = gmul(a, wb[1], gmul(a, mhh, gmul(a, D, gsub(a, r, a.one))));
-            accP[2] = fma(wb[1], gmul(a, mhh, gmul(a, u, im)), gmul(a, wb[2], gmul(a, hh, gmul(a, bpar, u))));
-            accP[3] = gmul(a, wb[2], gmul(a, hh, gmul(a, Tmax, u)));
+            const double vEm = fmul<MUL_V>(K, fmul<MUL_V>(K, fmul<MUL_V>(K, E, im), v), v);        // v^2 E / m
+            accP[0] = fmul<MUL_V>(K, wb[1], fmul<MUL_V>(K, hh, vEm));
+            accP[1] = fmul<MUL_V>(K, wb[1], fmul<MUL_V>(K, mhh, fmul<MUL_V>(K, D, fsub(K, r, a.one))));
+            accP[2] = fma(wb[1], fmul<MUL_V>(K, mhh, fmul<MUL_V>(K, u, im)), fmul<MUL_V>(K, wb[2], fmul<MUL_V>(K, hh, fmul<MUL_V>(K, bpar, u))));
+            accP[3] = fmul<MUL_V>(K, wb[2], fmul<MUL_V>(K, hh, fmul<MUL_V>(K, Tmax, u)));
           }
         }
         if (doH && own) {
@@ -261,25 +288,25 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
               const double* row = a.y + a.nb + (int64_t)k * N;
               const double yl = (j >= 1) ? __ldg(row + j - 1) : 0.0;
               const double yr = (j < N) ? __ldg(row + j) : 0.0;
-              yb[k] = gadd(a, yl, yr);
+              yb[k] = fadd(K, yl, yr);
             }
           }
-          const double y1 = gmul(a, mhh, yb[1]);
-          const double ir4 = gmul(a, ir2, ir2);
+          const double y1 = fmul<MUL_H>(K, mhh, yb[1]);
+          const double ir4 = fmul<MUL_H>(K, ir2, ir2);
           double hd[7];
-          hd[0] = gmul(a, y1, fma(-gmul(a, beta, beta), D, gmul(a, -6.0, ir4)));   // (r, r)
-          hd[1] = gmul(a, y1, gmul(a, -beta, av));                                 // (v, r)
-          hd[2] = gmul(a, y1, gmul(a, -2.0, q1));                                    // (v, v)
-          hd[3] = gmul(a, y1, gmul(a, gmul(a, -beta, D), im));                     // (m, r)
-          hd[4] = gmul(a, y1, gmul(a, -av, im));                                     // (m, v)
-          hd[5] = gmul(a, y1, gmul(a, gmul(a, 2.0, gsub(a, gmul(a, u, aU), D)), gmul(a, im, im)));  // (m, m)
-          hd[6] = gmul(a, y1, gmul(a, -aU, im));                                     // (u, m)
+          hd[0] = fmul<MUL_H>(K, y1, fma(-fmul<MUL_H>(K, beta, beta), D, fmul<MUL_H>(K, -6.0, ir4)));   // (r, r)
+          hd[1] = fmul<MUL_H>(K, y1, fmul<MUL_H>(K, -beta, av));                                 // (v, r)
+          hd[2] = fmul<MUL_H>(K, y1, fmul<MUL_H>(K, -2.0, q1));                                    // (v, v)
+          hd[3] = fmul<MUL_H>(K, y1, fmul<MUL_H>(K, fmul<MUL_H>(K, -beta, D), im));                     // (m, r)
+          hd[4] = fmul<MUL_H>(K, y1, fmul<MUL_H>(K, -av, im));                                     // (m, v)
+          hd[5] = fmul<MUL_H>(K, y1, fmul<MUL_H>(K, fmul<MUL_H>(K, 2.0, fsub(K, fmul<MUL_H>(K, u, aU), D)), fmul<MUL_H>(K, im, im)));  // (m, m)
+          hd[6] = fmul<MUL_H>(K, y1, fmul<MUL_H>(K, -aU, im));                                     // (u, m)
           double tr = 0.0, tv = 0.0, tm = 0.0, tu = 0.0;  // tf row: -kappa sum_k ybar_k df_k/dz
           if (FREE) {
-            tr = gmul(a, mk, gmul(a, yb[1], ar));
-            tv = gmul(a, mk, fma(yb[1], av, yb[0]));
-            tm = gmul(a, mk, gmul(a, yb[1], am));
-            tu = gmul(a, mk, fma(yb[1], aU, gmul(a, -bT, yb[2])));
+            tr = fmul<MUL_H>(K, mk, fmul<MUL_H>(K, yb[1], ar));
+            tv = fmul<MUL_H>(K, mk, fma(yb[1], av, yb[0]));
+            tm = fmul<MUL_H>(K, mk, fmul<MUL_H>(K, yb[1], am));
+            tu = fmul<MUL_H>(K, mk, fma(yb[1], aU, fmul<MUL_H>(K, -bT, yb[2])));
           }
           if (sH) {
 #pragma unroll
@@ -296,13 +323,13 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
           }
           if (WHV) {
             double o[4];
-            o[0] = fma(hd[0], vz[0], fma(hd[1], vz[1], gmul(a, hd[3], vz[2])));
-            o[1] = fma(hd[1], vz[0], fma(hd[2], vz[1], gmul(a, hd[4], vz[2])));
-            o[2] = fma(hd[3], vz[0], fma(hd[4], vz[1], fma(hd[5], vz[2], gmul(a, hd[6], vz[3]))));
-            o[3] = gmul(a, hd[6], vz[2]);
+            o[0] = fma(hd[0], vz[0], fma(hd[1], vz[1], fmul<MUL_V>(K, hd[3], vz[2])));
+            o[1] = fma(hd[1], vz[0], fma(hd[2], vz[1], fmul<MUL_V>(K, hd[4], vz[2])));
+            o[2] = fma(hd[3], vz[0], fma(hd[4], vz[1], fma(hd[5], vz[2], fmul<MUL_V>(K, hd[6], vz[3]))));
+            o[3] = fmul<MUL_V>(K, hd[6], vz[2]);
             if (FREE) {
               o[0] = fma(tr, vt, o[0]); o[1] = fma(tv, vt, o[1]); o[2] = fma(tm, vt, o[2]); o[3] = fma(tu, vt, o[3]);
-              accH = fma(tr, vz[0], fma(tv, vz[1], fma(tm, vz[2], gmul(a, tu, vz[3]))));
+              accH = fma(tr, vz[0], fma(tv, vz[1], fma(tm, vz[2], fmul<MUL_V>(K, tu, vz[3]))));
             }
             a.ohv[3 * j] = o[0]; a.ohv[3 * j + 1] = o[1]; a.ohv[3 * j + 2] = o[2];
             a.ohv[a.uoff + j] = o[3];
@@ -318,7 +345,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
           a.g[a.uoff + j] = 0.0;
           if (FREE && j == 0) a.g[a.tau] = 0.0;
         }
-        if (sF && bnd && j == N) *a.f = fma(a.mayer[0], r, fma(a.mayer[1], v, gmul(a, a.mayer[2], m)));
+        if (sF && bnd && j == N) *a.f = fma(a.mayer[0], r, fma(a.mayer[1], v, fmul(K, a.mayer[2], m)));
         if (j == 0) {
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
@@ -335,7 +362,7 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
           }
         }
       }
-    }
+    });
     // ---- defect rows: the right node's share comes from lane+1 (or the next warp's lane 0)
     double nbp[3], nbA[3], nbF[3];
 #pragma unroll
@@ -360,16 +387,16 @@ __global__ void __launch_bounds__(GT) k_god(const __grid_constant__ GodArgs a) {
         const int64_t row = a.nb + (int64_t)k * N + j;
         if (sC) {
           const double right = (lane == 31) ? sEdge[(warp + 1) * 3 + k] : nbp[k];
-          a.c[row] = gsub(a, right, pa[k]);
+          a.c[row] = fsub(K0, right, pa[k]);
         }
         if (WJV) {
           const double right = (lane == 31) ? sEdge[3 * EW + (warp + 1) * 3 + k] : nbA[k];
-          a.ojv[row] = gadd(a, jB[k], right);
+          a.ojv[row] = fadd(K0, jB[k], right);
         }
         if (FREE && WJ && sJ) {  // the tf entry closes the row
           const double right = (lane == 31) ? sEdge[6 * EW + (warp + 1) * 3 + k] : nbF[k];
           const int off = (k == 0) ? t * CR + CR - 1 : (k == 1) ? OV + t * CV + CV - 1 : OM + t * CM + CM - 1;
-          sm[off] = gadd(a, fk[k], right);
+          sm[off] = fadd(K0, fk[k], right);
         }
       }
     }
@@ -443,6 +470,7 @@ static void fill_god(const ocp* h, GodArgs& a) {
   for (int k = 0; k < 3; ++k) a.finpos[k] = -1;
   for (size_t i = 0; i < P.fin.size(); ++i) a.finpos[P.fin[i]] = (int)i;
   a.one = 1.0;
+  a.many = soft_launch(h->N + 1, h->num_sms);
   a.mz = -0.0;
   a.partials = h->d_partials;
   a.counter = h->d_counter;
@@ -454,7 +482,9 @@ static cudaError_t god_launch(const GodArgs& a, cudaStream_t s) {
   const size_t smem = (OUT & O_J) ? sizeof(double) * (size_t)(16 + 3 * F1) * (GT - 1) : 0;
   const int64_t tiles = a.ntiles - a.tile0;
   const int grid = (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff);
-  k_god<OUT, FREE><<<grid, GT, smem, s>>>(a);  // (G_DP, G_PAR bits in OUT)
+  constexpr bool DYN = (OUT & (O_C | O_J | O_H | O_JV | O_JTV | O_HV)) != 0;   // the dynamics' products
+  if (DYN && a.many) k_god<OUT, FREE, DYN><<<grid, GT, smem, s>>>(a);  // (G_DP, G_PAR bits in OUT)
+  else k_god<OUT, FREE, false><<<grid, GT, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -24,6 +24,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstring>
+
+#include "soft_mul.cuh"
+
 namespace ocpg {
 
 // Kernel-side model constants (filled by the host from the handle's parameters).
@@ -33,7 +37,46 @@ struct ModelConst {
   double one;      // 1.0 and -0.0, passed at run time (see fadd / fmul below)
   double mz;
   double c[16];    // model-specific precomputed constants (see each model)
+  int soft;        // this launch uses integer products (soft_launch and soft_consts)
+  int many;        // soft_launch alone (for parameters that are read on the device)
 };
+
+// Classes of a node's plain products: intermediates of the dynamics, entries of the Jacobian, of
+// the Hessian, of the gradient and objective, and the terms of Jv, J^T w and H v.
+enum : unsigned { MUL_P = 1u, MUL_J = 2u, MUL_H = 4u, MUL_G = 8u, MUL_V = 16u, MUL_ALL = 31u };
+
+// The constants of a node's work whose plain products of the classes in MASK run on the integer
+// pipes (soft_mul.cuh).  Functions of the node work take either type: fmul<class> is the integer
+// product for those classes, and `worst` keeps the furthest exponent sum (the work is redone
+// with ModelConst beyond SOFT_SPAN).
+template <unsigned MASK>
+struct SoftConst : ModelConst {
+  mutable uint32_t worst;
+  __device__ __forceinline__ explicit SoftConst(const ModelConst& k) : ModelConst(k), worst(0u) {}
+};
+
+// Integer products pay where the FP64 pipe is saturated: from two warps of nodes per sub-partition
+// on.  A warp alone issues an FP64 instruction every 64 cycles whatever it depends on, and an integer
+// product's 34 dependent instructions take it longer (evaluation, N = 8000: Van der Pol 8.9 us without
+// and 10.2 with them, Goddard 12.8 and 14.6; N = 30000: 8.8 and 9.6, cart-pole 14.9 and 14.7; N = 1e5: 13.5 and
+// 12.7, cart-pole 31.1 and 25.0, Goddard 27.1 and 22.9).
+inline bool soft_launch(int64_t nodes, int num_sms) { return nodes >= (int64_t)256 * num_sms; }
+
+// h/2 and the first n model constants: non-zero and of moderate size
+__host__ __device__ __forceinline__ bool soft_consts(const ModelConst& K, int n) {
+  auto hi = [](const double& v) {
+#ifdef __CUDA_ARCH__
+    return (uint32_t)__double2hiint(v);
+#else
+    uint64_t b;
+    memcpy(&b, &v, 8);
+    return (uint32_t)(b >> 32);
+#endif
+  };
+  bool ok = soft_input_hi(hi(K.hh));
+  for (int i = 0; i < n; ++i) ok = ok && soft_input_hi(hi(K.c[i]));
+  return ok;
+}
 
 // GB300's FP64 pipe sustains FMAs at its full rate but separate adds and multiplies about 18%
 // slower (measured), so sums, differences and products are issued as FMAs against the run-time
@@ -42,7 +85,26 @@ struct ModelConst {
 // from kernel parameters so that the compiler cannot fold the FMAs back.
 __device__ __forceinline__ double fadd(const ModelConst& K, double a, double b) { return fma(a, K.one, b); }
 __device__ __forceinline__ double fsub(const ModelConst& K, double a, double b) { return fma(-b, K.one, a); }
+template <unsigned C = MUL_P>
 __device__ __forceinline__ double fmul(const ModelConst& K, double a, double b) { return fma(a, b, K.mz); }
+template <unsigned C = MUL_P, unsigned MASK>
+__device__ __forceinline__ double fmul(const SoftConst<MASK>& K, double a, double b) {
+  if constexpr ((MASK & C) == 0) return fma(a, b, K.mz);
+  uint32_t x;
+  const double r = soft_product(a, b, x);
+  K.worst = max(K.worst, x - SOFT_BASE);   // (unsigned: sums below the range wrap to large values)
+  return r;
+}
+// c * v, c a cost weight or diagonal that may be zero for the whole launch (a zero with the product's sign)
+template <unsigned C>
+__device__ __forceinline__ double fmul_w(const ModelConst& K, double c, double v) { return fmul<C>(K, c, v); }
+template <unsigned C, unsigned MASK>
+__device__ __forceinline__ double fmul_w(const SoftConst<MASK>& K, double c, double v) {
+  if constexpr ((MASK & C) == 0) return fma(c, v, K.mz);
+  const int hi = __double2hiint(c);
+  if (((hi << 1) | __double2loint(c)) == 0) return __hiloint2double((hi ^ __double2hiint(v)) & (int)0x80000000, 0);
+  return fmul<C>(K, c, v);
+}
 
 // Operand sources matter as well (measured with the library's FP64 throughput probe, all
 // operands independent): an FMA whose multiplier is a register issues at the pipe's full rate,
@@ -67,6 +129,22 @@ __device__ __forceinline__ double recip(double one, double d) {
   r = fma(r, e, r);
   e = fma(-d, r, one);
   return fma(r, e, r);
+}
+
+// The same in a node's work, whose integer products rely on a moderate denominator.
+__device__ __forceinline__ double recip(const ModelConst& K, double d) { return recip(K.one, d); }
+template <unsigned MASK>
+__device__ __forceinline__ double recip(const SoftConst<MASK>& K, double d) {
+  if (!soft_value(d)) K.worst = 0xffffffffu;
+  return recip(K.one, d);
+}
+
+// The double of an integer 0 <= |k| < 2^24, without the FP64 pipe (a conversion instruction takes
+// a slot of it): through the float of k, whose fields move to the double's places.
+__device__ __forceinline__ double small_int(int k) {
+  const uint32_t f = __float_as_uint(__int2float_rn(k));
+  const uint32_t hi = (f & 0x80000000u) | (((f & 0x7fffffffu) >> 3) + 0x38000000u);
+  return __hiloint2double(k == 0 ? 0 : (int)hi, (int)(f << 29));
 }
 
 // sin x and cos x together, without the library routine's branches (CUDA's sincos executes about

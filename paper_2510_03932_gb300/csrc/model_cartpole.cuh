@@ -1,6 +1,7 @@
 // Device model of the cart-pole dynamics (the conventions of every model are stated in
 // model_base.cuh).
 #pragma once
+#include "kernel_config.h"
 #include "model_base.cuh"
 #include "sincos_table.cuh"
 
@@ -31,7 +32,18 @@ namespace ocpg {
 // only through the constants hh/l (defects, Jacobian) and the multiplier of the Hessian terms.
 // ------------------------------------------------------------------------------------
 struct CartPole {
-  static constexpr int EVAL_MIN_CTAS = 0;
+  // classes of products on the integer pipes (see soft_kernel), at N = 1e6: step 293.8 -> 223.9 us,
+  // evaluation 209.4 -> 155.5, J + H 160.1 -> 103.3, J 108.8 -> 69.6, H 135.9 -> 90.6, c 84.4 -> 67.9, Jv
+  // 139.5 -> 92.5, J^T w 127.5 -> 87.5, Hv 160.1 -> 98.8, (dc/dp)^T w with J^T w 249.9 -> 197
+  template <unsigned OUT> static constexpr unsigned SOFT = OUT == O_G ? 0u : MUL_ALL;
+  // resident CTAs of 128 (see min_ctas): with the step capped at 96 registers (224 us; 231 uncapped), the
+  // evaluation and J + H at 72 (155 and 103 us; 177 and 105); the gradient, which has none, at 80 (14.7 us; 20.8)
+  template <unsigned OUT> static constexpr int CTAS =
+      OUT == O_STEP ? 5 : (OUT == O_ALL || OUT == (O_J | O_H) || OUT == O_H) ? 7 : (OUT == O_JTV || OUT == O_HV) ? 6 : 0;
+  template <unsigned OUT> static constexpr int CTAS_FP64 = OUT == O_G ? 6 : 0;   // without integer products
+  template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  static constexpr int EVAL_TILE = TILE_CARTPOLE;
+  static constexpr int NC = 15;  // leading constants c[] that products use
   static constexpr int NX = 4, NU = 1, NZ = 5;
   static constexpr int MAXRX = 3, MAXRU = 1;
   OCP_TABLE1(RX, int, NX, {2, 3, 2, 2})
@@ -80,8 +92,8 @@ struct CartPole {
   //   dthdd/dl  = -(mp s w^2 c / D + Bu / l) / l,   dthdd/dg = -(mc + mp) s / (l D)
   // (D_mc = 1, D_mp = s^2; A and B are linear in each parameter).
   static constexpr bool FUSED_DP = true;
-  template <bool WC, bool WJ, bool WH, bool WP = false>
-  __device__ __forceinline__ static void eval(const ModelConst& K, const double (&z)[NZ], const double (&yb)[NX],
+  template <bool WC, bool WJ, bool WH, bool WP = false, class KC>
+  __device__ __forceinline__ static void eval(const KC& K, const double (&z)[NZ], const double (&yb)[NX],
                                               const double (&cqd)[NZ], double (&pa)[NX], double (&pb)[NX],
                                               double (&mjx)[NX][MAXRX], double (&mju)[NX][MAXRU],
                                               double (&hd)[NHD], double (*mdp)[NP] = nullptr) {
@@ -93,7 +105,7 @@ struct CartPole {
     sincos_tab(K, th, s, c);
     const double ms = fmul(K, mp, s);
     const double D = fma(ms, s, mcm);
-    const double iD = recip(K.one, D);
+    const double iD = recip(K, D);
     const double w2 = fmul(K, w, w);
     const double lw2 = fmul(K, l, w2);
     const double gl = fma(g, c, lw2);             // l w^2 + g c
@@ -125,11 +137,11 @@ struct CartPole {
       const double mhiD = fmul(K, mhh, iD);
       if (WJ) {
         mjx[0][0] = 0.0; mjx[0][1] = mhh; mjx[0][2] = 0.0;
-        mjx[1][0] = 0.0; mjx[1][1] = fmul(K, mhh, pdd_t); mjx[1][2] = fmul(K, mhiD, A_w);
+        mjx[1][0] = 0.0; mjx[1][1] = fmul<MUL_J>(K, mhh, pdd_t); mjx[1][2] = fmul<MUL_J>(K, mhiD, A_w);
         mju[1][0] = mhiD;
         mjx[2][0] = 0.0; mjx[2][1] = mhh; mjx[2][2] = 0.0;
-        mjx[3][0] = fmul(K, mhhil, Bu_t); mjx[3][1] = fmul(K, mhhil, Bu_w);
-        mju[3][0] = fmul(K, mhhil, Bu_F);
+        mjx[3][0] = fmul<MUL_J>(K, mhhil, Bu_t); mjx[3][1] = fmul<MUL_J>(K, mhhil, Bu_w);
+        mju[3][0] = fmul<MUL_J>(K, mhhil, Bu_F);
       }
       if (WP) {
 #pragma unroll
@@ -150,14 +162,14 @@ struct CartPole {
         // Every second derivative above is (numerator) / D: the multipliers carry the 1/D (and
         // for the angular rows the 1/l), m1 = -hh ybar_1 / D and m3 = -hh ybar_3 / (l D), and the
         // numerators are combined directly (those of the angular rows scaled by l).
-        const double m1 = fmul(K, mhiD, yb[1]), m3 = fmul(K, fmul(K, mhhil, yb[3]), iD);
-        const double Dpp = fmul(K, mp2, c2s2);
-        const double mDp2 = fmul(K, -2.0, Dp);
+        const double m1 = fmul<MUL_H>(K, mhiD, yb[1]), m3 = fmul<MUL_H>(K, fmul<MUL_H>(K, mhhil, yb[3]), iD);
+        const double Dpp = fmul<MUL_H>(K, mp2, c2s2);
+        const double mDp2 = fmul<MUL_H>(K, -2.0, Dp);
         // A_tt = -mp s (l w^2 + 4 g c)
-        const double A_tt = fmul(K, -ms, fma(g4, c, lw2));
+        const double A_tt = fmul<MUL_H>(K, -ms, fma(g4, c, lw2));
         const double n_pdd_tt = fma(-pdd, Dpp, fma(pdd_t, mDp2, A_tt));
         // B_tt = F c + 4 mp l w^2 s c + (mc+mp) g s = -B + 3 mp l w^2 s c
-        const double B_tt = fma(sc, fmul(K, K.c[13], w2), -B);
+        const double B_tt = fma(sc, fmul<MUL_H>(K, K.c[13], w2), -B);
         const double n_bu_tt = fma(-Bu, Dpp, fma(Bu_t, mDp2, B_tt));
         hd[0] = fma(m1, n_pdd_tt, fma(m3, n_bu_tt, cqd[2]));   // (th, th)
         // The other three entries, with t = m3 c - m1 and e = D' / D, from
@@ -166,17 +178,19 @@ struct CartPole {
         //   pdd_tw = 2 mp l w (c - s e) / D,  Bu_tw = -2 mp l w (c^2 - s^2 - s c e) / D
         //                                    -> (w, th) = 2 mp l w (m1 c - m3 (c^2 - s^2) + e s t)
         const double t = fma(m3, c, -m1);
-        const double e = fmul(K, Dp, iD);
-        hd[1] = fmul(K, lw, fma(fmul(K, e, s), t, fma(m1, c, -fmul(K, m3, c2s2))));   // (w, th)
-        hd[2] = fma(-t, fmul(K, mpl2, s), cqd[3]);                                  // (w, w)
-        hd[3] = fma(e, t, fmul(K, m3, s));                                          // (F, th)
+        const double e = fmul<MUL_H>(K, Dp, iD);
+        hd[1] = fmul<MUL_H>(K, lw, fma(fmul<MUL_H>(K, e, s), t, fma(m1, c, -fmul<MUL_H>(K, m3, c2s2))));   // (w, th)
+        hd[2] = fma(-t, fmul<MUL_H>(K, mpl2, s), cqd[3]);                                  // (w, w)
+        hd[3] = fma(e, t, fmul<MUL_H>(K, m3, s));                                          // (F, th)
       }
     }
   }
-  __device__ __forceinline__ static void dparam(const ModelConst&, const double (&)[NZ], double (&mdp)[NX]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparam(const KC&, const double (&)[NZ], double (&mdp)[NX]) {
     mdp[0] = mdp[1] = mdp[2] = mdp[3] = 0.0;
   }
-  __device__ __forceinline__ static void dparam_grad(const ModelConst&, const double (&)[NZ], const double (&)[NX],
+  template <class KC>
+  __device__ __forceinline__ static void dparam_grad(const KC&, const double (&)[NZ], const double (&)[NX],
                                                      double (&out)[NZ]) {
     for (int v = 0; v < NZ; ++v) out[v] = 0.0;
   }

@@ -1,6 +1,7 @@
 // Device model of the double integrator dynamics (the conventions of every model are stated in
 // model_base.cuh).
 #pragma once
+#include "kernel_config.h"
 #include "model_base.cuh"
 
 namespace ocpg {
@@ -9,7 +10,12 @@ namespace ocpg {
 // Double integrator (paper Sec. 5):  f0 = x2,  f1 = u.  Linear: no Hessian.
 // ------------------------------------------------------------------------------------
 struct Dint {
-  static constexpr int EVAL_MIN_CTAS = 0;
+  template <unsigned OUT> static constexpr int CTAS = 0;
+  template <unsigned OUT> static constexpr unsigned SOFT = 0u;  // (see soft_kernel)
+  template <unsigned OUT> static constexpr int CTAS_FP64 = 0;   // without integer products
+  template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  static constexpr int EVAL_TILE = TILE_DINT;
+  static constexpr int NC = 0;  // leading constants c[] that products use
   static constexpr int NX = 2, NU = 1, NZ = 3;
   static constexpr int MAXRX = 2, MAXRU = 1;
   OCP_TABLE1(RX, int, NX, {2, 1})
@@ -35,8 +41,8 @@ struct Dint {
   __device__ __forceinline__ static void device_param(ModelConst&, double) {}
   __device__ __forceinline__ static void device_params(ModelConst&, const double*) {}
 
-  template <bool WC, bool WJ, bool WH>
-  __device__ __forceinline__ static void eval(const ModelConst& K, const double (&z)[NZ], const double (&)[NX],
+  template <bool WC, bool WJ, bool WH, class KC>
+  __device__ __forceinline__ static void eval(const KC& K, const double (&z)[NZ], const double (&)[NX],
                                               const double (&)[NZ], double (&pa)[NX], double (&pb)[NX],
                                               double (&mjx)[NX][MAXRX], double (&mju)[NX][MAXRU], double (&)[1]) {
     if (WJ) {
@@ -52,13 +58,16 @@ struct Dint {
       pb[1] = fma(K.mhh, z[2], z[1]);
     }
   }
-  __device__ __forceinline__ static void dparam(const ModelConst&, const double (&)[NZ], double (&mdp)[NX]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparam(const KC&, const double (&)[NZ], double (&mdp)[NX]) {
     mdp[0] = 0.0; mdp[1] = 0.0;
   }
-  __device__ __forceinline__ static void dparams(const ModelConst&, const double (&)[NZ], double (&mdp)[NX][1]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparams(const KC&, const double (&)[NZ], double (&mdp)[NX][1]) {
     mdp[0][0] = 0.0; mdp[1][0] = 0.0;
   }
-  __device__ __forceinline__ static void dparam_grad(const ModelConst&, const double (&)[NZ], const double (&)[NX],
+  template <class KC>
+  __device__ __forceinline__ static void dparam_grad(const KC&, const double (&)[NZ], const double (&)[NX],
                                                      double (&out)[NZ]) {
     out[0] = out[1] = out[2] = 0.0;
   }

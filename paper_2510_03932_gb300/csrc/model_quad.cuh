@@ -1,6 +1,7 @@
 // Device model of the quadrotor dynamics (the conventions of every model are stated in
 // model_base.cuh).
 #pragma once
+#include "kernel_config.h"
 #include "model_base.cuh"
 #include "sincos_table.cuh"
 
@@ -30,10 +31,21 @@ namespace ocpg {
 // Constants: c[0] = g.
 // ------------------------------------------------------------------------------------
 struct Quadrotor {
-  // 3 CTAs of 128 threads per SM (168 registers) for the evaluation kernels: measured faster than
-  // the allocator's own choice (14% for the evaluation, 4% for the fused step, at 64-node tiles
-  // and 6 CTAs) and than 4 CTAs (128 registers, larger spills: fused step 911 vs 832 us)
-  static constexpr int EVAL_MIN_CTAS = 3;
+  // classes of products on the integer pipes (see soft_kernel), at N = 1e6: Jv 274.5 -> 193 us, J^T w
+  // 252.3 -> 180, Hv 324.0 -> 231, H 242.1 -> 188, c 180.6 -> 145.8, objective 97.4 -> 69, gradient 78.3 -> 66;
+  // none in the kernels with the Jacobian rows, which run three warps per sub-partition and are
+  // bound by latency (with every product the evaluation takes 484 us instead of 455 and the step
+  // 1369 instead of 781; with the gradient's and the products' alone 446 and 755, but 68 instead of 67
+  // and 112 instead of 105 at N = 1e5)
+  template <unsigned OUT> static constexpr unsigned SOFT = (OUT & O_J) ? 0u : MUL_ALL;
+  // resident CTAs (see min_ctas), of 128 threads for the evaluation kernels: 3 at 168 registers (4 at 128
+  // spill), H alone 4 (188 us; 203 at 3); of 64 for the products: 8
+  template <unsigned OUT> static constexpr int CTAS =
+      (OUT == O_JV || OUT == O_JTV || OUT == O_HV) ? 8 : OUT == O_H ? 4 : 0;
+  template <unsigned OUT> static constexpr int CTAS_FP64 = (OUT == O_JV || OUT == O_JTV || OUT == O_HV) ? 0 : 3;   // without integer products
+  template <unsigned OUT> static constexpr int CTAS_EULER = OUT == O_STEP ? 3 : 0;  // (N = 50000: 69.2 us uncapped, 51.5)
+  static constexpr int EVAL_TILE = TILE_QUAD_EVAL;
+  static constexpr int NC = 0;  // leading constants c[] that products use
   static constexpr int NX = 9, NU = 4, NZ = 13;
   static constexpr int MAXRX = 4, MAXRU = 3;
   OCP_TABLE1(RX, int, NX, {2, 4, 2, 4, 2, 3, 2, 2, 3})
@@ -66,8 +78,8 @@ struct Quadrotor {
   __device__ __forceinline__ static void device_param(ModelConst&, double) {}
   __device__ __forceinline__ static void device_params(ModelConst& K, const double* p) { K.c[0] = __ldg(p); }
 
-  template <bool WC, bool WJ, bool WH>
-  __device__ __forceinline__ static void eval(const ModelConst& K, const double (&z)[NZ], const double (&yb)[NX],
+  template <bool WC, bool WJ, bool WH, class KC>
+  __device__ __forceinline__ static void eval(const KC& K, const double (&z)[NZ], const double (&yb)[NX],
                                               const double (&cqd)[NZ], double (&pa)[NX], double (&pb)[NX],
                                               double (&mjx)[NX][MAXRX], double (&mju)[NX][MAXRU],
                                               double (&hd)[NHD]) {
@@ -77,7 +89,7 @@ struct Quadrotor {
     sincos_tab(K, z[6], s7, c7);
     sincos_tab(K, z[7], s8, c8);
     sincos_tab(K, z[8], s9, c9);
-    const double e = recip(K.one, c8);
+    const double e = recip(K, c8);
     const double t = fmul(K, s8, e);
     const double c7s8 = fmul(K, c7, s8), s7s8 = fmul(K, s7, s8);
     const double c7c8 = fmul(K, c7, c8), s7c8 = fmul(K, s7, c8);
@@ -103,67 +115,70 @@ struct Quadrotor {
       const double Q8 = fmul(K, c7c8, s9);
       const double e2 = fmul(K, e, e);
       if (WJ) {
-        const double mu1 = fmul(K, mhh, u1);
+        const double mu1 = fmul<MUL_J>(K, mhh, u1);
         mjx[0][0] = 0.0; mjx[0][1] = mhh;
-        mjx[1][0] = 0.0; mjx[1][1] = fmul(K, mu1, P7); mjx[1][2] = fmul(K, mu1, P8); mjx[1][3] = fmul(K, mu1, P9);
-        mju[1][0] = fmul(K, mhh, P);
+        mjx[1][0] = 0.0; mjx[1][1] = fmul<MUL_J>(K, mu1, P7); mjx[1][2] = fmul<MUL_J>(K, mu1, P8); mjx[1][3] = fmul<MUL_J>(K, mu1, P9);
+        mju[1][0] = fmul<MUL_J>(K, mhh, P);
         mjx[2][0] = 0.0; mjx[2][1] = mhh;
-        mjx[3][0] = 0.0; mjx[3][1] = fmul(K, mu1, Q7); mjx[3][2] = fmul(K, mu1, Q8); mjx[3][3] = fmul(K, mu1, P);
-        mju[3][0] = fmul(K, mhh, Q);
+        mjx[3][0] = 0.0; mjx[3][1] = fmul<MUL_J>(K, mu1, Q7); mjx[3][2] = fmul<MUL_J>(K, mu1, Q8); mjx[3][3] = fmul<MUL_J>(K, mu1, P);
+        mju[3][0] = fmul<MUL_J>(K, mhh, Q);
         mjx[4][0] = 0.0; mjx[4][1] = mhh;
-        mjx[5][0] = 0.0; mjx[5][1] = fmul(K, -mu1, s7c8); mjx[5][2] = fmul(K, -mu1, c7s8);
-        mju[5][0] = fmul(K, mhh, c7c8);
-        const double mhe = fmul(K, mhh, e);
-        mjx[6][0] = fmul(K, mhe, b); mjx[6][1] = fmul(K, fmul(K, mhh, ae), t);
-        mju[6][0] = fmul(K, mhe, c7); mju[6][1] = fmul(K, mhe, s7);
-        mjx[7][0] = fmul(K, hh, a); mjx[7][1] = 0.0;
-        mju[7][0] = fmul(K, hh, s7); mju[7][1] = fmul(K, mhh, c7);
-        const double mht = fmul(K, mhh, t);
-        mjx[8][0] = fmul(K, mht, b); mjx[8][1] = fmul(K, fmul(K, mhh, a), e2); mjx[8][2] = 0.0;
-        mju[8][0] = fmul(K, mht, c7); mju[8][1] = fmul(K, mht, s7); mju[8][2] = mhh;
+        mjx[5][0] = 0.0; mjx[5][1] = fmul<MUL_J>(K, -mu1, s7c8); mjx[5][2] = fmul<MUL_J>(K, -mu1, c7s8);
+        mju[5][0] = fmul<MUL_J>(K, mhh, c7c8);
+        const double mhe = fmul<MUL_J>(K, mhh, e);
+        mjx[6][0] = fmul<MUL_J>(K, mhe, b); mjx[6][1] = fmul<MUL_J>(K, fmul<MUL_J>(K, mhh, ae), t);
+        mju[6][0] = fmul<MUL_J>(K, mhe, c7); mju[6][1] = fmul<MUL_J>(K, mhe, s7);
+        mjx[7][0] = fmul<MUL_J>(K, hh, a); mjx[7][1] = 0.0;
+        mju[7][0] = fmul<MUL_J>(K, hh, s7); mju[7][1] = fmul<MUL_J>(K, mhh, c7);
+        const double mht = fmul<MUL_J>(K, mhh, t);
+        mjx[8][0] = fmul<MUL_J>(K, mht, b); mjx[8][1] = fmul<MUL_J>(K, fmul<MUL_J>(K, mhh, a), e2); mjx[8][2] = 0.0;
+        mju[8][0] = fmul<MUL_J>(K, mht, c7); mju[8][1] = fmul<MUL_J>(K, mht, s7); mju[8][2] = mhh;
       }
       if (WH) {
         // -hh ybar_k for the rows with a Hessian, and the u1-scaled ones of the rotation rows
-        const double m1 = fmul(K, mhh, yb[1]), m3 = fmul(K, mhh, yb[3]), m5 = fmul(K, mhh, yb[5]);
-        const double m6 = fmul(K, mhh, yb[6]), m7 = fmul(K, mhh, yb[7]), m8 = fmul(K, mhh, yb[8]);
-        const double w1 = fmul(K, m1, u1), w3 = fmul(K, m3, u1), w5 = fmul(K, m5, u1);
-        const double A1 = fma(m6, e, fmul(K, m8, t));      // coefficient of -a at (x7, x7) and of -s7 / c7
-        const double B1 = fma(m6, t, fmul(K, m8, e));      // (x8, x7) and mixed x8 terms, times e
-        const double C1 = fma(w1, c9, fmul(K, w3, s9));
-        const double PQ = fma(w1, P, fmul(K, w3, Q));
+        const double m1 = fmul<MUL_H>(K, mhh, yb[1]), m3 = fmul<MUL_H>(K, mhh, yb[3]), m5 = fmul<MUL_H>(K, mhh, yb[5]);
+        const double m6 = fmul<MUL_H>(K, mhh, yb[6]), m7 = fmul<MUL_H>(K, mhh, yb[7]), m8 = fmul<MUL_H>(K, mhh, yb[8]);
+        const double w1 = fmul<MUL_H>(K, m1, u1), w3 = fmul<MUL_H>(K, m3, u1), w5 = fmul<MUL_H>(K, m5, u1);
+        const double A1 = fma(m6, e, fmul<MUL_H>(K, m8, t));      // coefficient of -a at (x7, x7) and of -s7 / c7
+        const double B1 = fma(m6, t, fmul<MUL_H>(K, m8, e));      // (x8, x7) and mixed x8 terms, times e
+        const double C1 = fma(w1, c9, fmul<MUL_H>(K, w3, s9));
+        const double PQ = fma(w1, P, fmul<MUL_H>(K, w3, Q));
         // (x7, x7)
         hd[0] = fsub(K, cqd[6], fma(w5, c7c8, fma(a, A1, fma(m7, b, PQ))));
         // (x8, x7)
-        hd[1] = fma(fmul(K, b, e), B1, fma(w5, s7s8, fmul(K, -s7c8, C1)));
+        hd[1] = fma(fmul<MUL_H>(K, b, e), B1, fma(w5, s7s8, fmul<MUL_H>(K, -s7c8, C1)));
         // (x8, x8): a e (m6 (t^2 + e^2) + 2 m8 e t)
-        const double q88 = fma(m6, fma(t, t, e2), fmul(K, fmul(K, 2.0, m8), fmul(K, e, t)));
-        hd[2] = fma(ae, q88, fsub(K, cqd[7], fma(c7s8, C1, fmul(K, w5, c7c8))));
+        const double q88 = fma(m6, fma(t, t, e2), fmul<MUL_H>(K, fmul<MUL_H>(K, 2.0, m8), fmul<MUL_H>(K, e, t)));
+        hd[2] = fma(ae, q88, fsub(K, cqd[7], fma(c7s8, C1, fmul<MUL_H>(K, w5, c7c8))));
         // (x9, x7), (x9, x8), (x9, x9)
-        hd[3] = fma(w3, P7, fmul(K, -w1, Q7));
-        hd[4] = fma(w3, P8, fmul(K, -w1, Q8));
+        hd[3] = fma(w3, P7, fmul<MUL_H>(K, -w1, Q7));
+        hd[4] = fma(w3, P8, fmul<MUL_H>(K, -w1, Q8));
         hd[5] = fsub(K, cqd[8], PQ);
         // (u1, x7), (u1, x8), (u1, x9)
-        hd[6] = fma(m1, P7, fma(m3, Q7, fmul(K, -m5, s7c8)));
-        hd[7] = fma(m1, P8, fma(m3, Q8, fmul(K, -m5, c7s8)));
-        hd[8] = fma(m1, P9, fmul(K, m3, P));
+        hd[6] = fma(m1, P7, fma(m3, Q7, fmul<MUL_H>(K, -m5, s7c8)));
+        hd[7] = fma(m1, P8, fma(m3, Q8, fmul<MUL_H>(K, -m5, c7s8)));
+        hd[8] = fma(m1, P9, fmul<MUL_H>(K, m3, P));
         // (u2, x7), (u2, x8), (u3, x7), (u3, x8)
-        hd[9] = fma(-s7, A1, fmul(K, -m7, c7));
-        hd[10] = fmul(K, fmul(K, c7, e), B1);
-        hd[11] = fma(c7, A1, fmul(K, -m7, s7));
-        hd[12] = fmul(K, fmul(K, s7, e), B1);
+        hd[9] = fma(-s7, A1, fmul<MUL_H>(K, -m7, c7));
+        hd[10] = fmul<MUL_H>(K, fmul<MUL_H>(K, c7, e), B1);
+        hd[11] = fma(c7, A1, fmul<MUL_H>(K, -m7, s7));
+        hd[12] = fmul<MUL_H>(K, fmul<MUL_H>(K, s7, e), B1);
       }
     }
   }
-  __device__ __forceinline__ static void dparam(const ModelConst&, const double (&)[NZ], double (&mdp)[NX]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparam(const KC&, const double (&)[NZ], double (&mdp)[NX]) {
     for (int k = 0; k < NX; ++k) mdp[k] = 0.0;
   }
   // -hh df_k/dg: only x6' = u1 R - g depends on g
-  __device__ __forceinline__ static void dparams(const ModelConst& K, const double (&)[NZ], double (&mdp)[NX][NP]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparams(const KC& K, const double (&)[NZ], double (&mdp)[NX][NP]) {
 #pragma unroll
     for (int k = 0; k < NX; ++k) mdp[k][0] = 0.0;
     mdp[5][0] = K.hh;
   }
-  __device__ __forceinline__ static void dparam_grad(const ModelConst&, const double (&)[NZ], const double (&)[NX],
+  template <class KC>
+  __device__ __forceinline__ static void dparam_grad(const KC&, const double (&)[NZ], const double (&)[NX],
                                                      double (&out)[NZ]) {
     for (int v = 0; v < NZ; ++v) out[v] = 0.0;
   }

@@ -1,6 +1,7 @@
 // Device model of the Van der Pol dynamics (the conventions of every model are stated in
 // model_base.cuh).
 #pragma once
+#include "kernel_config.h"
 #include "model_base.cuh"
 
 namespace ocpg {
@@ -13,7 +14,19 @@ namespace ocpg {
 // Constants: c[0] = 2 hh mu, c[1] = hh mu, c[2] = -hh mu.
 // ------------------------------------------------------------------------------------
 struct VdP {
-  static constexpr int EVAL_MIN_CTAS = 0;
+  // classes of products on the integer pipes (see soft_kernel), at N = 1e6: step 101.2 -> 80.0 us,
+  // evaluation 58.0 -> 50.0, objective 23.3 -> 21.3, Jv 28.9 -> 22.9, J^T w 26.9 -> 20.9, Hv 24.8 -> 16.7
+  // (18.7 with its Hessian entries' two as well)
+  template <unsigned OUT> static constexpr unsigned SOFT =
+      OUT == O_HV ? MUL_ALL & ~MUL_H
+                  : (OUT == O_STEP || OUT == O_ALL || OUT == O_F || OUT == O_JV || OUT == O_JTV) ? MUL_ALL : 0u;
+  // resident CTAs of 256 (see min_ctas): the step's 48 registers (80.0 us; 83.4 at 64, 95.2 at the
+  // allocator's choice), the evaluation's 32 (50.0 us; 55.9)
+  template <unsigned OUT> static constexpr int CTAS = OUT == O_STEP ? 5 : (OUT == O_ALL || OUT == O_F) ? 8 : 0;
+  template <unsigned OUT> static constexpr int CTAS_FP64 = 0;   // without integer products
+  template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  static constexpr int EVAL_TILE = TILE_VDP;
+  static constexpr int NC = 3;  // leading constants c[] that products use
   static constexpr int NX = 2, NU = 1, NZ = 3;
   static constexpr int MAXRX = 2, MAXRU = 1;
   OCP_TABLE1(RX, int, NX, {2, 2})
@@ -47,8 +60,8 @@ struct VdP {
   }
   __device__ __forceinline__ static void device_params(ModelConst& K, const double* p) { device_param(K, __ldg(p)); }
 
-  template <bool WC, bool WJ, bool WH>
-  __device__ __forceinline__ static void eval(const ModelConst& K, const double (&z)[NZ], const double (&yb)[NX],
+  template <bool WC, bool WJ, bool WH, class KC>
+  __device__ __forceinline__ static void eval(const KC& K, const double (&z)[NZ], const double (&yb)[NX],
                                               const double (&cqd)[NZ], double (&pa)[NX], double (&pb)[NX],
                                               double (&mjx)[NX][MAXRX], double (&mju)[NX][MAXRU],
                                               double (&hd)[NHD]) {
@@ -60,7 +73,7 @@ struct VdP {
       if (WJ) {
         mjx[0][0] = 0.0;                              // x1 in row 0: identity only
         mjx[0][1] = K.mhh;                            // x2 in row 0: -hh * 1
-        mjx[1][0] = fma(K.c[0], fmul(K, x1, x2), K.hh);  // -hh (-2 mu x1 x2 - 1)
+        mjx[1][0] = fma(K.c[0], fmul<MUL_J>(K, x1, x2), K.hh);  // -hh (-2 mu x1 x2 - 1)
         mjx[1][1] = m12;
         mju[1][0] = K.mhh;
       }
@@ -74,26 +87,29 @@ struct VdP {
       }
     }
     if (WH) {
-      const double t = fmul(K, K.c[0], yb[1]);
+      const double t = fmul<MUL_H>(K, K.c[0], yb[1]);
       hd[0] = fma(t, x2, cqd[0]);   // (x1, x1)
-      hd[1] = fmul(K, t, x1);       // (x2, x1)
+      hd[1] = fmul<MUL_H>(K, t, x1);       // (x2, x1)
     }
   }
 
   // -hh df_k/dmu
-  __device__ __forceinline__ static void dparam(const ModelConst& K, const double (&z)[NZ], double (&mdp)[NX]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparam(const KC& K, const double (&z)[NZ], double (&mdp)[NX]) {
     const double x1 = z[0], x2 = z[1];
     mdp[0] = 0.0;
     mdp[1] = fmul(K, K.mhh, fmul(K, fma(-x1, x1, 1.0), x2));
   }
-  __device__ __forceinline__ static void dparams(const ModelConst& K, const double (&z)[NZ], double (&mdp)[NX][NP]) {
+  template <class KC>
+  __device__ __forceinline__ static void dparams(const KC& K, const double (&z)[NZ], double (&mdp)[NX][NP]) {
     double t[NX];
     dparam(K, z, t);
     mdp[0][0] = t[0];
     mdp[1][0] = t[1];
   }
   // sum_k wbar_k (-hh d2 f_k / dmu dz_v) for every local v
-  __device__ __forceinline__ static void dparam_grad(const ModelConst& K, const double (&z)[NZ],
+  template <class KC>
+  __device__ __forceinline__ static void dparam_grad(const KC& K, const double (&z)[NZ],
                                                      const double (&wb)[NX], double (&out)[NZ]) {
     const double x1 = z[0], x2 = z[1];
     const double t = fmul(K, K.mhh, wb[1]);

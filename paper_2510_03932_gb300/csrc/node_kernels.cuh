@@ -216,13 +216,16 @@ __device__ __forceinline__ void load_node(const NodeArgs<M>& a, int64_t j, doubl
 template <class M, bool PAR>
 __device__ __forceinline__ ModelConst launch_consts(const NodeArgs<M>& a) {
   ModelConst K = a.K;
-  if constexpr (PAR) M::device_params(K, a.p0_dev);
+  if constexpr (PAR) {
+    M::device_params(K, a.p0_dev);
+    K.soft = K.many && soft_consts(K, M::NC);
+  }
   return K;
 }
 
 // ybar_k = w_{k,j-1} + w_{k,j} over the defect rows of component k (zero outside 0..N-1)
-template <class M>
-__device__ __forceinline__ void load_bar(const NodeArgs<M>& a, const ModelConst& K, const double* w, int64_t j, double (&wb)[M::NX],
+template <class M, class KC>
+__device__ __forceinline__ void load_bar(const NodeArgs<M>& a, const KC& K, const double* w, int64_t j, double (&wb)[M::NX],
                                          double (&wl)[M::NX], double (&wr)[M::NX]) {
 #pragma unroll
   for (int k = 0; k < M::NX; ++k) {
@@ -242,8 +245,8 @@ __device__ __forceinline__ void node_cq(const NodeArgs<M>& a, bool endp, double 
   for (int v = 0; v < M::NZ; ++v) cqd[v] = endp ? a.cq_end[v] : a.cq_in[v];
 }
 
-template <class M>
-__device__ __forceinline__ void load_ybar(const NodeArgs<M>& a, const ModelConst& K, const double* w, int64_t j,
+template <class M, class KC>
+__device__ __forceinline__ void load_ybar(const NodeArgs<M>& a, const KC& K, const double* w, int64_t j,
                                           double (&wb)[M::NX]) {
 #pragma unroll
   for (int k = 0; k < M::NX; ++k) {
@@ -260,8 +263,8 @@ __device__ __forceinline__ void load_ybar(const NodeArgs<M>& a, const ModelConst
 
 // gradient entries g_v = 2 w_j q_v (z_v - ref_v); returns 2 w_j f0(z_j) = sum_v g_v (z_v - ref_v)
 // (ref_v of a tracked state component is read from the per-node table xtrack)
-template <class M, bool REF, bool WG>
-__device__ __forceinline__ double node_grad(const NodeArgs<M>& a, const ModelConst& K, const double (&z)[M::NZ], bool endp,
+template <class M, bool REF, bool WG, class KC>
+__device__ __forceinline__ double node_grad(const NodeArgs<M>& a, const KC& K, const double (&z)[M::NZ], bool endp,
                                            int64_t j) {
   double s = 0.0;
 #pragma unroll
@@ -270,12 +273,12 @@ __device__ __forceinline__ double node_grad(const NodeArgs<M>& a, const ModelCon
     if (REF && v < M::NX && a.xtrack && a.trk[v < M::NX ? v : 0] >= 0)
       rv = __ldg(a.xtrack + (int64_t)a.ntrk * j + a.trk[v < M::NX ? v : 0]);
     const double d = REF ? fsub(K, z[v], rv) : z[v];
-    const double gv = fmul(K, endp ? a.gq_end[v] : a.gq_in[v], d);
+    const double gv = fmul_w<MUL_G>(K, endp ? a.gq_end[v] : a.gq_in[v], d);
     if (WG) {
       if (v < M::NX) a.g[(int64_t)M::NX * j + v] = gv;
       else a.g[a.uoff + (int64_t)M::NU * j + (v - M::NX)] = gv;
     }
-    s = (v == 0) ? fmul(K, gv, d) : fma(gv, d, s);
+    s = (v == 0) ? fmul_w<MUL_G>(K, gv, d) : fma(gv, d, s);
   }
   return s;
 }
@@ -284,8 +287,8 @@ __device__ __forceinline__ double node_grad(const NodeArgs<M>& a, const ModelCon
 // Jv: with p_k = -hh grad f_k(z_j) . v_{z_j} (+ -hh df_k/dmu * pdir), A_k = p_k + v_{X_j,k} is the
 // node's share of row (k, j-1) and B_k = p_k - v_{X_j,k} its share of row (k, j); the last term
 // of p_k is fused into both.
-template <class M, bool PDIR>
-__device__ __forceinline__ void jv_node(const ModelConst& K, const double (&mjx)[M::NX][M::MAXRX],
+template <class M, bool PDIR, class KC>
+__device__ __forceinline__ void jv_node(const KC& K, const double (&mjx)[M::NX][M::MAXRX],
                                         const double (&mju)[M::NX][M::MAXRU],
                                         const double (&mdp)[M::NX], double pd, const double (&vz)[M::NZ],
                                         double (&A)[M::NX], double (&Bm)[M::NX]) {
@@ -303,7 +306,7 @@ __device__ __forceinline__ void jv_node(const ModelConst& K, const double (&mjx)
     if (PDIR) { cf[nt] = mdp[k]; vv[nt] = pd; ++nt; }
     double s = 0.0;
 #pragma unroll
-    for (int i = 0; i + 1 < nt; ++i) s = (i == 0) ? fmul(K, cf[i], vv[i]) : fma(cf[i], vv[i], s);
+    for (int i = 0; i + 1 < nt; ++i) s = (i == 0) ? fmul<MUL_V>(K, cf[i], vv[i]) : fma(cf[i], vv[i], s);
     const double vk = vz[k];
     if (nt == 0) {
       A[k] = vk;
@@ -322,8 +325,8 @@ __device__ __forceinline__ void jv_node(const ModelConst& K, const double (&mjx)
 
 // J^T w at node j: (w_{a,j-1} - w_{a,j}) + sum_k wbar_k mjx_{k,a}, the control entries
 // sum_k wbar_k mju_{k,i}, plus the boundary rows' w at j = 0 / N (bnd: this CTA may hold them).
-template <class M>
-__device__ __forceinline__ void jtv_node(const NodeArgs<M>& a, const ModelConst& K, const double* w, int64_t j, bool bnd,
+template <class M, class KC>
+__device__ __forceinline__ void jtv_node(const NodeArgs<M>& a, const KC& K, const double* w, int64_t j, bool bnd,
                                          const double (&mjx)[M::NX][M::MAXRX], const double (&mju)[M::NX][M::MAXRU],
                                          const double (&wl)[M::NX], const double (&wr)[M::NX],
                                          const double (&wb)[M::NX], double (&o)[M::NZ]) {
@@ -351,14 +354,14 @@ __device__ __forceinline__ void jtv_node(const NodeArgs<M>& a, const ModelConst&
     for (int k = 0; k < NX; ++k)
 #pragma unroll
       for (int e = 0; e < M::MAXRU; ++e)
-        if (e < M::RU(k) && M::UV(k, e) == i) { s = first ? fmul(K, wb[k], mju[k][e]) : fma(wb[k], mju[k][e], s); first = false; }
+        if (e < M::RU(k) && M::UV(k, e) == i) { s = first ? fmul<MUL_V>(K, wb[k], mju[k][e]) : fma(wb[k], mju[k][e], s); first = false; }
     o[NX + i] = s;
   }
 }
 
 // H v at node j: the full symmetric block (structural entries only) times v_{z_j}.
-template <class M>
-__device__ __forceinline__ void hv_node(const NodeArgs<M>& a, const ModelConst& K, const double* hd, const double (&cqd)[M::NZ],
+template <class M, class KC>
+__device__ __forceinline__ void hv_node(const NodeArgs<M>& a, const KC& K, const double* hd, const double (&cqd)[M::NZ],
                                         const double (&vz)[M::NZ], double (&o)[M::NZ]) {
   constexpr HTmpl<M> HT{};
   bool first[M::NZ];
@@ -369,10 +372,10 @@ __device__ __forceinline__ void hv_node(const NodeArgs<M>& a, const ModelConst& 
     if (a.hpos[e] >= 0) {
       const int aa = HT.a[e], bb = HT.b[e];
       const double val = (HT.dyn[e] >= 0) ? hd[HT.dyn[e] >= 0 ? HT.dyn[e] : 0] : cqd[aa];
-      o[aa] = first[aa] ? fmul(K, val, vz[bb]) : fma(val, vz[bb], o[aa]);
+      o[aa] = first[aa] ? (HT.dyn[e] >= 0 ? fmul<MUL_V>(K, val, vz[bb]) : fmul_w<MUL_V>(K, val, vz[bb])) : fma(val, vz[bb], o[aa]);
       first[aa] = false;
       if (aa != bb) {
-        o[bb] = first[bb] ? fmul(K, val, vz[aa]) : fma(val, vz[aa], o[bb]);
+        o[bb] = first[bb] ? fmul<MUL_V>(K, val, vz[aa]) : fma(val, vz[aa], o[bb]);
         first[bb] = false;
       }
     }
@@ -395,22 +398,91 @@ __device__ __forceinline__ void store_nz(const NodeArgs<M>& a, double* out, int6
   for (int i = 0; i < M::NU; ++i) out[a.uoff + M::NU * j + i] = o[M::NX + i];
 }
 
+// The classes of plain products that a kernel does on the integer pipes (soft_mul.cuh) in a large
+// launch (IP; chosen by soft_launch): where the FP64 pipe bounds it.  Not in the kernels near the HBM
+// rate, which the extra instructions and registers slow down (Van der Pol J + H 23.9 us at N = 1e6, its
+// gradient 10.5 -> 12.3 us with them), nor for the double integrator, whose products are its cost's alone.
+template <class M, unsigned OUT, bool IP>
+constexpr unsigned soft_kernel() { return IP ? M::template SOFT<OUT> : 0u; }
+
+// Resident CTAs per SM that a kernel's registers are capped for (0: the allocator's own choice).
+template <class M, unsigned OUT, bool IP, bool EULER = false>
+constexpr int min_ctas() { return soft_kernel<M, OUT, IP>() ? M::template CTAS<OUT> : EULER ? M::template CTAS_EULER<OUT> : M::template CTAS_FP64<OUT>; }
+
+// The inputs of a node's work that its products multiply (see soft_mul.cuh): the node's variables,
+// the multipliers of the rows with a Hessian, the directions.  High words only; the work's own
+// loads of the same lines follow.
+template <class M, bool Y, bool V, bool W>
+__device__ __forceinline__ bool soft_node(const NodeArgs<M>& a, const double* y, const double* v, const double* w, int64_t j) {
+  // (no short circuits: every load is issued before the first test waits; at j = 0 and j = N the
+  // missing row's place is taken by the other one)
+  const int64_t jl = max(j - 1, (int64_t)0), jr = min(j, a.N - 1);
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < M::NX; ++k) {
+    ok &= soft_input(a.x + M::NX * j + k);
+    if (V) ok &= soft_input(v + M::NX * j + k);
+    if (Y && M::HK(k)) {
+      const double* row = y + a.nb + (int64_t)k * a.N;
+      ok &= soft_input(row + jl) & soft_input(row + jr);
+    }
+    if (W) {
+      const double* row = w + a.nb + (int64_t)k * a.N;
+      ok &= soft_input(row + jl) & soft_input(row + jr);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < M::NU; ++i) {
+    ok &= soft_input(a.x + a.uoff + M::NU * j + i);
+    if (V) ok &= soft_input(v + a.uoff + M::NU * j + i);
+  }
+  return ok;
+}
+
+// The same for a node of the Euler scheme (its own rows' multipliers).
+template <class M, bool Y, bool V, bool W>
+__device__ __forceinline__ bool soft_euler(const NodeArgs<M>& a, const double* y, const double* v, const double* w, int64_t j) {
+  bool ok = soft_node<M, false, V, false>(a, nullptr, v, nullptr, j);
+#pragma unroll
+  for (int k = 0; k < M::NX; ++k) {
+    if (Y && M::HK(k)) ok &= soft_input(y + a.nb + (int64_t)k * a.N + j);
+    if (W) ok &= soft_input(w + a.nb + (int64_t)k * a.N + j);
+  }
+  return ok;
+}
+
+// Runs work(K) for the lanes with `act`, with the products of SoftConst where the warp's inputs
+// (ok) allow it and none came out of range, else (or again) with ModelConst: the same values, bit
+// for bit.  Called by whole warps.
+template <unsigned SOFT, class F>
+__device__ __forceinline__ void with_products(const ModelConst& K, bool act, bool ok, F&& work) {
+  bool done = false;
+  if constexpr (SOFT != 0) {
+    if (K.soft && __all_sync(0xffffffffu, !act || ok)) {   // (K.soft: the same for the whole launch)
+      const SoftConst<SOFT> KS(K);
+      if (act) work(KS);
+      done = __all_sync(0xffffffffu, KS.worst <= SOFT_SPAN);
+    }
+  }
+  if (!done && act) work(K);
+}
+
 // One tile of the fused evaluation.  The CTA's TILE threads cover NPT*TILE consecutive
 // nodes r0.. (thread t takes nodes r0 + NPT t + q, q < NPT: consecutive pairs give each thread
 // independent FP64 dependency chains) and own the first NPT*TILE - 1 of them.  `a` may live in
 // parameter or shared memory.  The tile's objective term (2 w_j f0 summed in a fixed order)
 // goes to *partial.
-template <class M, int TILE, int NPT, unsigned OUT>
-__device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const ModelConst& K, int64_t tile, double* sm,
+template <class M, int TILE, int NPT, unsigned OUT, bool IP>
+__device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const ModelConst& K0, int64_t tile, double* sm,
                                                double* sEdge, double* partial) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NT = NPT * TILE;  // nodes per tile
   constexpr bool WF = OUT & O_F, WC = OUT & O_C, WG = OUT & O_G, WJ = OUT & O_J, WH = OUT & O_H;
   constexpr bool WJV = OUT & O_JV, WJTV = OUT & O_JTV, WHV = OUT & O_HV;  // fused step products
   constexpr bool NEEDJ = WJ || WJV || WJTV, NEEDH = WH || WHV;
+  constexpr unsigned SOFT = soft_kernel<M, OUT, IP>();
   // the full kernel also serves output subsets: NULL outputs are computed but not stored
   const bool sF = WF && a.f, sC = WC && a.c, sG = WG && a.g, sJ = WJ && a.jv, sH = WH && a.hv;
-  constexpr HTmpl<M> HT{};
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   constexpr int R = NT - 1;            // owned rows / nodes per tile
   constexpr int oRED = (OUT & O_J) ? jrow_total<M>() * R : 0;
@@ -434,11 +506,16 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
     const bool act = j < eval_end;
     const bool own = lt < nown;
     const bool endp = (j == 0) || (j == a.N);
-    double z[NZ], yb[NX], cqd[NZ], mjx[NX][M::MAXRX], mju[NX][M::MAXRU], hd[NHD];
 #pragma unroll
     for (int k = 0; k < NX; ++k) { pa[q][k] = 0.0; pb[q][k] = 0.0; jA[q][k] = 0.0; jB[q][k] = 0.0; }
-    double vz[NZ];
-    if (act) {
+    bool ok = false;
+    if constexpr (SOFT != 0) {
+      if (K0.soft && act) ok = soft_node<M, NEEDH, (WJV || WHV), WJTV>(a, a.y, a.v, a.wv, j);
+    }
+    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
+      constexpr HTmpl<M> HT{};   // (not captured: a captured table lives in local memory)
+      double z[NZ], yb[NX], cqd[NZ], mjx[NX][M::MAXRX], mju[NX][M::MAXRU], hd[NHD];
+      double vz[NZ];
       load_node<M>(a, j, z);
       if (NEEDH) {
         load_ybar<M>(a, K, a.y, j, yb);
@@ -451,34 +528,33 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
         double mdp[NX];
         jv_node<M, false>(K, mjx, mju, mdp, 0.0, vz, jA[q], jB[q]);
       }
-    }
-    // ---- Jacobian rows staged in shared memory: left part of row lt, right part of row lt-1
-    if (WJ && act) {
+      // ---- Jacobian rows staged in shared memory: left part of row lt, right part of row lt-1
+      if (WJ) {
 #pragma unroll
-      for (int k = 0; k < NX; ++k) {
-        const int cnt = row_count<M>(k);
-        double* sj = sm + jrow_off<M>(k) * R;
-        if (lt < nrows) {
-          double* rp = sj + lt * cnt;
+        for (int k = 0; k < NX; ++k) {
+          const int cnt = row_count<M>(k);
+          double* sj = sm + jrow_off<M>(k) * R;
+          if (lt < nrows) {
+            double* rp = sj + lt * cnt;
 #pragma unroll
-          for (int e = 0; e < M::MAXRX; ++e)
-            if (e < M::RX(k)) rp[e] = (M::XV(k, e) == k) ? (M::JZ(k, e) ? -1.0 : fma(mjx[k][e], K.one, -1.0)) : mjx[k][e];
+            for (int e = 0; e < M::MAXRX; ++e)
+              if (e < M::RX(k)) rp[e] = (M::XV(k, e) == k) ? (M::JZ(k, e) ? -1.0 : fma(mjx[k][e], K.one, -1.0)) : mjx[k][e];
 #pragma unroll
-          for (int e = 0; e < M::MAXRU; ++e)
-            if (e < M::RU(k)) rp[2 * M::RX(k) + e] = mju[k][e];
-        }
-        if (lt >= 1 && lt - 1 < nrows) {
-          double* rp = sj + (lt - 1) * cnt;
+            for (int e = 0; e < M::MAXRU; ++e)
+              if (e < M::RU(k)) rp[2 * M::RX(k) + e] = mju[k][e];
+          }
+          if (lt >= 1 && lt - 1 < nrows) {
+            double* rp = sj + (lt - 1) * cnt;
 #pragma unroll
-          for (int e = 0; e < M::MAXRX; ++e)
-            if (e < M::RX(k)) rp[M::RX(k) + e] = (M::XV(k, e) == k) ? (M::JZ(k, e) ? 1.0 : fma(mjx[k][e], K.one, 1.0)) : mjx[k][e];
+            for (int e = 0; e < M::MAXRX; ++e)
+              if (e < M::RX(k)) rp[M::RX(k) + e] = (M::XV(k, e) == k) ? (M::JZ(k, e) ? 1.0 : fma(mjx[k][e], K.one, 1.0)) : mjx[k][e];
 #pragma unroll
-          for (int e = 0; e < M::MAXRU; ++e)
-            if (e < M::RU(k)) rp[2 * M::RX(k) + M::RU(k) + e] = mju[k][e];
+            for (int e = 0; e < M::MAXRU; ++e)
+              if (e < M::RU(k)) rp[2 * M::RX(k) + M::RU(k) + e] = mju[k][e];
+          }
         }
       }
-    }
-    if (own) {
+      if (!own) return;
       if (WJTV) {
         double wb[NX], wl[NX], wr[NX], o[NZ];
         load_bar<M>(a, K, a.wv, j, wb, wl, wr);
@@ -500,8 +576,6 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
           for (int k = 0; k < NX; ++k) a.ojv[NX + k] = vz[k];
         }
       }
-    }
-    if (own) {
       // ---- Hessian block of node j (stored directly; X block then U block)
       if (sH) {
 #pragma unroll
@@ -519,7 +593,7 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
         double s2;
         if (a.has_ref) s2 = sG ? node_grad<M, true, true>(a, K, z, endp, j) : node_grad<M, true, false>(a, K, z, endp, j);
         else s2 = sG ? node_grad<M, false, true>(a, K, z, endp, j) : node_grad<M, false, false>(a, K, z, endp, j);
-        objterm = (q == 0) ? s2 : fadd(K, objterm, s2);
+        objterm = (NPT == 1 || q == 0) ? s2 : fadd(K, objterm, s2);
       }
       // ---- boundary rows X_{0,k} (and X_{N,k}): constraint value and the constant Jacobian entry
       if (j == 0) {
@@ -536,8 +610,9 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
           if (sJ) a.jv[NX + k] = 1.0;
         }
       }
-    }
+    });
   }
+  const ModelConst& K = K0;
   // ---- defects (and Jv rows): the right node's share is this thread's next node, or lane+1's first
   double nbv[NX], nbA[NX];
   if (WC) {
@@ -627,35 +702,21 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
   if (WC || WJ || WF || WJV) __syncthreads();
 }
 
-// The fused evaluation kernel.  A model may ask for a minimum of resident CTAs per SM
-// (M::EVAL_MIN_CTAS > 0, a register cap for models whose fused kernels would otherwise need
-// all 255 registers); by default the register allocator's own heuristic applies.
-template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
+// The fused evaluation kernel.
+template <class M, int TILE, int NPT, unsigned OUT, bool PAR, bool IP>
 __device__ __forceinline__ void node_eval_kernel_body(const NodeArgs<M>& a) {
   constexpr bool WF = OUT & O_F;
   extern __shared__ __align__(16) double sm[];
   __shared__ double sEdge[2 * (TILE / 32 + 1) * M::NX];
   const ModelConst K = launch_consts<M, PAR>(a);
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x)
-    node_eval_tile<M, TILE, NPT, OUT>(a, K, tile, sm, sEdge, a.partials + tile);
+    node_eval_tile<M, TILE, NPT, OUT, IP>(a, K, tile, sm, sEdge, a.partials + tile);
   if (WF && a.f) finish_tiles<TILE>(a.partials, a.ntiles, a.counter, a.f, 0.5, sm);
 }
 
-template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
-__global__ void __launch_bounds__(TILE) k_node_eval(const __grid_constant__ NodeArgs<M> a) {
-  node_eval_kernel_body<M, TILE, NPT, OUT, PAR>(a);
-}
-
-template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
-__global__ void __launch_bounds__(TILE, (M::EVAL_MIN_CTAS > 0 ? M::EVAL_MIN_CTAS : 1))
-    k_node_eval_capped(const __grid_constant__ NodeArgs<M> a) {
-  node_eval_kernel_body<M, TILE, NPT, OUT, PAR>(a);
-}
-
-template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
-auto eval_kernel() {
-  if constexpr (M::EVAL_MIN_CTAS > 0) return k_node_eval_capped<M, TILE, NPT, OUT, PAR>;
-  else return k_node_eval<M, TILE, NPT, OUT, PAR>;
+template <class M, int TILE, int NPT, unsigned OUT, bool PAR, bool IP>
+__global__ void __launch_bounds__(TILE, min_ctas<M, OUT, IP>()) k_node_eval(const __grid_constant__ NodeArgs<M> a) {
+  node_eval_kernel_body<M, TILE, NPT, OUT, PAR, IP>(a);
 }
 
 // ======================================================================================
@@ -663,13 +724,14 @@ auto eval_kernel() {
 // p_k(j) = -hh grad f_k(z_j) . v_{z_j}  (+ -hh df_k/dmu(z_j) * pdir for the parameter).
 // Same overlapping tiles as the evaluation; the right-node term comes from lane+1.
 // ======================================================================================
-template <class M, int TILE, bool PDIR, bool PAR>
-__global__ void __launch_bounds__(TILE) k_node_jprod(const __grid_constant__ NodeArgs<M> a) {
+template <class M, int TILE, bool PDIR, bool PAR, bool IP>
+__global__ void __launch_bounds__(TILE, min_ctas<M, O_JV, IP>()) k_node_jprod(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
+  constexpr unsigned SOFT = soft_kernel<M, O_JV, IP>();
   __shared__ double sEdge[(TILE / 32 + 1) * NX];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  ModelConst K = launch_consts<M, PAR>(a);
+  const ModelConst K0 = launch_consts<M, PAR>(a);
   double pd = 0.0;
   if (PDIR) pd = a.pdir_dev ? __ldg(a.pdir_dev) : a.pdir;
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
@@ -682,7 +744,11 @@ __global__ void __launch_bounds__(TILE) k_node_jprod(const __grid_constant__ Nod
     double p[NX], vx[NX], A[NX];
 #pragma unroll
     for (int k = 0; k < NX; ++k) { p[k] = 0.0; vx[k] = 0.0; A[k] = 0.0; }
-    if (act) {
+    bool ok = false;
+    if constexpr (SOFT != 0) {
+      if (K0.soft && act) ok = soft_node<M, false, true, false>(a, nullptr, a.v, nullptr, j);
+    }
+    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
       double z[NZ], vz[NZ], yb[NX], cqd[NZ], pa[NX], pb[NX], mjx[NX][M::MAXRX], mju[NX][M::MAXRU], hd[NHD];
       load_node<M>(a, j, z);
       load_vz<M>(a, a.v, j, vz);
@@ -692,6 +758,8 @@ __global__ void __launch_bounds__(TILE) k_node_jprod(const __grid_constant__ Nod
       double mdp[NX];
       if (PDIR) M::dparam(K, z, mdp);
       jv_node<M, PDIR>(K, mjx, mju, mdp, pd, vz, A, p);
+    });
+    if (act) {
       if (j == 0) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) a.out[k] = vx[k];
@@ -712,7 +780,7 @@ __global__ void __launch_bounds__(TILE) k_node_jprod(const __grid_constant__ Nod
 #pragma unroll
       for (int k = 0; k < NX; ++k) {
         const double right = (lane == 31) ? sEdge[(warp + 1) * NX + k] : nbv[k];
-        a.out[a.nb + (int64_t)k * a.N + j] = fadd(K, p[k], right);
+        a.out[a.nb + (int64_t)k * a.N + j] = fadd(K0, p[k], right);
       }
     }
     __syncthreads();
@@ -725,13 +793,14 @@ __global__ void __launch_bounds__(TILE) k_node_jprod(const __grid_constant__ Nod
 // With DPAR, also (dc/dp_i)^T w = sum_j sum_k wbar_k mdp_k,i(z_j) for every dynamics
 // parameter i < M::NP (mdp = -hh df/dp; one deterministic reduction per parameter).
 // ======================================================================================
-template <class M, int TILE, bool DPAR, bool PAR>
-__global__ void __launch_bounds__(TILE) k_node_jtprod(const __grid_constant__ NodeArgs<M> a) {
+template <class M, int TILE, bool DPAR, bool PAR, bool IP>
+__global__ void __launch_bounds__(TILE, min_ctas<M, O_JTV, IP>()) k_node_jtprod(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   constexpr int NP = M::NP, NPA = (NP > 0) ? NP : 1;
+  constexpr unsigned SOFT = soft_kernel<M, O_JTV, IP>();
   __shared__ double red[TILE * NPA];
-  ModelConst K = launch_consts<M, PAR>(a);
+  const ModelConst K0 = launch_consts<M, PAR>(a);
   const int64_t nchunks = (a.E - a.B + TILE - 1) / TILE;   // the nodes [B, E) in chunks of TILE
   for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
     const int64_t j0 = a.B + chunk * TILE, j = j0 + threadIdx.x;
@@ -739,7 +808,12 @@ __global__ void __launch_bounds__(TILE) k_node_jtprod(const __grid_constant__ No
     double acc[NPA];
 #pragma unroll
     for (int i = 0; i < NPA; ++i) acc[i] = 0.0;
-    if (j < a.E) {
+    const bool act = j < a.E;
+    bool ok = false;
+    if constexpr (SOFT != 0) {
+      if (K0.soft && act) ok = soft_node<M, false, false, true>(a, nullptr, nullptr, a.v, j);
+    }
+    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
       double z[NZ], yb[NX], cqd[NZ], pa[NX], pb[NX], mjx[NX][M::MAXRX], mju[NX][M::MAXRU], hd[NHD];
       double wb[NX], wl[NX], wr[NX];
       load_node<M>(a, j, z);
@@ -756,15 +830,17 @@ __global__ void __launch_bounds__(TILE) k_node_jtprod(const __grid_constant__ No
       store_nz<M>(a, a.out, j, o);
       if (DPAR && NP > 0) {
 #pragma unroll
-        for (int i = 0; i < NPA; ++i)
+        for (int i = 0; i < NPA; ++i) {
+          acc[i] = 0.0;
 #pragma unroll
           for (int k = 0; k < NX; ++k)
             if (M::DP(k, i)) acc[i] = fma(wb[k], mdp[k][i], acc[i]);
+        }
       }
-    }
+    });
     if (DPAR) {
       double ts[NPA];
-      tile_sum_n<TILE, NPA>(acc, red, K.one, ts);
+      tile_sum_n<TILE, NPA>(acc, red, K0.one, ts);
       if (threadIdx.x == 0) {
 #pragma unroll
         for (int i = 0; i < NPA; ++i) a.partials[i * nchunks + chunk] = ts[i];
@@ -780,29 +856,31 @@ __global__ void __launch_bounds__(TILE) k_node_jtprod(const __grid_constant__ No
 // With MIX (autograd double backward), also adds mixs * m_j, m_j = sum_k mixwbar_k
 // (-hh d2 f_k / dmu dz)(z_j), and reduces sum_j m_j . v_{z_j} into *dmu.
 // ======================================================================================
-template <class M, int TILE, bool MIX, bool PAR>
-__global__ void __launch_bounds__(TILE) k_node_hprod(const __grid_constant__ NodeArgs<M> a) {
+template <class M, int TILE, bool MIX, bool PAR, bool IP>
+__global__ void __launch_bounds__(TILE, min_ctas<M, O_HV, IP>()) k_node_hprod(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
-  constexpr HTmpl<M> HT{};
+  constexpr unsigned SOFT = soft_kernel<M, O_HV, IP && !MIX>();
   __shared__ double red[TILE];
-  ModelConst K = launch_consts<M, PAR>(a);
+  const ModelConst K0 = launch_consts<M, PAR>(a);
   double ms = 0.0;
   if (MIX) ms = a.mixs ? __ldg(a.mixs) : 0.0;
   const int64_t nchunks = (a.N + TILE) / TILE;
   for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
     const int64_t j = chunk * TILE + threadIdx.x;
     double acc_mu = 0.0;
-    if (j <= a.N) {
+    const bool act = j <= a.N;
+    bool ok = false;
+    if constexpr (SOFT != 0) {
+      if (K0.soft && act) ok = soft_node<M, true, true, false>(a, a.y, a.v, nullptr, j);
+    }
+    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
       double z[NZ], vz[NZ], yb[NX], cqd[NZ], pa[NX], pb[NX], mjx[NX][M::MAXRX], mju[NX][M::MAXRU], hd[NHD];
       load_node<M>(a, j, z);
       load_ybar<M>(a, K, a.y, j, yb);
       const bool endp = (j == 0) || (j == a.N);
       node_cq<M>(a, endp, cqd);
-#pragma unroll
-      for (int k = 0; k < NX; ++k) vz[k] = __ldg(a.v + NX * j + k);
-#pragma unroll
-      for (int i = 0; i < M::NU; ++i) vz[NX + i] = __ldg(a.v + a.uoff + M::NU * j + i);
+      load_vz<M>(a, a.v, j, vz);
       M::template eval<false, false, true>(K, z, yb, cqd, pa, pb, mjx, mju, hd);
       double o[NZ];
       hv_node<M>(a, K, hd, cqd, vz, o);
@@ -810,6 +888,7 @@ __global__ void __launch_bounds__(TILE) k_node_hprod(const __grid_constant__ Nod
         double mb[NX], mg[NZ], wl[NX], wr[NX];
         load_bar<M>(a, K, a.mixw, j, mb, wl, wr);
         M::dparam_grad(K, z, mb, mg);
+        acc_mu = 0.0;
 #pragma unroll
         for (int v = 0; v < NZ; ++v) {
           o[v] = fma(mg[v], ms, o[v]);
@@ -817,9 +896,9 @@ __global__ void __launch_bounds__(TILE) k_node_hprod(const __grid_constant__ Nod
         }
       }
       store_nz<M>(a, a.out, j, o);
-    }
+    });
     if (MIX && a.dmu) {
-      const double ts = tile_sum<TILE>(acc_mu, red, K.one);
+      const double ts = tile_sum<TILE>(acc_mu, red, K0.one);
       if (threadIdx.x == 0) a.partials[chunk] = ts;
       __syncthreads();
     }
@@ -840,6 +919,8 @@ void fill_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   a.has_final = h->has_final ? 1 : 0;
   a.has_ref = h->has_ref ? 1 : 0;
   M::host_consts(h->params.data(), h->hh, a.K);
+  a.K.many = soft_launch(h->N + 1, h->num_sms);
+  a.K.soft = a.K.many && soft_consts(a.K, M::NC);
   for (int v = 0; v < M::NZ; ++v) {
     const double w = v < M::NX ? h->q[v] : h->r[v - M::NX];
     a.gq_in[v] = 2.0 * h->h * w;
@@ -862,10 +943,13 @@ void fill_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   for (int i = 0; i < h->ntrk; ++i) a.trk[h->trk_comp[i]] = (int8_t)i;
 }
 
-template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
-ocp_status launch_eval_k(ocp* h, const EvalCall& c, cudaStream_t s) {
-  NodeArgs<M> a;
-  fill_args<M>(h, c.sigma, a);
+// Whether the launch takes the integer-product instance of its kernel (the device reads the parameters
+// itself with PAR, and tests the constants made of them there).
+template <class M, unsigned OUT, bool PAR>
+bool soft_choice(const NodeArgs<M>& a) { return M::template SOFT<OUT> != 0 && (PAR ? a.K.many : a.K.soft); }
+
+template <class M, int TILE, int NPT, unsigned OUT, bool PAR, bool IP>
+ocp_status launch_eval_ip(ocp* h, const EvalCall& c, NodeArgs<M>& a, cudaStream_t s) {
   a.x = c.x; a.y = c.y; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
   a.v = c.vn; a.wv = c.vm; a.ojv = c.ojv; a.ojtv = c.ojtv; a.ohv = c.ohv;
   a.B = c.B; a.E = c.E;
@@ -876,7 +960,7 @@ ocp_status launch_eval_k(ocp* h, const EvalCall& c, cudaStream_t s) {
   if (a.ntiles < 1) a.ntiles = 1;
   if (a.ntiles > h->max_partials) return set_err(h, OCP_EDIM, "too many tiles for the reduction scratch");
   using S = EvalSmem<M, TILE, NPT, OUT>;
-  auto kern = eval_kernel<M, TILE, NPT, OUT, PAR>();
+  auto kern = k_node_eval<M, TILE, NPT, OUT, PAR, IP>;
   static unsigned attr_done = 0;
   if (!(attr_done & (1u << (h->device & 31)))) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::bytes);
@@ -886,6 +970,16 @@ ocp_status launch_eval_k(ocp* h, const EvalCall& c, cudaStream_t s) {
   const int grid = occupancy_grid(h, (const void*)kern, TILE, S::bytes, a.ntiles);
   kern<<<grid, TILE, S::bytes, s>>>(a);
   return cuda_err(h, cudaGetLastError(), "k_node_eval launch");
+}
+
+template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
+ocp_status launch_eval_k(ocp* h, const EvalCall& c, cudaStream_t s) {
+  NodeArgs<M> a;
+  fill_args<M>(h, c.sigma, a);
+  if constexpr (M::template SOFT<OUT> != 0) {
+    if (soft_choice<M, OUT, PAR>(a)) return launch_eval_ip<M, TILE, NPT, OUT, PAR, true>(h, c, a, s);
+  }
+  return launch_eval_ip<M, TILE, NPT, OUT, PAR, false>(h, c, a, s);
 }
 
 template <class M, int TILE, int NPT, unsigned OUT>
@@ -924,20 +1018,20 @@ __host__ __device__ constexpr int euler_off(int k) {
   return s;
 }
 
-template <class M, int TILE, unsigned OUT, bool PAR>
-__global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs<M> a) {
+template <class M, int TILE, unsigned OUT, bool PAR, bool IP>
+__global__ void __launch_bounds__(TILE, min_ctas<M, OUT, IP, true>()) k_euler(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr bool WF = OUT & O_F, WC = OUT & O_C, WG = OUT & O_G, WJ = OUT & O_J, WH = OUT & O_H;
   constexpr bool WJV = OUT & O_JV, WJTV = OUT & O_JTV, WHV = OUT & O_HV;
   constexpr bool NEEDJ = WJ || WJV || WJTV, NEEDH = WH || WHV;
-  constexpr HTmpl<M> HT{};
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   extern __shared__ __align__(16) double sm[];   // staged rows: component k at euler_off(k) * TILE
   __shared__ double red[TILE];
   const bool sF = WF && a.f, sC = WC && a.c, sG = WG && a.g, sJ = WJ && a.jv, sH = WH && a.hv;
   const bool doH = sH || WHV;
+  constexpr unsigned SOFT = soft_kernel<M, OUT, IP>();
   const int t = threadIdx.x;
-  ModelConst K = launch_consts<M, PAR>(a);
+  const ModelConst K0 = launch_consts<M, PAR>(a);
   const int64_t N = a.N;
   const int64_t xN = (int64_t)NX * N;  // first entry of X_N
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
@@ -945,7 +1039,13 @@ __global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs
     const int64_t j = r0 + t;
     const int nrows = (int)min((int64_t)TILE, max(N - r0, (int64_t)0));
     double objterm = 0.0;
-    if (j < N) {
+    const bool act = j < N;
+    bool ok = false;
+    if constexpr (SOFT != 0) {
+      if (K0.soft && act) ok = soft_euler<M, NEEDH, (WJV || WHV), WJTV>(a, a.y, a.v, a.wv, j);
+    }
+    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
+      constexpr HTmpl<M> HT{};
       double z[NZ], yb[NX], cqd[NZ], pa[NX], pb[NX], mjx[NX][M::MAXRX], mju[NX][M::MAXRU], hd[NHD];
       load_node<M>(a, j, z);
       if (NEEDH) {  // own rows' multipliers y_{k,j} (not the sum of two rows)
@@ -1022,7 +1122,8 @@ __global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs
           if (sJ) a.jv[k] = 1.0;
         }
       }
-    } else if (r0 + TILE > N && j == N) {  // the last node: states only (CTA-uniform test first)
+    });
+    if (r0 + TILE > N && j == N) {  // the last node: states only (CTA-uniform test first)
       if (sG) {
 #pragma unroll
         for (int k = 0; k < NX; ++k) a.g[xN + k] = 0.0;
@@ -1039,7 +1140,7 @@ __global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs
 #pragma unroll
         for (int k = 0; k < NX; ++k) {
           double o = __ldg(a.wv + a.nb + (int64_t)k * N + N - 1);
-          if (a.has_final) o = fadd(K, o, __ldg(a.wv + NX + k));
+          if (a.has_final) o = fadd(K0, o, __ldg(a.wv + NX + k));
           a.ojtv[xN + k] = o;
         }
       }
@@ -1076,7 +1177,7 @@ __global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs
       }
     }
     if (sF) {
-      const double ts = tile_sum<TILE>(objterm, red, K.one);
+      const double ts = tile_sum<TILE>(objterm, red, K0.one);
       if (t == 0) a.partials[tile] = ts;
     }
     __syncthreads();
@@ -1084,18 +1185,26 @@ __global__ void __launch_bounds__(TILE) k_euler(const __grid_constant__ NodeArgs
   if (sF) finish_tiles<TILE>(a.partials, a.ntiles, a.counter, a.f, 0.5, red);
 }
 
-template <class M, int TILE, unsigned OUT, bool PAR>
-ocp_status launch_euler_k(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
+template <class M, int TILE, unsigned OUT, bool PAR, bool IP>
+ocp_status launch_euler_ip(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
   a.ntiles = (h->N + 1 + TILE - 1) / TILE;
   if (a.ntiles > h->max_partials) return set_err(h, OCP_EDIM, "too many tiles for the reduction scratch");
   const size_t smem = (OUT & O_J) ? sizeof(double) * (size_t)euler_total<M>() * TILE : 0;
-  auto kern = k_euler<M, TILE, OUT, PAR>;
+  auto kern = k_euler<M, TILE, OUT, PAR, IP>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_err(h, e, "cudaFuncSetAttribute(euler)");
   }
   kern<<<(int)a.ntiles, TILE, smem, s>>>(a);
   return cuda_err(h, cudaGetLastError(), "k_euler launch");
+}
+
+template <class M, int TILE, unsigned OUT, bool PAR>
+ocp_status launch_euler_k(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
+  if constexpr (M::template SOFT<OUT> != 0) {
+    if (soft_choice<M, OUT, PAR>(a)) return launch_euler_ip<M, TILE, OUT, PAR, true>(h, a, s);
+  }
+  return launch_euler_ip<M, TILE, OUT, PAR, false>(h, a, s);
 }
 
 template <class M, int TILE, unsigned OUT>
@@ -1112,6 +1221,7 @@ template <class M>
 void fill_euler_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   fill_args<M>(h, sigma, a);
   M::host_consts(h->params.data(), h->h, a.K);   // the scheme's step is h (not h/2)
+  a.K.soft = soft_consts(a.K, M::NC);
   a.B = 0;
   a.E = h->N + 1;
 }
@@ -1169,8 +1279,8 @@ ocp_status node_eval_dispatch(ocp* h, unsigned out, const EvalCall& c, cudaStrea
   }
 }
 
-template <class M, int TILE, bool PAR>
-cudaError_t node_prod_launch(ocp* h, const ProdCall& c, const NodeArgs<M>& a, cudaStream_t s) {
+template <class M, int TILE, bool PAR, bool IP>
+cudaError_t node_prod_launch_ip(ocp* h, const ProdCall& c, const NodeArgs<M>& a, cudaStream_t s) {
   auto go = [&](auto kern, int64_t units) {
     const int grid = occupancy_grid(h, (const void*)kern, TILE, 0, units);
     kern<<<grid, TILE, 0, s>>>(a);
@@ -1179,18 +1289,28 @@ cudaError_t node_prod_launch(ocp* h, const ProdCall& c, const NodeArgs<M>& a, cu
   // model alone (the C-ABI rejects them for the others)
   constexpr bool VDP = M::HAS_DPARAM;
   if (c.kind == P_JPROD) {
-    if (VDP && (c.pdir != 0.0 || c.pdir_dev)) go(k_node_jprod<M, TILE, VDP, PAR>, a.ntiles);
-    else go(k_node_jprod<M, TILE, false, PAR>, a.ntiles);
+    if (VDP && (c.pdir != 0.0 || c.pdir_dev)) go(k_node_jprod<M, TILE, VDP, PAR, IP>, a.ntiles);
+    else go(k_node_jprod<M, TILE, false, PAR, IP>, a.ntiles);
   } else if (c.kind == P_JTPROD) {
     const int64_t blocks = (a.E - a.B + TILE - 1) / TILE;
-    if (c.dmu) go(k_node_jtprod<M, TILE, true, PAR>, blocks);
-    else go(k_node_jtprod<M, TILE, false, PAR>, blocks);
+    if (c.dmu) go(k_node_jtprod<M, TILE, true, PAR, IP>, blocks);
+    else go(k_node_jtprod<M, TILE, false, PAR, IP>, blocks);
   } else {
     const int64_t blocks = (h->N + 1 + TILE - 1) / TILE;
-    if (VDP && c.mixw && c.mixs) go(k_node_hprod<M, TILE, VDP, PAR>, blocks);
-    else go(k_node_hprod<M, TILE, false, PAR>, blocks);
+    if (VDP && c.mixw && c.mixs) go(k_node_hprod<M, TILE, VDP, PAR, false>, blocks);
+    else go(k_node_hprod<M, TILE, false, PAR, IP>, blocks);
   }
   return cudaGetLastError();
+}
+
+template <class M, int TILE, bool PAR>
+cudaError_t node_prod_launch(ocp* h, const ProdCall& c, const NodeArgs<M>& a, cudaStream_t s) {
+  static_assert((M::template SOFT<O_JV> != 0) == (M::template SOFT<O_JTV> != 0) &&
+                (M::template SOFT<O_JV> != 0) == (M::template SOFT<O_HV> != 0), "the products choose alike");
+  if constexpr (M::template SOFT<O_JV> != 0) {
+    if (soft_choice<M, O_JV, PAR>(a)) return node_prod_launch_ip<M, TILE, PAR, true>(h, c, a, s);
+  }
+  return node_prod_launch_ip<M, TILE, PAR, false>(h, c, a, s);
 }
 
 template <class M, int TILE>

@@ -18,19 +18,21 @@ namespace ocpg {
 // where sin a, cos a come from kSinCosTable (the doubles nearest the exact values), sin r =
 // r - r^3/6 + r^5/120 and cos r - 1 = -r^2/2 + r^4/24 (the omitted terms are below 2e-19 of the
 // result on |r| <= pi/1024); the quadrant then swaps and negates (sign bits only) and sin takes
-// the sign of x (sin is odd, cos even), which keeps sin(-0) = -0.  15 FP64 instructions, against
+// the sign of x (sin is odd, cos even), which keeps sin(-0) = -0.  14 FP64 instructions (three of
+// them products, on the integer pipes where the work runs with those), against
 // 24 for sincos_red's Taylor polynomials on |r| <= pi/4; within two ulps of the correctly
 // rounded values (ocp_probe_sincos_table).  A warp whose active lanes are not all finite with
 // |x| <= 1e5 takes the library routine (a uniform branch).
-__device__ __forceinline__ void sincos_tab(const ModelConst& K, double x, double& s, double& c) {
+template <class KC>
+__device__ __forceinline__ void sincos_tab(const KC& K, double x, double& s, double& c) {
   if (__all_sync(__activemask(), fabs(x) <= 1.0e5)) {
     const double ax = fabs(x);
     const double t = fma(ax, 0x1.45f306dc9c883p+7, 0x1.8p52);   // 512/pi
-    const double k = fsub(K, t, 0x1.8p52);
+    const int ki = __double2loint(t);                            // k < 2^24
+    const double k = small_int(ki);
     double r = fma(-k, 0x1.921fb54442d18p-8, ax);                // P1
     r = fma(-k, 0x1.1a62633145c07p-62, r);                       // P2
     r = fma(-k, -0x1.f1976b7ed8fbcp-118, r);                     // P3
-    const int ki = __double2loint(t);                            // k mod 2^32
     const double2 sc = __ldg(&kSinCosTable[ki & 255]);           // sin a, cos a
     const double z = fmul(K, r, r);
     const double sr = fma(fmul(K, r, z), fma(z, 0x1.1111111111111p-7, -0x1.5555555555555p-3), r);  // 1/5!, -1/3!
