@@ -209,18 +209,27 @@ __device__ __forceinline__ void load_node(const NodeArgs<M>& a, int64_t j, doubl
 }
 
 // The model constants of a launch.  With PAR (device-resident parameters: params[0] bound by
-// ocp_bind_param0, or the model's whole parameter vector for one call) the
-// parameter-dependent constants are recomputed from them.  PAR is a
-// template argument rather than a run-time test: a branch this short is if-converted, and
-// its predicated-off FP64 instructions would still take FP64 pipe slots in every warp.
+// ocp_bind_param0, or the model's whole parameter vector for one call) the parameter-dependent
+// constants are recomputed from them, by one thread for the CTA: the cart-pole's take a division and
+// some fourteen products, a quarter of the FP64 work of a node when every thread forms them (J^T w
+// with the parameter derivatives at N = 1e6: 197 us so, 178 now).  PAR is a template argument
+// rather than a run-time test: a branch this short is if-converted, and its predicated-off FP64
+// instructions would still take FP64 pipe slots in every warp.
 template <class M, bool PAR>
 __device__ __forceinline__ ModelConst launch_consts(const NodeArgs<M>& a) {
-  ModelConst K = a.K;
   if constexpr (PAR) {
-    M::device_params(K, a.p0_dev);
-    K.soft = K.many && soft_consts(K, M::NC);
+    __shared__ ModelConst s_k;
+    if (threadIdx.x == 0) {
+      ModelConst K = a.K;
+      M::device_params(K, a.p0_dev);
+      K.soft = K.many && soft_consts(K, M::NC);
+      s_k = K;
+    }
+    __syncthreads();
+    return s_k;
+  } else {
+    return a.K;
   }
-  return K;
 }
 
 // ybar_k = w_{k,j-1} + w_{k,j} over the defect rows of component k (zero outside 0..N-1)
