@@ -37,9 +37,56 @@ __device__ __forceinline__ int64_t var_index(const ObjArgs& a, int64_t j, int v)
   return v < a.nx ? (int64_t)a.nx * j + v : a.uoff + (int64_t)a.nu * j + (v - a.nx);
 }
 
-// HVP = false: out = s * grad F.   HVP = true: out = s * Hess F v, dot = grad F . v
-template <bool HVP>
-__global__ void __launch_bounds__(OBJ_THREADS) k_obj(const __grid_constant__ ObjArgs a) {
+// out = s * grad F: elementwise over the X entries (regions of 2048, blocks [0, xblocks)) and the U
+// entries.  Bound by HBM: 16 bytes and one or two FP64 operations per entry, with the factors
+// s 2 w_j q_v (interior and end nodes) formed once per block.  (One thread per node looping over its
+// variables, each forming the factor again: 33.2 us for the 5e6 entries of the cart-pole at N = 1e6, 15.3 now.)
+constexpr int OBJ_PER = 8, OBJ_CHUNK = OBJ_THREADS * OBJ_PER;
+
+__global__ void __launch_bounds__(OBJ_THREADS) k_obj_grad(const __grid_constant__ ObjArgs a, int64_t xblocks) {
+  __shared__ double s_in[OBJ_MAXV], s_end[OBJ_MAXV];
+  const double s = __ldg(a.s);
+  for (int v = threadIdx.x; v < a.nx + a.nu; v += OBJ_THREADS) {
+    s_in[v] = fma(s, a.gq_in[v], a.mz);
+    s_end[v] = fma(s, a.gq_end[v], a.mz);
+  }
+  __syncthreads();
+  const bool xs = blockIdx.x < xblocks;
+  const int w = xs ? a.nx : a.nu, v0 = xs ? 0 : a.nx;       // entries per node, first local variable
+  const int64_t e0 = (xs ? (int64_t)blockIdx.x : (int64_t)blockIdx.x - xblocks) * OBJ_CHUNK;
+  const int64_t len = (int64_t)w * (a.N + 1);
+  const int n = (int)min((int64_t)OBJ_CHUNK, len - e0);
+  const int64_t j0 = e0 / w;
+  const int o0 = (int)(e0 - j0 * w);
+  const float inv = 1.0f / (float)w;
+  const double* __restrict__ x = a.x + (xs ? 0 : a.uoff) + e0;
+  double* __restrict__ out = a.out + (xs ? 0 : a.uoff) + e0;
+  double z[OBJ_PER];
+#pragma unroll
+  for (int q = 0; q < OBJ_PER; ++q) {
+    const int i = threadIdx.x + q * OBJ_THREADS;
+    z[q] = i < n ? __ldg(x + i) : 0.0;
+  }
+#pragma unroll
+  for (int q = 0; q < OBJ_PER; ++q) {
+    const int i = threadIdx.x + q * OBJ_THREADS;
+    if (i >= n) continue;
+    // floor((o0 + i) / w): at least 1 / (2 w) from an integer, off by less than 2^-10 / w (as kkt_div)
+    const int u = o0 + i, jl = (int)__fmul_rz((float)u + 0.5f, inv);
+    const int v = v0 + (u - jl * w);
+    const int64_t j = j0 + jl;
+    double d = z[q];
+    if (a.has_ref) {
+      double rv = a.ref[v];
+      if (v < a.nx && a.xtrack && a.trk[v] >= 0) rv = __ldg(a.xtrack + (int64_t)a.ntrk * j + a.trk[v]);
+      d = fma(-rv, a.one, z[q]);
+    }
+    out[i] = fma((j == 0 || j == a.N) ? s_end[v] : s_in[v], d, a.mz);
+  }
+}
+
+// out = s * Hess F v, dot = grad F . v
+__global__ void __launch_bounds__(OBJ_THREADS) k_obj_hvp(const __grid_constant__ ObjArgs a) {
   __shared__ double red[OBJ_THREADS];
   const double s = __ldg(a.s);
   const int nz = a.nx + a.nu;
@@ -57,22 +104,18 @@ __global__ void __launch_bounds__(OBJ_THREADS) k_obj(const __grid_constant__ Obj
         if (v < a.nx && a.xtrack && a.trk[v] >= 0) rv = __ldg(a.xtrack + (int64_t)a.ntrk * j + a.trk[v]);
         const double d = a.has_ref ? fma(-rv, a.one, z) : z;
         const double sg = fma(s, gq, a.mz);
-        if (HVP) {
-          const double vv = __ldg(a.v + idx);
-          a.out[idx] = fma(sg, vv, a.mz);
-          acc = fma(fma(gq, d, a.mz), vv, acc);
-        } else {
-          a.out[idx] = fma(sg, d, a.mz);
-        }
+        const double vv = __ldg(a.v + idx);
+        a.out[idx] = fma(sg, vv, a.mz);
+        acc = fma(fma(gq, d, a.mz), vv, acc);
       }
     }
-    if (HVP && a.dot) {
+    if (a.dot) {
       const double ts = tile_sum<OBJ_THREADS>(acc, red, a.one);
       if (threadIdx.x == 0) a.partials[chunk] = ts;
       __syncthreads();
     }
   }
-  if (HVP && a.dot) finish_tiles<OBJ_THREADS>(a.partials, nchunks, a.counter, a.dot, 1.0, red);
+  if (a.dot) finish_tiles<OBJ_THREADS>(a.partials, nchunks, a.counter, a.dot, 1.0, red);
 }
 
 ocp_status obj_launch(ocp* h, bool hvp, const double* x, const double* s, const double* v, double* out,
@@ -101,10 +144,14 @@ ocp_status obj_launch(ocp* h, bool hvp, const double* x, const double* s, const 
     a.gq_end[v2] = h->h * w;
     a.ref[v2] = v2 < h->nx ? h->xref[v2] : h->uref[v2 - h->nx];
   }
-  const int64_t nchunks = (h->N + OBJ_THREADS) / OBJ_THREADS;
-  const int grid = occupancy_grid(h, nullptr, OBJ_THREADS, 0, nchunks);
-  if (hvp) k_obj<true><<<grid, OBJ_THREADS, 0, st>>>(a);
-  else k_obj<false><<<grid, OBJ_THREADS, 0, st>>>(a);
+  if (hvp) {
+    const int64_t nchunks = (h->N + OBJ_THREADS) / OBJ_THREADS;
+    k_obj_hvp<<<occupancy_grid(h, nullptr, OBJ_THREADS, 0, nchunks), OBJ_THREADS, 0, st>>>(a);
+  } else {
+    auto blocks = [&](int w) { return ((int64_t)w * (h->N + 1) + OBJ_CHUNK - 1) / OBJ_CHUNK; };
+    const int64_t xb = blocks(h->nx);
+    k_obj_grad<<<(int)(xb + blocks(h->nu)), OBJ_THREADS, 0, st>>>(a, xb);
+  }
   return cuda_err(h, cudaGetLastError(), "objective kernel launch");
 }
 
