@@ -557,7 +557,7 @@ ocp_status ocp_eval_step(ocp_t* h, const double* x, const double* y, double sigm
     b.kind = P_JTPROD; b.x = x; b.v = vm; b.out = Jtv;
     c.kind = P_HPROD; c.x = x; c.y = y; c.sigma = sigma; c.v = vn; c.out = Hv;
     cudaStream_t s = (cudaStream_t)stream;
-    if (st == OCP_OK) st = heat_prod2(h, a, b, &c, s);
+    if (st == OCP_OK) st = heat_prod3(h, a, b, c, s);
     return st == OCP_OK ? extra_prod3(h, a, b, c, s) : st;
   }
   EvalCall c = full_call(h);

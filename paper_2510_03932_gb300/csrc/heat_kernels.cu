@@ -27,8 +27,15 @@ namespace ocpg {
 
 constexpr int HEAT_MAXC = 128;
 constexpr int HT_LANES = HEAT_TILE_NODES;
-constexpr int HT_WARPS = 8;
+constexpr int HT_WARPS = 8;                          // most warps of a whole-tile CTA
 constexpr int HT_THREADS = HT_LANES * HT_WARPS;
+// Warps of a whole-tile CTA: one per group of eight cells, 1, 2, 4 or 8, in launches of more than one
+// wave of CTAs (with eight for every cell count, seven of eight warps of an 8-cell problem only
+// waited: its step at N = 1e5 115 -> 101 us); eight in smaller ones, where all of them stage a tile.
+static int heat_warps(int n, int64_t tiles, int num_sms) {
+  if (tiles <= (int64_t)5 * num_sms || n > 32) return HT_WARPS;
+  return n <= 8 ? 1 : n <= 16 ? 2 : 4;
+}
 
 struct HeatArgs {
   const double* __restrict__ x;
@@ -47,6 +54,7 @@ struct HeatArgs {
   double di_m1, di_p1, dl_m1, dl_p1;  // d_in - 1, d_in + 1, d_last - 1, d_last + 1
   double h3, h6, hidx2;     // 3 hh, 6 hh, hh/dx^2
   double one, mz;           // 1.0 and -0.0 at run time: sums and products are issued as FMAs
+  int soft;                 // integer products (soft_mul.cuh): the constants allow them and the launch is large
   double cq_in[HEAT_MAXC + 1], cq_end[HEAT_MAXC + 1];
   double gq_in[HEAT_MAXC + 1], gq_end[HEAT_MAXC + 1];
   double ref[HEAT_MAXC + 1];
@@ -65,17 +73,31 @@ __device__ __forceinline__ double hadd(const HeatArgs& a, double u, double v) { 
 __device__ __forceinline__ double hsub(const HeatArgs& a, double u, double v) { return fma(-v, a.one, u); }
 __device__ __forceinline__ double hmul(const HeatArgs& a, double u, double v) { return fma(u, v, a.mz); }
 
+// The plain products of a cell's work: on the FP64 pipe (ModelConst) or, in large launches, on the
+// integer pipes (SoftConst, soft_mul.cuh).  A warp (32 nodes of one cell) decides for each cell,
+// from the operands that the cell's inputs give (`ok`); lanes without a node work on ones.  With them
+// (64 cells) the step takes 105 us at N = 2e4 and 743 at 2e5 (124 and 914 before), J + H 21.8 (24.8), Jv 23.0
+// (27.0), H v 16.9 (19.0), c 25.0 (31.0).
+template <bool IP>
+__device__ __forceinline__ ModelConst heat_consts(const HeatArgs& a) {
+  ModelConst K;
+  K.one = a.one; K.mz = a.mz;
+  K.soft = IP ? a.soft : 0;
+  return K;
+}
+
 // Stage the states (and controls) of nodes [r0, r0+nn) into sX[t*(n+1) + k], sX[t*(n+1) + n] = u.
+template <int THREADS>
 __device__ __forceinline__ void heat_stage(const HeatArgs& a, const double* __restrict__ src, int64_t r0, int nn,
                                            double* sX) {
   const int n = a.n, ld = n + 1;
   const int total = nn * n;
   const double* base = src + (int64_t)n * r0;
-  for (int i = threadIdx.x; i < total; i += HT_THREADS) {
+  for (int i = threadIdx.x; i < total; i += THREADS) {
     const int t = i / n, k = i - t * n;
     sX[t * ld + k] = __ldg(base + i);
   }
-  for (int t = threadIdx.x; t < nn; t += HT_THREADS) sX[t * ld + n] = __ldg(src + a.uoff + r0 + t);
+  for (int t = threadIdx.x; t < nn; t += THREADS) sX[t * ld + n] = __ldg(src + a.uoff + r0 + t);
 }
 
 // ======================================================================================
@@ -123,32 +145,77 @@ __device__ __forceinline__ void heat_jbound(const HeatArgs& a, int k, int64_t j)
   if (a.has_final && j == a.N) a.jv[a.n + k] = 1.0;
 }
 
-// Hessian diagonal of cell k at node j: 6 hh ybar_k x_k + the objective's sigma w q_k
-// (yl, yr = y_{k,j-1}, y_{k,j}, zero beyond the first and last rows)
-__device__ __forceinline__ double heat_hdiag_y(const HeatArgs& a, int k, bool endp, double xk, double yl, double yr) {
-  const double ty = hmul(a, a.h6, hadd(a, yl, yr));
+// Hessian diagonal of cell k at node j: 6 hh ybar_k x_k + the objective's sigma w q_k (ybar_k =
+// y_{k,j-1} + y_{k,j}, zero beyond the first and last rows)
+template <class KC>
+__device__ __forceinline__ double heat_hdiag(const HeatArgs& a, const KC& K, int k, bool endp, double xk, double yb) {
+  const double ty = fmul(K, a.h6, yb);
   return fma(ty, xk, endp ? a.cq_end[k] : a.cq_in[k]);
 }
-__device__ __forceinline__ double heat_hdiag(const HeatArgs& a, int k, int64_t j, bool endp, double xk) {
+// y_{k,j-1} + y_{k,j}
+__device__ __forceinline__ double heat_ybar(const HeatArgs& a, int k, int64_t j) {
   const double yl = (j >= 1) ? __ldg(a.y + a.nb + (int64_t)k * a.N + j - 1) : 0.0;
   const double yr = (j < a.N) ? __ldg(a.y + a.nb + (int64_t)k * a.N + j) : 0.0;
-  return heat_hdiag_y(a, k, endp, xk, yl, yr);
+  return hadd(a, yl, yr);
 }
 
-// gradient entry of cell k at node j and its objective term
-__device__ __forceinline__ void heat_grad(const HeatArgs& a, int k, int64_t j, bool endp, double xk, bool WG, bool WF,
-                                          double& objacc) {
-  const double d = a.has_ref ? hsub(a, xk, a.ref[k]) : xk;
-  const double gk = hmul(a, endp ? a.gq_end[k] : a.gq_in[k], d);
-  if (WF) objacc = fma(gk, d, objacc);
+// gradient entry of cell k at node j and its objective term (d = x_k - ref_k)
+template <class KC>
+__device__ __forceinline__ void heat_grad(const HeatArgs& a, const KC& K, int k, int64_t j, bool endp, double d, bool WG,
+                                          bool WF, double obj0, double& objacc) {
+  const double gk = fmul_w<MUL_G>(K, endp ? a.gq_end[k] : a.gq_in[k], d);
+  if (WF) objacc = fma(gk, d, obj0);
   if (WG) a.g[(int64_t)a.n * j + k] = gk;
 }
 
-template <unsigned OUT>
-__global__ void __launch_bounds__(HT_THREADS, (OUT & O_C) ? 5 : 8) k_heat_eval(const __grid_constant__ HeatArgs a) {
+// tile_sum and finish_tiles for a CTA of W warps, in the order that HT_WARPS warps give (the
+// missing ones add nothing to a tile; the tiles' sums go to HT_THREADS places whatever the CTA).
+template <int W>
+__device__ __forceinline__ double heat_tile_sum(double v, double* red, double one) {
+  red[threadIdx.x] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+    s = red[threadIdx.x];
+    #pragma unroll
+    for (int i = 1; i < W; ++i) s = fma(red[threadIdx.x + 32 * i], one, s);
+    s = warp_sum(s, one);
+  }
+  return s;
+}
+template <int W>
+__device__ __forceinline__ void heat_finish(const HeatArgs& a, double* red) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = (atomicAdd(a.counter, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31;
+  for (int w = threadIdx.x >> 5; w < HT_WARPS; w += W) {
+    double s = 0.0;
+    for (int64_t i = 32 * w + lane; i < a.ntiles; i += HT_THREADS) s = s + __ldcg(a.partials + i);
+    s = warp_sum(s, 1.0);
+    if (lane == 0) red[w] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < HT_WARPS; ++w) s = fma(red[w], 1.0, s);
+    *a.f = 0.5 * s;
+    *a.counter = 0u;
+  }
+}
+
+template <unsigned OUT, bool IP, int W>
+__global__ void __launch_bounds__(32 * W, (OUT & O_C) ? (W > 1 ? 40 / W : 32) : (W > 1 ? 64 / W : 32)) k_heat_eval(const __grid_constant__ HeatArgs a) {
   constexpr bool CF = OUT & O_F, CC = OUT & O_C, CG = OUT & O_G, CJ = OUT & O_J, CH = OUT & O_H;
   // the full kernel also serves output subsets: NULL outputs are skipped
   const bool WF = CF && a.f, WC = CC && a.c, WG = CG && a.g, WJ = CJ && a.jv, WH = CH && a.hv;
+  constexpr int THREADS = 32 * W;
   extern __shared__ __align__(16) double sm[];
   const int n = a.n, ld = n + 1;
   // shared memory: states, then only the staging buffers this variant needs.  The gradient
@@ -160,6 +227,8 @@ __global__ void __launch_bounds__(HT_THREADS, (OUT & O_C) ? 5 : 8) k_heat_eval(c
   double* red = sX;                                            // reduction, 256 (after the stores)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double objacc = 0.0;
+  const ModelConst K0 = heat_consts<IP>(a);
+  constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
 
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
     const int64_t r0 = a.B + tile * (HT_LANES - 1);
@@ -174,15 +243,21 @@ __global__ void __launch_bounds__(HT_THREADS, (OUT & O_C) ? 5 : 8) k_heat_eval(c
     const bool act = t < nn;
     const bool own = t < nown;
     const bool endp = (j == 0) || (j == a.N);
-    heat_stage(a, a.x, r0, nn, sX);
+    heat_stage<THREADS>(a, a.x, r0, nn, sX);
     __syncthreads();
     // ---- Hessian diagonal of every owned (node, cell), elementwise: warps take whole cells
     // (lanes = nodes, the multipliers' rows coalesced), so no load waits inside the cell loop
     // (measured: the separate pass speeds up the full evaluation; J + H alone is faster with
     // the diagonal computed in its cell loop)
-    if (CC && WH && own) {
+    if (CC && WH) {
 #pragma unroll 2
-      for (int k = warp; k < n; k += HT_WARPS) sN[t * ld + k] = heat_hdiag(a, k, j, endp, sX[t * ld + k]);
+      for (int k = warp; k < n; k += W) {
+        const double yb = own ? heat_ybar(a, k, j) : 1.0, xk = own ? sX[t * ld + k] : 1.0;
+        with_products<SOFT>(K0, true, soft_value(yb), [&](const auto& K) __attribute__((always_inline)) {
+          const double h = heat_hdiag(a, K, k, endp, xk, yb);
+          if (own) sN[t * ld + k] = h;
+        });
+      }
     }
 
     // ---- control entries (warp 0): gradient, objective, Hessian (u,u)
@@ -202,50 +277,58 @@ __global__ void __launch_bounds__(HT_THREADS, (OUT & O_C) ? 5 : 8) k_heat_eval(c
       // One cell k of the tile's nodes; LAST: k is the Neumann end n-1.  The end cell is
       // peeled out of the loop so that its Laplacian and diagonal constant are compile-time
       // choices: a run-time select between two FP64 results issues both on every cell.
-      auto cell = [&](const int k, auto last_tag) {
+      // (xl, xk, xr: the left neighbour (the control for k = 0), the cell, its right neighbour)
+      auto cell = [&](const int k, auto last_tag, const double xl, const double xk, const double xr) {
         constexpr bool LAST = decltype(last_tag)::value;
-        double xk = 0.0, xl = 0.0, xr = 0.0;
-        if (act) {
-          xk = sX[t * ld + k];
-          xl = (k == 0) ? sX[t * ld + n] : sX[t * ld + k - 1];
-          xr = LAST ? xk : sX[t * ld + k + 1];
-        }
-        const double x2 = hmul(a, xk, xk);
-        if (WJ) heat_jrows(a, k, LAST, t, act, nrows, r0, x2);
+        const double d = ((WG || WF) && a.has_ref) ? hsub(a, xk, a.ref[k]) : xk;
+        const double obj0 = objacc;
+        const bool ok = !act || (soft_value(xk) & soft_value(d));
+        with_products<SOFT>(K0, true, ok, [&](const auto& K) __attribute__((always_inline)) {
+          const double x2 = fmul(K, xk, xk);
+          if (WJ) heat_jrows(a, k, LAST, t, act, nrows, r0, x2);
+          if (WC) {
+            // hh f_k = hh (lap / dx^2 - x^3)
+            // pa = x + hh f, pb = x - hh f, with hh f = hh/dx^2 lap - hh x^3
+            const double lap = LAST ? hsub(a, xl, xk) : fma(-2.0, xk, hadd(a, xl, xr));
+            const double x3 = fmul(K, x2, xk);
+            const double pa = fma(a.hidx2, lap, fma(a.mhh, x3, xk));
+            const double pb = fma(-a.hidx2, lap, fma(a.hh, x3, xk));
+            const double nb = __shfl_down_sync(0xffffffffu, pb, 1);
+            if (t < nrows) a.c[a.nb + (int64_t)k * a.N + j] = hsub(a, nb, pa);
+          }
+          if (own && (WG || WF)) heat_grad(a, K, k, j, endp, d, WG, WF, obj0, objacc);
+        });
         if (WJ && own) heat_jbound(a, k, j);
         if (WC) {
-          // hh f_k = hh (lap / dx^2 - x^3)
-          // pa = x + hh f, pb = x - hh f, with hh f = hh/dx^2 lap - hh x^3
-          const double lap = LAST ? hsub(a, xl, xk) : fma(-2.0, xk, hadd(a, xl, xr));
-          const double x3 = hmul(a, x2, xk);
-          const double pa = fma(a.hidx2, lap, fma(a.mhh, x3, xk));
-          const double pb = fma(-a.hidx2, lap, fma(a.hh, x3, xk));
-          const double nb = __shfl_down_sync(0xffffffffu, pb, 1);
-          if (t < nrows) a.c[a.nb + (int64_t)k * a.N + j] = hsub(a, nb, pa);
           if (own && j == 0) a.c[k] = xk;
           if (own && a.has_final && j == a.N) a.c[n + k] = xk;
         }
-        if (own && (WG || WF)) heat_grad(a, k, j, endp, xk, WG, WF, objacc);
       };
-      for (int gi = warp; gi < ngroups; gi += HT_WARPS) {
+      auto state = [&](int k) { return act ? sX[t * ld + k] : 1.0; };
+      for (int gi = warp; gi < ngroups; gi += W) {
         const int k0 = gi * 8, k1 = min(k0 + 8, n);
         const int kin = min(k1, n - 1);  // interior cells of the group: k0 .. kin-1
+        double xl = state(k0 == 0 ? n : k0 - 1), xk = state(k0);
 #pragma unroll 1
-        for (int k = k0; k < kin; ++k) cell(k, std::false_type{});
-        if (k1 == n) cell(n - 1, std::true_type{});
+        for (int k = k0; k < kin; ++k) {
+          const double xr = state(k + 1);
+          cell(k, std::false_type{}, xl, xk, xr);
+          xl = xk;
+          xk = xr;
+        }
+        if (k1 == n) cell(n - 1, std::true_type{}, xl, xk, xk);
       }
     } else {
       // without the constraints one loop body for every cell (smaller and measured faster)
-      for (int gi = warp; gi < ngroups; gi += HT_WARPS) {
+      for (int gi = warp; gi < ngroups; gi += W) {
         const int k0 = gi * 8, k1 = min(k0 + 8, n);
         for (int k = k0; k < k1; ++k) {
           const bool last = (k == n - 1);
-          double xk = 0.0;
-          if (act) xk = sX[t * ld + k];
+          const double xk = act ? sX[t * ld + k] : 1.0;
           if (WJ) heat_jrows(a, k, last, t, act, nrows, r0, hmul(a, xk, xk));
           if (WJ && own) heat_jbound(a, k, j);
-          if (own && WH) sN[t * ld + k] = heat_hdiag(a, k, j, endp, xk);
-          if (own && (WG || WF)) heat_grad(a, k, j, endp, xk, WG, WF, objacc);
+          if (own && WH) sN[t * ld + k] = heat_hdiag(a, K0, k, endp, xk, heat_ybar(a, k, j));
+          if (own && (WG || WF)) heat_grad(a, K0, k, j, endp, a.has_ref ? hsub(a, xk, a.ref[k]) : xk, WG, WF, objacc, objacc);
         }
       }
     }
@@ -253,20 +336,20 @@ __global__ void __launch_bounds__(HT_THREADS, (OUT & O_C) ? 5 : 8) k_heat_eval(c
     if (WH) {
       const int total = nown * n;
       double* dst = a.hv + (int64_t)n * r0;
-      for (int i = threadIdx.x; i < total; i += HT_THREADS) {
+      for (int i = threadIdx.x; i < total; i += THREADS) {
         const int tt = i / n, k = i - tt * n;
         dst[i] = sN[tt * ld + k];
       }
     }
     if (WF) {
       __syncthreads();  // red is the states' buffer, read by the loop above
-      const double ts = tile_sum<HT_THREADS>(objacc, red, a.one);
+      const double ts = heat_tile_sum<W>(objacc, red, a.one);
       if (threadIdx.x == 0) a.partials[tile] = ts;
       objacc = 0.0;
     }
     __syncthreads();
   }
-  if (WF) finish_tiles<HT_THREADS>(a.partials, a.ntiles, a.counter, a.f, 0.5, red);
+  if (WF) heat_finish<W>(a, red);
 }
 
 // ======================================================================================
@@ -279,7 +362,7 @@ __global__ void __launch_bounds__(HT_THREADS, (OUT & O_C) ? 5 : 8) k_heat_eval(c
 // ======================================================================================
 constexpr int HJ_CELLS = 16, HJ_WARPS = 2, HJ_THREADS = 32 * HJ_WARPS, HJ_LD = HJ_CELLS + 1;
 
-template <unsigned OUT>
+template <unsigned OUT, bool IP>
 __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_jh(const __grid_constant__ HeatArgs a, int cgroups) {
   constexpr bool CJ = OUT & O_J, CH = OUT & O_H;
   const bool WJ = CJ && a.jv, WH = CH && a.hv;
@@ -289,6 +372,8 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_jh(const __grid_constan
   __shared__ double sY[HJ_CELLS * HT_LANES];
   const int n = a.n;
   const int t = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const ModelConst K0 = heat_consts<IP>(a);
+  constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
   const int64_t units = a.ntiles * cgroups;
   for (int64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
     const int64_t tile = unit / cgroups;
@@ -322,12 +407,17 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_jh(const __grid_constan
     const int k1 = min(8 * warp + 8, nc);
     for (int kk = 8 * warp; kk < k1; ++kk) {
       const int k = c0 + kk;
-      double xk = 0.0;
-      if (act) xk = sX[t * HJ_LD + kk];
-      if (WJ) heat_jrows(a, k, k == n - 1, t, act, nrows, r0, hmul(a, xk, xk));
-      if (WJ && own) heat_jbound(a, k, j);
+      const double xk = act ? sX[t * HJ_LD + kk] : 1.0;
       // an owned lane t <= 30 reads the multipliers of rows j-1 and j at positions t and t+1
-      if (own && WH) sX[t * HJ_LD + kk] = heat_hdiag_y(a, k, endp, xk, sY[kk * HT_LANES + t], sY[kk * HT_LANES + t + 1]);
+      const double yb = (own && WH) ? hadd(a, sY[kk * HT_LANES + t], sY[kk * HT_LANES + t + 1]) : 1.0;
+      with_products<SOFT>(K0, true, (!WJ || soft_value(xk)) & soft_value(yb), [&](const auto& K) __attribute__((always_inline)) {
+        if (WJ) heat_jrows(a, k, k == n - 1, t, act, nrows, r0, fmul(K, xk, xk));
+        if (WH) {
+          const double h = heat_hdiag(a, K, k, endp, xk, yb);
+          if (own) sX[t * HJ_LD + kk] = h;
+        }
+      });
+      if (WJ && own) heat_jbound(a, k, j);
     }
     __syncthreads();
     if (WH) {
@@ -347,12 +437,16 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_jh(const __grid_constan
 // other products, 23.3 against 24.3 us at N = 2e4, 39.4 against 41.1 at N = 5e4); at most 51
 // registers: five CTAs per SM, one wave of 626 tiles at N = 2e4 (measured faster)
 // ======================================================================================
-__global__ void __launch_bounds__(HT_THREADS, 5) k_heat_hprod(const __grid_constant__ HeatArgs a) {
+template <bool IP, int W>
+__global__ void __launch_bounds__(32 * W, W > 1 ? 40 / W : 32) k_heat_hprod(const __grid_constant__ HeatArgs a) {
+  constexpr int THREADS = 32 * W;
   extern __shared__ __align__(16) double sm[];
   const int n = a.n, ld = n + 1;
   double* sX = sm;
   double* sV = sX + HT_LANES * ld;  // the direction
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const ModelConst K0 = heat_consts<IP>(a);
+  constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
     const int64_t r0 = tile * HT_LANES;
     const int nn = (int)min((int64_t)HT_LANES, a.N + 1 - r0);
@@ -360,11 +454,11 @@ __global__ void __launch_bounds__(HT_THREADS, 5) k_heat_hprod(const __grid_const
     const int64_t j = r0 + t;
     const bool act = t < nn;
     const bool endp = (j == 0) || (j == a.N);
-    heat_stage(a, a.x, r0, nn, sX);
-    heat_stage(a, a.v, r0, nn, sV);
+    heat_stage<THREADS>(a, a.x, r0, nn, sX);
+    heat_stage<THREADS>(a, a.v, r0, nn, sV);
     __syncthreads();
     const int ngroups = (n + 7) / 8;
-    for (int gi = warp; gi < ngroups; gi += HT_WARPS) {
+    for (int gi = warp; gi < ngroups; gi += W) {
       const int k0 = gi * 8, k1 = min(k0 + 8, n);
       // elementwise: the group's multiplier rows are loaded before any arithmetic needs them
       double yl[8], yr[8];
@@ -377,11 +471,13 @@ __global__ void __launch_bounds__(HT_THREADS, 5) k_heat_hprod(const __grid_const
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int k = k0 + q;
-        if (act && k < k1) {
-          const double xk = sX[t * ld + k];
-          const double hk = fma(hmul(a, a.h6, hadd(a, yl[q], yr[q])), xk, endp ? a.cq_end[k] : a.cq_in[k]);
-          sX[t * ld + k] = hmul(a, hk, sV[t * ld + k]);  // in place: x no longer needed for cell k
-        }
+        if (k >= k1) continue;   // (warp-uniform)
+        const double xk = act ? sX[t * ld + k] : 1.0, vk = act ? sV[t * ld + k] : 1.0;
+        const double yb = act ? hadd(a, yl[q], yr[q]) : 1.0;
+        with_products<SOFT>(K0, true, soft_value(vk) & soft_value(yb), [&](const auto& K) __attribute__((always_inline)) {
+          const double h = fmul(K, heat_hdiag(a, K, k, endp, xk, yb), vk);
+          if (act) sX[t * ld + k] = h;   // in place: x no longer needed for cell k
+        });
       }
     }
     if (warp == 0 && act) {
@@ -392,11 +488,11 @@ __global__ void __launch_bounds__(HT_THREADS, 5) k_heat_hprod(const __grid_const
     {
       const int total = nn * n;
       double* dst = a.out + (int64_t)n * r0;
-      for (int i = threadIdx.x; i < total; i += HT_THREADS) {
+      for (int i = threadIdx.x; i < total; i += THREADS) {
         const int tt = i / n, k = i - tt * n;
         dst[i] = sX[tt * ld + k];
       }
-      for (int tt = threadIdx.x; tt < nn; tt += HT_THREADS) a.out[a.uoff + r0 + tt] = sX[tt * ld + n];
+      for (int tt = threadIdx.x; tt < nn; tt += THREADS) a.out[a.uoff + r0 + tt] = sX[tt * ld + n];
     }
     __syncthreads();
   }
@@ -422,7 +518,7 @@ __global__ void __launch_bounds__(HT_THREADS, 5) k_heat_hprod(const __grid_const
 enum : int { HP_JPROD = 0, HP_JTPROD = 1, HP_BOTH = 2, HP_ALL3 = 3 };
 constexpr int HP_LDV = HJ_CELLS + 3;  // padded row of the staged direction (or J^T w result)
 
-template <int KIND>
+template <int KIND, bool IP>
 __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_constant__ HeatArgs a, int cgroups) {
   constexpr bool ALL3 = KIND == HP_ALL3, BOTH = KIND == HP_BOTH || ALL3;
   constexpr bool JP = KIND == HP_JPROD || BOTH, JT = KIND == HP_JTPROD || BOTH;
@@ -434,6 +530,8 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
   double* const wout = BOTH ? a.out2 : a.out;
   const int n = a.n;
   const int t = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const ModelConst K0 = heat_consts<IP>(a);
+  constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
   const int64_t units = a.ntiles * cgroups;
   for (int64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
     const int64_t tile = unit / cgroups;
@@ -482,25 +580,22 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
       }
       for (int kk = kb; kk < ke; ++kk) {
         const int k = c0 + kk;
-        double p = 0.0, vk = 0.0;
-        if (act) {
-          const double xk = sX[t * HJ_LD + kk];
-          const bool last = (k == n - 1);
-          if (ALL3 && jown) {  // H v: (2 sigma w q_k + 6 hh ybar_k x_k) v_k
-            const double* yrow = a.y + a.nb + (int64_t)k * a.N;
-            const double yl = (j >= 1) ? __ldg(yrow + j - 1) : 0.0;
-            const double yr = (j < a.N) ? __ldg(yrow + j) : 0.0;
-            const double hk = fma(hmul(a, a.h6, hadd(a, yl, yr)), xk, endp ? a.cq_end[k] : a.cq_in[k]);
-            a.out3[(int64_t)n * j + k] = hmul(a, hk, sV[t * HP_LDV + kk + 1]);
+        const bool last = (k == n - 1);
+        const double xk = act ? sX[t * HJ_LD + kk] : 1.0, vk = act ? sV[t * HP_LDV + kk + 1] : 1.0;
+        const double yb = (ALL3 && jown) ? heat_ybar(a, k, j) : 1.0;
+        // the left neighbour's entry (the control's for k = 0), plus the right one's
+        const double vl = sV[t * HP_LDV + kk];
+        const double nsum = last ? vl : hadd(a, vl, sV[t * HP_LDV + kk + 2]);
+        with_products<SOFT>(K0, true, soft_value(xk) & soft_value(vk) & soft_value(yb), [&](const auto& K) __attribute__((always_inline)) {
+          if (ALL3) {  // H v: (2 sigma w q_k + 6 hh ybar_k x_k) v_k
+            const double h = fmul(K, heat_hdiag(a, K, k, endp, xk, yb), vk);
+            if (jown) a.out3[(int64_t)n * j + k] = h;
           }
-          vk = sV[t * HP_LDV + kk + 1];
-          const double vl = sV[t * HP_LDV + kk];  // cell k-1, or the control for k = 0
-          const double dk = fma(a.h3, hmul(a, xk, xk), last ? a.d_last : a.d_in);
-          const double nsum = last ? vl : hadd(a, vl, sV[t * HP_LDV + kk + 2]);
-          p = fma(a.mhidx2, nsum, hmul(a, dk, vk));
-        }
-        const double right = __shfl_down_sync(0xffffffffu, hadd(a, p, vk), 1);
-        if (t < nrows) a.out[a.nb + (int64_t)k * a.N + j] = hadd(a, hsub(a, p, vk), right);
+          const double dk = fma(a.h3, fmul(K, xk, xk), last ? a.d_last : a.d_in);
+          const double p = fma(a.mhidx2, nsum, fmul(K, dk, vk));
+          const double right = __shfl_down_sync(0xffffffffu, hadd(a, p, vk), 1);
+          if (t < nrows) a.out[a.nb + (int64_t)k * a.N + j] = hadd(a, hsub(a, p, vk), right);
+        });
         if (act && j == 0) a.out[k] = vk;
         if (act && a.has_final && j == a.N && t < nown) a.out[n + k] = vk;
       }
@@ -590,6 +685,20 @@ static void heat_fill(const ocp* h, double sigma, HeatArgs& a) {
   }
   a.partials = h->d_partials;
   a.counter = h->d_counter;
+  // (a thread takes eight cells of a node, so a node counts n / 8 times)
+  auto fits = [](double v) { return v >= 0x1p-64 && v < 0x1p64; };
+  a.soft = soft_launch((h->N + 1) * (int64_t)n / 8, h->num_sms) && fits(a.h6);
+}
+
+// Calls fn with the number of warps as a compile-time constant.
+template <class Fn>
+static cudaError_t with_warps(int w, Fn&& fn) {
+  switch (w) {
+    case 1: return fn(std::integral_constant<int, 1>{});
+    case 2: return fn(std::integral_constant<int, 2>{});
+    case 4: return fn(std::integral_constant<int, 4>{});
+    default: return fn(std::integral_constant<int, HT_WARPS>{});
+  }
 }
 
 template <unsigned OUT>
@@ -604,13 +713,16 @@ static ocp_status heat_eval_t(ocp* h, const EvalCall& c, cudaStream_t s) {
   if (a.ntiles > h->max_partials) return set_err(h, OCP_EDIM, "too many tiles for the reduction scratch");
   const int ld = h->nx + 1;
   const size_t smem = sizeof(double) * ((size_t)heat_xlen(h->nx) + ((OUT & O_H) ? (HT_LANES - 1) * ld : 0));
-  auto kern = k_heat_eval<OUT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_err(h, e, "cudaFuncSetAttribute(heat)");
-  const int grid = occupancy_grid(h, (const void*)kern, HT_THREADS, smem, a.ntiles);
-  if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
-  kern<<<grid, HT_THREADS, smem, s>>>(a);
-  return cuda_err(h, cudaGetLastError(), "k_heat_eval launch");
+  constexpr bool MUL = (OUT & O_C) != 0;   // integer products (the other instances are bound by other things)
+  auto go = [&](auto w) -> cudaError_t {
+    constexpr int W = decltype(w)::value;
+    auto kern = (MUL && a.soft) ? k_heat_eval<OUT, MUL, W> : k_heat_eval<OUT, false, W>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<occupancy_grid(h, (const void*)kern, 32 * W, smem, a.ntiles), 32 * W, smem, s>>>(a);
+    return cudaGetLastError();
+  };
+  return cuda_err(h, with_warps(heat_warps(h->nx, a.ntiles, h->num_sms), go), "k_heat_eval launch");
 }
 
 // Jacobian and / or Hessian values alone: units of one tile and 16 cells (k_heat_jh)
@@ -624,7 +736,7 @@ static ocp_status heat_jh_t(ocp* h, const EvalCall& c, cudaStream_t s) {
   a.ntiles = (nodes + (HT_LANES - 2)) / (HT_LANES - 1);
   if (a.ntiles < 1) a.ntiles = 1;
   const int cgroups = (h->nx + HJ_CELLS - 1) / HJ_CELLS;
-  auto kern = k_heat_jh<OUT>;
+  auto kern = a.soft ? k_heat_jh<OUT, true> : k_heat_jh<OUT, false>;
   const int grid = occupancy_grid(h, (const void*)kern, HJ_THREADS, 0, a.ntiles * cgroups);
   if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
   kern<<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
@@ -643,20 +755,19 @@ ocp_status heat_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
   }
 }
 
-// Jv (jp.v -> jp.out), J^T w (jt.v -> jt.out) and, with hp, H v (hp.y, hp.sigma, the direction
-// jp.v -> hp.out) of the heat model in one launch (the fused step)
-ocp_status heat_prod2(ocp* h, const ProdCall& jp, const ProdCall& jt, const ProdCall* hp, cudaStream_t s) {
+// Jv (jp.v -> jp.out), J^T w (jt.v -> jt.out) and H v (hp.y, hp.sigma, the direction jp.v ->
+// hp.out) of the heat model in one launch (the fused step)
+ocp_status heat_prod3(ocp* h, const ProdCall& jp, const ProdCall& jt, const ProdCall& hp, cudaStream_t s) {
   HeatArgs a;
-  heat_fill(h, hp ? hp->sigma : 1.0, a);
+  heat_fill(h, hp.sigma, a);
   a.x = jp.x; a.v = jp.v; a.out = jp.out; a.v2 = jt.v; a.out2 = jt.out;
-  if (hp) { a.y = hp->y; a.out3 = hp->out; }
+  a.y = hp.y; a.out3 = hp.out;
   const int cgroups = (h->nx + HJ_CELLS - 1) / HJ_CELLS;
   a.ntiles = (h->N + 1 + (HT_LANES - 2)) / (HT_LANES - 1);
-  const void* k = hp ? (const void*)k_heat_prod_unit<HP_ALL3> : (const void*)k_heat_prod_unit<HP_BOTH>;
-  const int grid = occupancy_grid(h, k, HJ_THREADS, 0, a.ntiles * cgroups);
+  auto k = a.soft ? k_heat_prod_unit<HP_ALL3, true> : k_heat_prod_unit<HP_ALL3, false>;
+  const int grid = occupancy_grid(h, (const void*)k, HJ_THREADS, 0, a.ntiles * cgroups);
   if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
-  if (hp) k_heat_prod_unit<HP_ALL3><<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
-  else k_heat_prod_unit<HP_BOTH><<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
+  k<<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
   return cuda_err(h, cudaGetLastError(), "heat product launch");
 }
 
@@ -667,21 +778,25 @@ ocp_status heat_prod(ocp* h, const ProdCall& c, cudaStream_t s) {
   if (c.kind == P_HPROD) {
     a.ntiles = (h->N + 1 + HT_LANES - 1) / HT_LANES;
     const size_t smem = sizeof(double) * (size_t)HT_LANES * (h->nx + 1) * 2;  // states and direction
-    auto k = k_heat_hprod;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_err(h, e, "cudaFuncSetAttribute(heat hprod)");
-    const int grid = occupancy_grid(h, (const void*)k, HT_THREADS, smem, a.ntiles);
-    k<<<grid, HT_THREADS, smem, s>>>(a);
-    return cuda_err(h, cudaGetLastError(), "heat product launch");
+    auto go = [&](auto w) -> cudaError_t {
+      constexpr int W = decltype(w)::value;
+      auto k = a.soft ? k_heat_hprod<true, W> : k_heat_hprod<false, W>;
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      k<<<occupancy_grid(h, (const void*)k, 32 * W, smem, a.ntiles), 32 * W, smem, s>>>(a);
+      return cudaGetLastError();
+    };
+    return cuda_err(h, with_warps(heat_warps(h->nx, a.ntiles, h->num_sms), go), "heat product launch");
   }
   const int cgroups = (h->nx + HJ_CELLS - 1) / HJ_CELLS;
   if (c.kind == P_JPROD) a.ntiles = (h->N + 1 + (HT_LANES - 2)) / (HT_LANES - 1);
   else a.ntiles = (h->N + 1 + HT_LANES - 1) / HT_LANES;
-  const void* k = (c.kind == P_JPROD) ? (const void*)k_heat_prod_unit<HP_JPROD> : (const void*)k_heat_prod_unit<HP_JTPROD>;
-  const int grid = occupancy_grid(h, k, HJ_THREADS, 0, a.ntiles * cgroups);
+  // (J^T w has one plain product per cell, left to the FP64 pipe)
+  auto k = c.kind == P_JTPROD ? k_heat_prod_unit<HP_JTPROD, false>
+                              : a.soft ? k_heat_prod_unit<HP_JPROD, true> : k_heat_prod_unit<HP_JPROD, false>;
+  const int grid = occupancy_grid(h, (const void*)k, HJ_THREADS, 0, a.ntiles * cgroups);
   if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
-  if (c.kind == P_JPROD) k_heat_prod_unit<HP_JPROD><<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
-  else k_heat_prod_unit<HP_JTPROD><<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
+  k<<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
   return cuda_err(h, cudaGetLastError(), "heat product launch");
 }
 
