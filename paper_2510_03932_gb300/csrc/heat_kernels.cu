@@ -509,25 +509,24 @@ __global__ void __launch_bounds__(32 * W, W > 1 ? 40 / W : 32) k_heat_hprod(cons
 //   J^T w:  out_a = (w_{a,j-1} - w_{a,j}) + wbar_a dd_a - hh/dx^2 (wbar_{a-1} + wbar_{a+1}),
 //           out_u = -hh/dx^2 wbar_0  (dd_a = -hh df_a/dx_a), node-local on disjoint tiles; the
 //           result is staged and stored node by node in runs of the unit's cells.
-//   Both (the heat model's fused step): the two products of the same unit in one launch, on the
+//   All three (the heat model's fused step): the products of the same unit in one launch, on the
 //           tiles of Jv; J^T w for the owned nodes, its result written over the staged states
-//           once Jv has read them.  All three: H v of the owned nodes as well, each entry formed
-//           in Jv's cell loop from the same state and direction values and stored by its lane.
-//           Each entry by the same expressions as the separate launches.
+//           (where Jv leaves -hh df_a/dx_a, which J^T w needs of them); H v of the owned nodes, each
+//           entry formed in Jv's cell loop from the same state and direction values and stored by
+//           its lane.  Each entry by the same expressions as the separate launches.
 // ======================================================================================
-enum : int { HP_JPROD = 0, HP_JTPROD = 1, HP_BOTH = 2, HP_ALL3 = 3 };
+enum : int { HP_JPROD = 0, HP_JTPROD = 1, HP_ALL3 = 3 };
 constexpr int HP_LDV = HJ_CELLS + 3;  // padded row of the staged direction (or J^T w result)
 
 template <int KIND, bool IP>
 __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_constant__ HeatArgs a, int cgroups) {
-  constexpr bool ALL3 = KIND == HP_ALL3, BOTH = KIND == HP_BOTH || ALL3;
-  constexpr bool JP = KIND == HP_JPROD || BOTH, JT = KIND == HP_JTPROD || BOTH;
+  constexpr bool ALL3 = KIND == HP_ALL3, JP = KIND == HP_JPROD || ALL3, JT = KIND == HP_JTPROD || ALL3;
   constexpr int LDV = JP ? HP_LDV : HJ_LD;
   __shared__ double sX[HT_LANES * HJ_LD];  // states of the unit's cells (both: then the J^T w result)
   __shared__ double sV[HT_LANES * LDV];    // Jv: the direction; J^T w alone: the result
-  double* const sO = BOTH ? sX : sV;       // the J^T w result (row length HJ_LD either way)
-  const double* const wv = BOTH ? a.v2 : a.v;
-  double* const wout = BOTH ? a.out2 : a.out;
+  double* const sO = ALL3 ? sX : sV;       // the J^T w result (row length HJ_LD either way)
+  const double* const wv = ALL3 ? a.v2 : a.v;
+  double* const wout = ALL3 ? a.out2 : a.out;
   const int n = a.n;
   const int t = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const ModelConst K0 = heat_consts<IP>(a);
@@ -553,10 +552,10 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
       nn = (int)min((int64_t)HT_LANES, a.N + 1 - r0);
       bnd = (tile == 0) || (r0 + HT_LANES > a.N);
     }
-    if (BOTH) bnd = (r0 == 0) || (r0 + nown == a.N + 1);  // the tile holds node 0 or node N
+    if (ALL3) bnd = (r0 == 0) || (r0 + nown == a.N + 1);  // the tile holds node 0 or node N
     const int64_t j = r0 + t;
     const bool act = t < nn;
-    const bool jown = BOTH ? (t < nown) : act;  // J^T w: the owned nodes
+    const bool jown = ALL3 ? (t < nown) : act;  // J^T w: the owned nodes
     for (int i = threadIdx.x; i < nn * nc; i += HJ_THREADS) {
       const int tt = i / nc, kk = i - tt * nc;
       sX[tt * HJ_LD + kk] = __ldg(a.x + (int64_t)n * (r0 + tt) + c0 + kk);
@@ -592,6 +591,7 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
             if (jown) a.out3[(int64_t)n * j + k] = h;
           }
           const double dk = fma(a.h3, fmul(K, xk, xk), last ? a.d_last : a.d_in);
+          if (JT) sX[t * HJ_LD + kk] = dk;   // J^T w needs of the state only this, in this thread
           const double p = fma(a.mhidx2, nsum, fmul(K, dk, vk));
           const double right = __shfl_down_sync(0xffffffffu, hadd(a, p, vk), 1);
           if (t < nrows) a.out[a.nb + (int64_t)k * a.N + j] = hadd(a, hsub(a, p, vk), right);
@@ -619,9 +619,8 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
         if (jown) {
           double wlp = 0.0, wrp = 0.0;
           if (k + 1 < n) { wbar(k + 1, wlp, wrp); wbp = hadd(a, wlp, wrp); } else wbp = 0.0;
-          const double xk = sX[t * HJ_LD + (k - c0)];
-          const bool last = (k == n - 1);
-          const double dk = fma(a.h3, hmul(a, xk, xk), last ? a.d_last : a.d_in);
+          double dk = sX[t * HJ_LD + (k - c0)];
+          if (!JP) dk = fma(a.h3, hmul(a, dk, dk), k == n - 1 ? a.d_last : a.d_in);   // (the state until here)
           double s = fma(wbc, dk, hsub(a, wlc, wrc));
           s = fma(a.mhidx2, hadd(a, wbm, wbp), s);
           if (bnd) {  // only the CTAs holding node 0 or node N (uniform branch)
@@ -637,7 +636,7 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
     if (JT) {
       // node-major results of the unit's cells, in runs of nc per node
       double* dst = wout + (int64_t)n * r0 + c0;
-      const int nst = BOTH ? nown : nn;
+      const int nst = ALL3 ? nown : nn;
       for (int i = threadIdx.x; i < nst * nc; i += HJ_THREADS) {
         const int tt = i / nc, kk = i - tt * nc;
         dst[(int64_t)n * tt + kk] = sO[tt * HJ_LD + kk];
