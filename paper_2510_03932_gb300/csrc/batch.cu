@@ -153,7 +153,7 @@ static const BatchConfig kConfigs[] = {{64, 1}, {128, 1}, {256, 1}, {64, 2}, {12
 template <class M>
 constexpr int batch_max_nodes() { return jrow_total<M>() > 32 ? 128 : 512; }
 
-// (integer products with one node per thread, in batches that soft_launch names large)
+// (integer products with one node per thread, in batches that large_launch names large)
 template <class M, int TILE, int NPT>
 static const void* batch_kernel(bool many) {
   if constexpr (TILE * NPT > batch_max_nodes<M>()) return nullptr;
@@ -188,7 +188,7 @@ struct ocp_batch_impl {
   std::vector<ocp*> items;
   std::vector<int64_t> xoff, coff, joff, hoff, tileoff;
   int threads = 128, npt = 1, ctas_per_sm = 0;
-  bool many = false;   // soft_launch of the whole batch
+  bool many = false;   // large_launch of the whole batch
   int64_t ntiles = 0;
   void* d_inst = nullptr;
   int64_t *d_tileoff = nullptr, *d_xoff = nullptr, *d_coff = nullptr, *d_joff = nullptr, *d_hoff = nullptr;
@@ -390,7 +390,7 @@ ocp_status ocp_batch_create(ocp_t* const* items, int count, ocp_batch_t** out) {
   b->model = model; b->count = count; b->device = items[0]->device; b->num_sms = items[0]->num_sms;
   int64_t nodes = 0;
   for (int i = 0; i < count; ++i) nodes += items[i]->N + 1;
-  b->many = soft_launch(nodes, b->num_sms);
+  b->many = large_launch(nodes, b->num_sms);
   b->items.assign(items, items + count);
   b->xoff.assign(count + 1, 0); b->coff.assign(count + 1, 0); b->joff.assign(count + 1, 0); b->hoff.assign(count + 1, 0);
   int64_t cap = 0;

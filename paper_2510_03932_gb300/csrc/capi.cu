@@ -289,10 +289,11 @@ ocp_status ocp_create(const ocp_dynamics* dyn, const ocp_cost* cost, int nx, int
     free_handle(h);
     return cuda_err(nullptr, e, "cudaDeviceGetAttribute");
   }
-  // one partial per tile of the smallest tile (31 owned nodes), plus slack: this also holds the
-  // four parameter sums per 128-node chunk of the cart-pole's and six series per 255-node tile
-  // of the Goddard model's (dc/dp)^T w
+  // one partial per tile of the smallest tile (31 owned nodes), plus slack: except in small launches this
+  // also holds the four parameter sums per 128-node chunk of the cart-pole's and six series per
+  // 255-node tile of the Goddard model's (dc/dp)^T w; small launches have them per small tile
   h->max_partials = (int)((N + 1) / 31 + 8);
+  if (small_launch(N + 1, h->num_sms)) h->max_partials *= 6;
   if ((e = ocpg::dev_malloc(&h->d_partials, sizeof(double) * h->max_partials)) != cudaSuccess ||
       (e = ocpg::dev_malloc(&h->d_counter, sizeof(unsigned))) != cudaSuccess ||
       (e = cudaMemset(h->d_counter, 0, sizeof(unsigned))) != cudaSuccess) {

@@ -34,7 +34,7 @@
 
 namespace ocpg {
 
-constexpr int GT = 256;  // threads (= nodes) per CTA; a tile owns GT-1 nodes and rows
+constexpr int GOD_TILE = 256;  // threads GT (= nodes) per CTA of large launches (TILE_SMALL in small ones); a tile owns GT-1 nodes
 
 struct GodArgs {
   const double* __restrict__ x;
@@ -58,7 +58,7 @@ struct GodArgs {
   double mayer[3];
   int finpos[3];                     // row of X_{N,k} among the final rows, or -1
   double one, mz;                    // 1.0 and -0.0 at run time (sums and products as FMAs)
-  int many;                          // soft_launch
+  int many, small;                   // large_launch, small_launch
 };
 
 // The inputs of node j's work that its products multiply (see soft_mul.cuh).
@@ -84,7 +84,7 @@ constexpr unsigned G_DP = 1u << 10, G_PAR = 1u << 11;
 
 // Last CTA to finish adds each series q < COUNT of tile sums, partials[q * ntiles + tile], in
 // tile order (see finish_tiles) into dst[q] (skipped where null).
-template <int COUNT>
+template <int GT, int COUNT>
 __device__ __forceinline__ void finish_sums(const double* partials, int64_t ntiles, unsigned* counter,
                                             double* const (&dst)[COUNT], double* red) {
   __shared__ int s_last;
@@ -109,12 +109,13 @@ __device__ __forceinline__ void finish_sums(const double* partials, int64_t ntil
 }
 
 // Resident CTAs per SM that the registers are capped for (0: the allocator's choice): the step at 80
-// (241.6 us at N = 1e6; 255.9 uncapped), the evaluation at 64 (136 us; 156).
-template <unsigned OUT, bool IP>
-constexpr int god_ctas() { return !IP ? 0 : OUT == O_STEP ? 3 : OUT == O_ALL ? 4 : 0; }
+// (241.6 us at N = 1e6; 255.9 uncapped), the evaluation at 64 (136 us; 156), J^T w with (dc/dp)^T w at 64 too
+// (133 us; 149 at 72).
+template <unsigned OUT, bool IP, int GT>
+constexpr int god_ctas() { return GT == TILE_SMALL ? 1 : !IP ? 0 : OUT == O_STEP ? 3 : (OUT == O_ALL || (OUT & G_DP)) ? 4 : 0; }
 
-template <unsigned OUT, bool FREE, bool IP>
-__global__ void __launch_bounds__(GT, god_ctas<OUT, IP>()) k_god(const __grid_constant__ GodArgs a) {
+template <unsigned OUT, bool FREE, bool IP, int GT>
+__global__ void __launch_bounds__(GT, god_ctas<OUT, IP, GT>()) k_god(const __grid_constant__ GodArgs a) {
   constexpr bool WF = OUT & O_F, WC = OUT & O_C, WG = OUT & O_G, WJ = OUT & O_J, WH = OUT & O_H;
   constexpr bool WJV = OUT & O_JV, WJTV = OUT & O_JTV, WHV = OUT & O_HV;
   constexpr bool NEEDD = WJ || WH || WJV || WJTV || WHV;   // first derivatives of f
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(GT, god_ctas<OUT, IP>()) k_god(const __grid_co
     double* const dst[6] = {(RED && WJTV) ? a.ojtv + a.tau : nullptr, (RED && WHV) ? a.ohv + a.tau : nullptr,
                             DP ? a.dpar : nullptr, DP ? a.dpar + 1 : nullptr, DP ? a.dpar + 2 : nullptr,
                             DP ? a.dpar + 3 : nullptr};
-    finish_sums<6>(a.partials, a.ntiles, a.counter, dst, red0);
+    finish_sums<GT, 6>(a.partials, a.ntiles, a.counter, dst, red0);
   }
 }
 
@@ -450,7 +451,10 @@ static void fill_god(const ocp* h, GodArgs& a) {
   a.nb = P.nb;
   a.uoff = 3 * (h->N + 1);
   a.tau = P.free_tf ? P.n - 1 : -1;
-  a.ntiles = (h->N + 1 + GT - 2) / (GT - 1);
+  a.many = large_launch(h->N + 1, h->num_sms);
+  a.small = small_launch(h->N + 1, h->num_sms);
+  const int owned = (a.small ? TILE_SMALL : GOD_TILE) - 1;
+  a.ntiles = (h->N + owned) / owned;
   for (int k = 0; k < 3; ++k) a.jbase[k] = P.jbase[k];
   a.hbase_u = P.hbase_u;
   a.hbase_t = P.hbase_t;
@@ -470,7 +474,6 @@ static void fill_god(const ocp* h, GodArgs& a) {
   for (int k = 0; k < 3; ++k) a.finpos[k] = -1;
   for (size_t i = 0; i < P.fin.size(); ++i) a.finpos[P.fin[i]] = (int)i;
   a.one = 1.0;
-  a.many = soft_launch(h->N + 1, h->num_sms);
   a.mz = -0.0;
   a.partials = h->d_partials;
   a.counter = h->d_counter;
@@ -479,12 +482,13 @@ static void fill_god(const ocp* h, GodArgs& a) {
 template <unsigned OUT, bool FREE>
 static cudaError_t god_launch(const GodArgs& a, cudaStream_t s) {
   constexpr int F1 = FREE ? 1 : 0;
-  const size_t smem = (OUT & O_J) ? sizeof(double) * (size_t)(16 + 3 * F1) * (GT - 1) : 0;
+  auto smem = [](int gt) { return (OUT & O_J) ? sizeof(double) * (size_t)(16 + 3 * F1) * (gt - 1) : 0; };
   const int64_t tiles = a.ntiles - a.tile0;
   const int grid = (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff);
   constexpr bool DYN = (OUT & (O_C | O_J | O_H | O_JV | O_JTV | O_HV)) != 0;   // the dynamics' products
-  if (DYN && a.many) k_god<OUT, FREE, DYN><<<grid, GT, smem, s>>>(a);  // (G_DP, G_PAR bits in OUT)
-  else k_god<OUT, FREE, false><<<grid, GT, smem, s>>>(a);
+  if (a.many) k_god<OUT, FREE, DYN, GOD_TILE><<<grid, GOD_TILE, smem(GOD_TILE), s>>>(a);  // (G_DP, G_PAR bits in OUT)
+  else if (!a.small) k_god<OUT, FREE, false, GOD_TILE><<<grid, GOD_TILE, smem(GOD_TILE), s>>>(a);
+  else k_god<OUT, FREE, false, TILE_SMALL><<<grid, TILE_SMALL, smem(TILE_SMALL), s>>>(a);
   return cudaGetLastError();
 }
 

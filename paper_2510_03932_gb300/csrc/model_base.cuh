@@ -37,8 +37,8 @@ struct ModelConst {
   double one;      // 1.0 and -0.0, passed at run time (see fadd / fmul below)
   double mz;
   double c[16];    // model-specific precomputed constants (see each model)
-  int soft;        // this launch uses integer products (soft_launch and soft_consts)
-  int many;        // soft_launch alone (for parameters that are read on the device)
+  int soft;        // this launch uses integer products (large_launch and soft_consts)
+  int many;        // large_launch alone (for parameters that are read on the device)
 };
 
 // Classes of a node's plain products: intermediates of the dynamics, entries of the Jacobian, of
@@ -54,13 +54,6 @@ struct SoftConst : ModelConst {
   mutable uint32_t worst;
   __device__ __forceinline__ explicit SoftConst(const ModelConst& k) : ModelConst(k), worst(0u) {}
 };
-
-// Integer products pay where the FP64 pipe is saturated: from two warps of nodes per sub-partition
-// on.  A warp alone issues an FP64 instruction every 64 cycles whatever it depends on, and an integer
-// product's 34 dependent instructions take it longer (evaluation, N = 8000: Van der Pol 8.9 us without
-// and 10.2 with them, Goddard 12.8 and 14.6; N = 30000: 8.8 and 9.6, cart-pole 14.9 and 14.7; N = 1e5: 13.5 and
-// 12.7, cart-pole 31.1 and 25.0, Goddard 27.1 and 22.9).
-inline bool soft_launch(int64_t nodes, int num_sms) { return nodes >= (int64_t)256 * num_sms; }
 
 // h/2 and the first n model constants: non-zero and of moderate size
 __host__ __device__ __forceinline__ bool soft_consts(const ModelConst& K, int n) {

@@ -42,6 +42,7 @@ struct CartPole {
       OUT == O_STEP ? 5 : (OUT == O_ALL || OUT == (O_J | O_H) || OUT == O_H) ? 7 : (OUT == O_JTV || OUT == O_HV) ? 6 : 0;
   template <unsigned OUT> static constexpr int CTAS_FP64 = OUT == O_G ? 6 : 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  static constexpr int PROD_TILE = TILE_CARTPOLE;
   static constexpr int EVAL_TILE = TILE_CARTPOLE;
   static constexpr int NC = 15;  // leading constants c[] that products use
   static constexpr int NX = 4, NU = 1, NZ = 5;

@@ -14,6 +14,7 @@ struct Dint {
   template <unsigned OUT> static constexpr unsigned SOFT = 0u;  // (see soft_kernel)
   template <unsigned OUT> static constexpr int CTAS_FP64 = 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  static constexpr int PROD_TILE = TILE_DINT;
   static constexpr int EVAL_TILE = TILE_DINT;
   static constexpr int NC = 0;  // leading constants c[] that products use
   static constexpr int NX = 2, NU = 1, NZ = 3;

@@ -408,15 +408,19 @@ __device__ __forceinline__ void store_nz(const NodeArgs<M>& a, double* out, int6
 }
 
 // The classes of plain products that a kernel does on the integer pipes (soft_mul.cuh) in a large
-// launch (IP; chosen by soft_launch): where the FP64 pipe bounds it.  Not in the kernels near the HBM
+// launch (IP; chosen by large_launch): where the FP64 pipe bounds it.  Not in the kernels near the HBM
 // rate, which the extra instructions and registers slow down (Van der Pol J + H 23.9 us at N = 1e6, its
 // gradient 10.5 -> 12.3 us with them), nor for the double integrator, whose products are its cost's alone.
 template <class M, unsigned OUT, bool IP>
 constexpr unsigned soft_kernel() { return IP ? M::template SOFT<OUT> : 0u; }
 
 // Resident CTAs per SM that a kernel's registers are capped for (0: the allocator's own choice).
-template <class M, unsigned OUT, bool IP, bool EULER = false>
-constexpr int min_ctas() { return soft_kernel<M, OUT, IP>() ? M::template CTAS<OUT> : EULER ? M::template CTAS_EULER<OUT> : M::template CTAS_FP64<OUT>; }
+// (The two-warp CTAs of small launches may take every register they ask for.)
+template <class M, int TILE, unsigned OUT, bool IP, bool EULER = false>
+constexpr int min_ctas() {
+  if (soft_kernel<M, OUT, IP>()) return M::template CTAS<OUT>;
+  return TILE == TILE_SMALL ? 1 : EULER ? M::template CTAS_EULER<OUT> : M::template CTAS_FP64<OUT>;
+}
 
 // The inputs of a node's work that its products multiply (see soft_mul.cuh): the node's variables,
 // the multipliers of the rows with a Hessian, the directions.  High words only; the work's own
@@ -458,6 +462,22 @@ __device__ __forceinline__ bool soft_euler(const NodeArgs<M>& a, const double* y
     if (W) ok &= soft_input(w + a.nb + (int64_t)k * a.N + j);
   }
   return ok;
+}
+
+// Starts the loads that a node's work makes late (its multipliers and directions) before the first
+// wait: a lone warp would otherwise sit through each of them in turn.
+__device__ __forceinline__ void prefetch(const double* p) { asm volatile("prefetch.global.L1 [%0];" :: "l"(p)); }
+template <class M, bool Y, bool V, bool W>
+__device__ __forceinline__ void prefetch_node(const NodeArgs<M>& a, const double* y, const double* v, const double* w, int64_t j) {
+  const int64_t jr = min(j, a.N - 1);
+#pragma unroll
+  for (int k = 0; k < M::NX; ++k) {
+    const int64_t row = a.nb + (int64_t)k * a.N + jr;
+    if (V && (k % 4 == 0 || k == M::NX - 1)) prefetch(v + M::NX * j + k);
+    if (Y && M::HK(k)) prefetch(y + row);
+    if (W) prefetch(w + row);
+  }
+  if (V) prefetch(v + a.uoff + M::NU * j);
 }
 
 // Runs work(K) for the lanes with `act`, with the products of SoftConst where the warp's inputs
@@ -520,6 +540,9 @@ __device__ __forceinline__ void node_eval_tile(const NodeArgs<M>& a, const Model
     bool ok = false;
     if constexpr (SOFT != 0) {
       if (K0.soft && act) ok = soft_node<M, NEEDH, (WJV || WHV), WJTV>(a, a.y, a.v, a.wv, j);
+    }
+    if constexpr (TILE == TILE_SMALL) {
+      if (act) prefetch_node<M, NEEDH, (WJV || WHV), WJTV>(a, a.y, a.v, a.wv, j);
     }
     with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
       constexpr HTmpl<M> HT{};   // (not captured: a captured table lives in local memory)
@@ -724,7 +747,7 @@ __device__ __forceinline__ void node_eval_kernel_body(const NodeArgs<M>& a) {
 }
 
 template <class M, int TILE, int NPT, unsigned OUT, bool PAR, bool IP>
-__global__ void __launch_bounds__(TILE, min_ctas<M, OUT, IP>()) k_node_eval(const __grid_constant__ NodeArgs<M> a) {
+__global__ void __launch_bounds__(TILE, min_ctas<M, TILE, OUT, IP>()) k_node_eval(const __grid_constant__ NodeArgs<M> a) {
   node_eval_kernel_body<M, TILE, NPT, OUT, PAR, IP>(a);
 }
 
@@ -734,7 +757,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, OUT, IP>()) k_node_eval(cons
 // Same overlapping tiles as the evaluation; the right-node term comes from lane+1.
 // ======================================================================================
 template <class M, int TILE, bool PDIR, bool PAR, bool IP>
-__global__ void __launch_bounds__(TILE, min_ctas<M, O_JV, IP>()) k_node_jprod(const __grid_constant__ NodeArgs<M> a) {
+__global__ void __launch_bounds__(TILE, min_ctas<M, TILE, O_JV, IP>()) k_node_jprod(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   constexpr unsigned SOFT = soft_kernel<M, O_JV, IP>();
@@ -803,7 +826,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, O_JV, IP>()) k_node_jprod(co
 // parameter i < M::NP (mdp = -hh df/dp; one deterministic reduction per parameter).
 // ======================================================================================
 template <class M, int TILE, bool DPAR, bool PAR, bool IP>
-__global__ void __launch_bounds__(TILE, min_ctas<M, O_JTV, IP>()) k_node_jtprod(const __grid_constant__ NodeArgs<M> a) {
+__global__ void __launch_bounds__(TILE, min_ctas<M, TILE, O_JTV, IP>()) k_node_jtprod(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   constexpr int NP = M::NP, NPA = (NP > 0) ? NP : 1;
@@ -866,7 +889,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, O_JTV, IP>()) k_node_jtprod(
 // (-hh d2 f_k / dmu dz)(z_j), and reduces sum_j m_j . v_{z_j} into *dmu.
 // ======================================================================================
 template <class M, int TILE, bool MIX, bool PAR, bool IP>
-__global__ void __launch_bounds__(TILE, min_ctas<M, O_HV, IP>()) k_node_hprod(const __grid_constant__ NodeArgs<M> a) {
+__global__ void __launch_bounds__(TILE, min_ctas<M, TILE, O_HV, IP>()) k_node_hprod(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   constexpr unsigned SOFT = soft_kernel<M, O_HV, IP && !MIX>();
@@ -928,7 +951,7 @@ void fill_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   a.has_final = h->has_final ? 1 : 0;
   a.has_ref = h->has_ref ? 1 : 0;
   M::host_consts(h->params.data(), h->hh, a.K);
-  a.K.many = soft_launch(h->N + 1, h->num_sms);
+  a.K.many = large_launch(h->N + 1, h->num_sms);
   a.K.soft = a.K.many && soft_consts(a.K, M::NC);
   for (int v = 0; v < M::NZ; ++v) {
     const double w = v < M::NX ? h->q[v] : h->r[v - M::NX];
@@ -951,6 +974,10 @@ void fill_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   for (int k = 0; k < M::NX; ++k) a.trk[k] = -1;
   for (int i = 0; i < h->ntrk; ++i) a.trk[h->trk_comp[i]] = (int8_t)i;
 }
+
+// Tiles that large launches use (the quadrotor's products have tiles of TILE_SMALL in every launch).
+template <class M, int TILE>
+constexpr bool ip_tile() { return TILE != TILE_SMALL || TILE == M::PROD_TILE; }
 
 // Whether the launch takes the integer-product instance of its kernel (the device reads the parameters
 // itself with PAR, and tests the constants made of them there).
@@ -985,7 +1012,7 @@ template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
 ocp_status launch_eval_k(ocp* h, const EvalCall& c, cudaStream_t s) {
   NodeArgs<M> a;
   fill_args<M>(h, c.sigma, a);
-  if constexpr (M::template SOFT<OUT> != 0) {
+  if constexpr (ip_tile<M, TILE>() && M::template SOFT<OUT> != 0) {
     if (soft_choice<M, OUT, PAR>(a)) return launch_eval_ip<M, TILE, NPT, OUT, PAR, true>(h, c, a, s);
   }
   return launch_eval_ip<M, TILE, NPT, OUT, PAR, false>(h, c, a, s);
@@ -1028,7 +1055,7 @@ __host__ __device__ constexpr int euler_off(int k) {
 }
 
 template <class M, int TILE, unsigned OUT, bool PAR, bool IP>
-__global__ void __launch_bounds__(TILE, min_ctas<M, OUT, IP, true>()) k_euler(const __grid_constant__ NodeArgs<M> a) {
+__global__ void __launch_bounds__(TILE, min_ctas<M, TILE, OUT, IP, true>()) k_euler(const __grid_constant__ NodeArgs<M> a) {
   constexpr int NX = M::NX, NZ = M::NZ;
   constexpr bool WF = OUT & O_F, WC = OUT & O_C, WG = OUT & O_G, WJ = OUT & O_J, WH = OUT & O_H;
   constexpr bool WJV = OUT & O_JV, WJTV = OUT & O_JTV, WHV = OUT & O_HV;
@@ -1210,7 +1237,7 @@ ocp_status launch_euler_ip(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
 
 template <class M, int TILE, unsigned OUT, bool PAR>
 ocp_status launch_euler_k(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
-  if constexpr (M::template SOFT<OUT> != 0) {
+  if constexpr (ip_tile<M, TILE>() && M::template SOFT<OUT> != 0) {
     if (soft_choice<M, OUT, PAR>(a)) return launch_euler_ip<M, TILE, OUT, PAR, true>(h, a, s);
   }
   return launch_euler_ip<M, TILE, OUT, PAR, false>(h, a, s);
@@ -1273,7 +1300,7 @@ ocp_status euler_prod_dispatch(ocp* h, const ProdCall& c, cudaStream_t s) {
 }
 
 template <class M, int TILE>
-ocp_status node_eval_dispatch(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
+ocp_status node_eval_tiles(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
   if (!M::HAS_DPARAM && h->p0_dev && out != O_C) return set_err(h, OCP_EMODEL, "device parameters: the constraints only");
   if (h->scheme == OCP_SCHEME_EULER) return euler_eval_dispatch<M, TILE>(h, out, c, s);
   switch (out) {
@@ -1316,14 +1343,14 @@ template <class M, int TILE, bool PAR>
 cudaError_t node_prod_launch(ocp* h, const ProdCall& c, const NodeArgs<M>& a, cudaStream_t s) {
   static_assert((M::template SOFT<O_JV> != 0) == (M::template SOFT<O_JTV> != 0) &&
                 (M::template SOFT<O_JV> != 0) == (M::template SOFT<O_HV> != 0), "the products choose alike");
-  if constexpr (M::template SOFT<O_JV> != 0) {
+  if constexpr (ip_tile<M, TILE>() && M::template SOFT<O_JV> != 0) {
     if (soft_choice<M, O_JV, PAR>(a)) return node_prod_launch_ip<M, TILE, PAR, true>(h, c, a, s);
   }
   return node_prod_launch_ip<M, TILE, PAR, false>(h, c, a, s);
 }
 
 template <class M, int TILE>
-ocp_status node_prod_dispatch(ocp* h, const ProdCall& c, cudaStream_t s) {
+ocp_status node_prod_tiles(ocp* h, const ProdCall& c, cudaStream_t s) {
   if (h->scheme == OCP_SCHEME_EULER) return euler_prod_dispatch<M, TILE>(h, c, s);
   NodeArgs<M> a;
   fill_args<M>(h, c.sigma, a);
@@ -1341,6 +1368,17 @@ ocp_status node_prod_dispatch(ocp* h, const ProdCall& c, cudaStream_t s) {
     e = node_prod_launch<M, TILE, false>(h, c, a, s);
   }
   return cuda_err(h, e, "node product launch");
+}
+
+// One tile size for every call of a handle: outputs that sum over tiles are the same in all of them.
+template <class M, int TILE>
+ocp_status node_eval_dispatch(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
+  return small_launch(h->N + 1, h->num_sms) ? node_eval_tiles<M, TILE_SMALL>(h, out, c, s)
+                                            : node_eval_tiles<M, TILE>(h, out, c, s);
+}
+template <class M, int TILE>
+ocp_status node_prod_dispatch(ocp* h, const ProdCall& c, cudaStream_t s) {
+  return small_launch(h->N + 1, h->num_sms) ? node_prod_tiles<M, TILE_SMALL>(h, c, s) : node_prod_tiles<M, TILE>(h, c, s);
 }
 
 }  // namespace ocpg

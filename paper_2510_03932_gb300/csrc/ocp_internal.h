@@ -163,6 +163,18 @@ cudaError_t dev_upload(void* dst, const void* src, size_t bytes);
 bool fault_dims();      // the armed 'dims' fault fires here (once)
 bool take_injected();   // whether the last failure on this thread was an injected one (clears it)
 ocp_status cuda_err(ocp* h, cudaError_t e, const char* what);
+// Large launches: those with at least two warps of nodes per SM sub-partition.  There the FP64 pipe is
+// saturated, and integer products (soft_mul.cuh) pay; below, one warp's own chain of FP64
+// instructions is what takes the time, 64 cycles each whatever they depend on, and an integer product's 34
+// dependent instructions take it longer (evaluation, N = 8000: Van der Pol 8.9 us without and 10.2 with
+// them, Goddard 12.8 and 14.6; N = 30000: 8.8 and 9.6, cart-pole 14.9 and 14.7; N = 1e5: 13.5 and 12.7, cart-pole
+// 31.1 and 25.0, Goddard 27.1 and 22.9).
+// Small launches: those with at most one warp per sub-partition.  CTAs of two warps (TILE_SMALL), with
+// all the registers they ask for and their late loads prefetched, give every warp a sub-partition of its own and few
+// values to sum (step, N = 8000: Van der Pol 11.0 -> 9.1 us, Goddard 21.0 -> 15.0, quadrotor 33.5 -> 25.1); with
+// more nodes they only make more CTAs and partial sums (N = 30000: Van der Pol 10.9 -> 11.9).
+inline bool large_launch(int64_t nodes, int num_sms) { return nodes >= (int64_t)256 * num_sms; }
+inline bool small_launch(int64_t nodes, int num_sms) { return nodes <= (int64_t)128 * num_sms; }
 int occupancy_grid(ocp* h, const void* kernel, int threads, size_t smem, int64_t work_tiles);
 
 // Host pattern compiler.
