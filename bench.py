@@ -110,7 +110,7 @@ KERNEL_SOURCES = {
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
 FP64_OPS_SRC = {"vdp": "647193dc2255", "vdp:euler": "647193dc2255", "cartpole": "88dcfb14a118",
-                "quadrotor": "3670848eaedf", "goddard": "0f8e124215e2", "heat64": "e541a33ddbba"}
+                "quadrotor": "3670848eaedf", "goddard": "0f8e124215e2", "heat64": "b4ff11c40444"}
 
 
 def kernel_source_tag(key):

@@ -549,16 +549,18 @@ ocp_status ocp_eval_step(ocp_t* h, const double* x, const double* y, double sigm
   NEED(x); NEED(y); NEED(vn); NEED(vm); NEED(f); NEED(cv); NEED(g); NEED(jvals); NEED(hvals);
   NEED(Jv); NEED(Jtv); NEED(Hv);
   if (h->model == OCP_MODEL_HEAT1D) {
-    // the heat model runs two kernels in sequence: the evaluation, and Jv, J^T w and H v in one
-    // launch; then the products' path and boundary terms in one launch (each array's own
-    // operations in the order of the separate calls: the same bits)
-    ocp_status st = ocp_eval_all(h, x, y, sigma, f, cv, g, jvals, hvals, stream);
+    // the heat model runs two kernels: the evaluation, and Jv, J^T w and H v in one launch; then
+    // the products' path and boundary terms in one launch (each array's own operations in the
+    // order of the separate calls: the same bits)
+    EvalCall e = full_call(h);
+    e.x = x; e.y = y; e.sigma = sigma; e.f = f; e.c = cv; e.g = g; e.jv = jvals; e.hv = hvals;
+    ocp_status st = dispatch_eval(h, O_ALL, e, stream);
     ProdCall a, b, c;
     a.kind = P_JPROD; a.x = x; a.v = vn; a.out = Jv;
     b.kind = P_JTPROD; b.x = x; b.v = vm; b.out = Jtv;
     c.kind = P_HPROD; c.x = x; c.y = y; c.sigma = sigma; c.v = vn; c.out = Hv;
     cudaStream_t s = (cudaStream_t)stream;
-    if (st == OCP_OK) st = heat_prod3(h, a, b, c, s);
+    if (st == OCP_OK) st = heat_prod3(h, a, b, c, heat_step_overlaps(h, e, vn, vm, Jv, Jtv, Hv), s);
     return st == OCP_OK ? extra_prod3(h, a, b, c, s) : st;
   }
   EvalCall c = full_call(h);

@@ -229,8 +229,12 @@ ocp_status goddard_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s)
 ocp_status goddard_prod(ocp* h, const ProdCall& c, cudaStream_t s);
 ocp_status heat_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s);
 ocp_status heat_prod(ocp* h, const ProdCall& c, cudaStream_t s);
-// The heat model's Jv (jp), J^T w (jt) and H v (hp) in one launch.
-ocp_status heat_prod3(ocp* h, const ProdCall& jp, const ProdCall& jt, const ProdCall& hp, cudaStream_t s);
+// The heat model's Jv (jp), J^T w (jt) and H v (hp) in one launch; after_eval: the launch before it
+// is the evaluation at the same point, and it may overlap its end.
+bool heat_step_overlaps(const ocp* h, const EvalCall& e, const double* vn, const double* vm, const double* Jv,
+                        const double* Jtv, const double* Hv);
+ocp_status heat_prod3(ocp* h, const ProdCall& jp, const ProdCall& jt, const ProdCall& hp, bool after_eval,
+                      cudaStream_t s);
 
 struct EvalCall;
 ocp_status dispatch_eval(ocp* h, unsigned out, const EvalCall& c, void* stream);
