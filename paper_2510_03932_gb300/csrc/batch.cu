@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(TILE, batch_ctas<M, TILE, IP>()) k_batch_eval(
   __shared__ long long s_tile;
   __shared__ int s_inst, s_fin;
   static_assert(sizeof(NodeArgs<M>) % 8 == 0, "argument block is copied in 8-byte words");
+  start_follow_on();
   for (;;) {
     // dynamic tile scheduling: results do not depend on which CTA takes which tile
     if (threadIdx.x == 0) s_tile = (long long)atomicAdd(b.work, 1ull);
@@ -327,8 +328,7 @@ static ocp_status batch_launch(ocp_batch* b, const double* x, const double* y, d
   const void* kern = kernel_for<M>(b->threads, b->npt, b->many);
   if (!kern) return berr(b, OCP_EINVAL, "configuration not provided for this model");
   void* args[] = {&a};
-  cudaLaunchKernel(kern, dim3(grid), dim3(b->threads), args, sm, s);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_args(true, kern, grid, b->threads, sm, s, args);
   if (e != cudaSuccess) return berr(b, OCP_ECUDA, std::string("batch launch: ") + cudaGetErrorString(e));
   return OCP_OK;
 }

@@ -554,13 +554,15 @@ ocp_status ocp_eval_step(ocp_t* h, const double* x, const double* y, double sigm
     // order of the separate calls: the same bits)
     EvalCall e = full_call(h);
     e.x = x; e.y = y; e.sigma = sigma; e.f = f; e.c = cv; e.g = g; e.jv = jvals; e.hv = hvals;
+    const bool beside = heat_step_overlaps(h, e, vn, vm, Jv, Jtv, Hv);
+    e.products_beside = beside;   // (the products start on the inputs: what wrote them has to have ended)
     ocp_status st = dispatch_eval(h, O_ALL, e, stream);
     ProdCall a, b, c;
     a.kind = P_JPROD; a.x = x; a.v = vn; a.out = Jv;
     b.kind = P_JTPROD; b.x = x; b.v = vm; b.out = Jtv;
     c.kind = P_HPROD; c.x = x; c.y = y; c.sigma = sigma; c.v = vn; c.out = Hv;
     cudaStream_t s = (cudaStream_t)stream;
-    if (st == OCP_OK) st = heat_prod3(h, a, b, c, heat_step_overlaps(h, e, vn, vm, Jv, Jtv, Hv), s);
+    if (st == OCP_OK) st = heat_prod3(h, a, b, c, beside, s);
     return st == OCP_OK ? extra_prod3(h, a, b, c, s) : st;
   }
   EvalCall c = full_call(h);

@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "follow_on.cuh"
 #include "ocp_internal.h"
 
 namespace ocpg {
@@ -231,6 +232,7 @@ __device__ __forceinline__ void end_block(const ExtraArgs& a) {
 
 template <bool WC, bool WJ, bool WH, bool WJV, bool WJTV, bool WHV>
 __global__ void __launch_bounds__(EX_THREADS) k_extra(const __grid_constant__ ExtraArgs a) {
+  start_follow_on();
   if (a.ends && blockIdx.x == 0) {
     end_block<WC, WJ, WH, WJV, WJTV, WHV>(a);
     return;
@@ -273,7 +275,8 @@ static ocp_status extra_launch(ocp* h, ExtraArgs& a, unsigned m, int64_t B, int6
   int64_t blocks = n > 0 ? std::min<int64_t>((n + EX_THREADS - 1) / EX_THREADS, (int64_t)h->num_sms * 8) : 0;
   blocks += a.ends;
   if (blocks < 1) return OCP_OK;
-  auto go = [&](auto kern) { kern<<<(int)blocks, EX_THREADS, 0, s>>>(a); };
+  cudaError_t e = cudaSuccess;
+  auto go = [&](auto kern) { e = launch(true, kern, blocks, EX_THREADS, 0, s, a); };
   switch (m) {
     case 0:          // f and g alone
     case O_C: go(k_extra<true, false, false, false, false, false>); break;
@@ -289,7 +292,7 @@ static ocp_status extra_launch(ocp* h, ExtraArgs& a, unsigned m, int64_t B, int6
     case O_JV | O_JTV | O_HV: go(k_extra<false, false, false, true, true, true>); break;
     default: go(k_extra<true, true, true, true, true, true>); break;   // the fused step: every output
   }
-  return cuda_err(h, cudaGetLastError(), "path and boundary terms launch");
+  return cuda_err(h, e, "path and boundary terms launch");
 }
 
 static bool any_extra(const ocp* h) { return h->pat.npath > 0 || h->pat.nbin > 0 || h->has_bol; }

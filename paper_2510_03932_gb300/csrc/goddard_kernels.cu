@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(GT, god_ctas<OUT, IP, GT>()) k_god(const __gri
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int64_t N = a.N;
   __shared__ double sHH;
+  start_follow_on();
   double hh = a.hh_fixed;
   if (FREE) {  // hh = tf / (2N): one division per CTA (a per-thread division costs every node)
     if (t == 0) sHH = (__ldg(a.x + a.tau) / (double)N) * 0.5;
@@ -486,10 +487,9 @@ static cudaError_t god_launch(const GodArgs& a, cudaStream_t s) {
   const int64_t tiles = a.ntiles - a.tile0;
   const int grid = (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff);
   constexpr bool DYN = (OUT & (O_C | O_J | O_H | O_JV | O_JTV | O_HV)) != 0;   // the dynamics' products
-  if (a.many) k_god<OUT, FREE, DYN, GOD_TILE><<<grid, GOD_TILE, smem(GOD_TILE), s>>>(a);  // (G_DP, G_PAR bits in OUT)
-  else if (!a.small) k_god<OUT, FREE, false, GOD_TILE><<<grid, GOD_TILE, smem(GOD_TILE), s>>>(a);
-  else k_god<OUT, FREE, false, TILE_SMALL><<<grid, TILE_SMALL, smem(TILE_SMALL), s>>>(a);
-  return cudaGetLastError();
+  if (a.many) return launch(true, k_god<OUT, FREE, DYN, GOD_TILE>, grid, GOD_TILE, smem(GOD_TILE), s, a);  // (G_DP, G_PAR bits in OUT)
+  if (!a.small) return launch(true, k_god<OUT, FREE, false, GOD_TILE>, grid, GOD_TILE, smem(GOD_TILE), s, a);
+  return launch(true, k_god<OUT, FREE, false, TILE_SMALL>, grid, TILE_SMALL, smem(TILE_SMALL), s, a);
 }
 
 template <unsigned OUT>

@@ -59,6 +59,7 @@ struct HeatArgs {
   double cq_in[HEAT_MAXC + 1], cq_end[HEAT_MAXC + 1];
   double gq_in[HEAT_MAXC + 1], gq_end[HEAT_MAXC + 1];
   double ref[HEAT_MAXC + 1];
+  int beside_eval;          // the fused step: the products run beside the evaluation's end
 };
 
 // Doubles of the first shared-memory region of k_heat_eval: the staged states (32 rows of n+1),
@@ -218,7 +219,8 @@ __global__ void __launch_bounds__(32 * W, (OUT & O_C) ? (W > 1 ? 40 / W : 32) : 
   const bool WF = CF && a.f, WC = CC && a.c, WG = CG && a.g, WJ = CJ && a.jv, WH = CH && a.hv;
   constexpr int THREADS = 32 * W;
   extern __shared__ __align__(16) double sm[];
-  if (OUT == O_ALL) let_next_start();   // (the fused step's products: heat_step_overlaps)
+  start_follow_on();
+  if (OUT == O_ALL && a.beside_eval) let_next_start();   // (the fused step's products: heat_step_overlaps)
   const int n = a.n, ld = n + 1;
   // shared memory: states, then only the staging buffers this variant needs.  The gradient
   // is stored straight from the cell loop (a lane's eight cells of a group fill whole 32-byte
@@ -374,6 +376,7 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_jh(const __grid_constan
   __shared__ double sY[HJ_CELLS * HT_LANES];
   const int n = a.n;
   const int t = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  start_follow_on();
   const ModelConst K0 = heat_consts<IP>(a);
   constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
   const int64_t units = a.ntiles * cgroups;
@@ -447,6 +450,7 @@ __global__ void __launch_bounds__(32 * W, W > 1 ? 40 / W : 32) k_heat_hprod(cons
   double* sX = sm;
   double* sV = sX + HT_LANES * ld;  // the direction
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  start_follow_on();
   const ModelConst K0 = heat_consts<IP>(a);
   constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
@@ -531,6 +535,7 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
   double* const wout = ALL3 ? a.out2 : a.out;
   const int n = a.n;
   const int t = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (!ALL3 || !a.beside_eval) start_follow_on();
   const ModelConst K0 = heat_consts<IP>(a);
   constexpr unsigned SOFT = IP ? MUL_ALL : 0u;
   const int64_t units = a.ntiles * cgroups;
@@ -646,7 +651,7 @@ __global__ void __launch_bounds__(HJ_THREADS, 18) k_heat_prod_unit(const __grid_
     }
     __syncthreads();
   }
-  if (ALL3) wait_for_previous();   // (they read nothing that the evaluation writes: heat_step_overlaps)
+  if (ALL3 && a.beside_eval) wait_for_previous();   // (they read nothing that the evaluation writes: heat_step_overlaps)
 }
 
 // ======================================================================================
@@ -708,6 +713,7 @@ static ocp_status heat_eval_t(ocp* h, const EvalCall& c, cudaStream_t s) {
   HeatArgs a;
   heat_fill(h, c.sigma, a);
   a.x = c.x; a.y = c.y; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
+  a.beside_eval = c.products_beside;
   a.B = c.B; a.E = c.E;
   const int64_t nodes = c.E - c.B;
   a.ntiles = (nodes + (HT_LANES - 2)) / (HT_LANES - 1);
@@ -721,8 +727,7 @@ static ocp_status heat_eval_t(ocp* h, const EvalCall& c, cudaStream_t s) {
     auto kern = (MUL && a.soft) ? k_heat_eval<OUT, MUL, W> : k_heat_eval<OUT, false, W>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<occupancy_grid(h, (const void*)kern, 32 * W, smem, a.ntiles), 32 * W, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch(!c.products_beside, kern, occupancy_grid(h, (const void*)kern, 32 * W, smem, a.ntiles), 32 * W, smem, s, a);
   };
   return cuda_err(h, with_warps(heat_warps(h->nx, a.ntiles, h->num_sms), go), "k_heat_eval launch");
 }
@@ -741,8 +746,7 @@ static ocp_status heat_jh_t(ocp* h, const EvalCall& c, cudaStream_t s) {
   auto kern = a.soft ? k_heat_jh<OUT, true> : k_heat_jh<OUT, false>;
   const int grid = occupancy_grid(h, (const void*)kern, HJ_THREADS, 0, a.ntiles * cgroups);
   if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
-  kern<<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
-  return cuda_err(h, cudaGetLastError(), "k_heat_jh launch");
+  return cuda_err(h, launch(true, kern, grid, HJ_THREADS, 0, s, a, cgroups), "k_heat_jh launch");
 }
 
 ocp_status heat_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
@@ -795,7 +799,8 @@ ocp_status heat_prod3(ocp* h, const ProdCall& jp, const ProdCall& jt, const Prod
   auto k = a.soft ? k_heat_prod_unit<HP_ALL3, true> : k_heat_prod_unit<HP_ALL3, false>;
   const int grid = occupancy_grid(h, (const void*)k, HJ_THREADS, 0, a.ntiles * cgroups);
   if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
-  return cuda_err(h, launch(after_eval, k, grid, HJ_THREADS, 0, s, a, cgroups), "heat product launch");
+  a.beside_eval = after_eval;
+  return cuda_err(h, launch(true, k, grid, HJ_THREADS, 0, s, a, cgroups), "heat product launch");
 }
 
 ocp_status heat_prod(ocp* h, const ProdCall& c, cudaStream_t s) {
@@ -810,8 +815,7 @@ ocp_status heat_prod(ocp* h, const ProdCall& c, cudaStream_t s) {
       auto k = a.soft ? k_heat_hprod<true, W> : k_heat_hprod<false, W>;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
-      k<<<occupancy_grid(h, (const void*)k, 32 * W, smem, a.ntiles), 32 * W, smem, s>>>(a);
-      return cudaGetLastError();
+      return launch(true, k, occupancy_grid(h, (const void*)k, 32 * W, smem, a.ntiles), 32 * W, smem, s, a);
     };
     return cuda_err(h, with_warps(heat_warps(h->nx, a.ntiles, h->num_sms), go), "heat product launch");
   }
@@ -823,8 +827,7 @@ ocp_status heat_prod(ocp* h, const ProdCall& c, cudaStream_t s) {
                               : a.soft ? k_heat_prod_unit<HP_JPROD, true> : k_heat_prod_unit<HP_JPROD, false>;
   const int grid = occupancy_grid(h, (const void*)k, HJ_THREADS, 0, a.ntiles * cgroups);
   if (grid <= 0) return set_err(h, OCP_ECUDA, "occupancy query failed");
-  k<<<grid, HJ_THREADS, 0, s>>>(a, cgroups);
-  return cuda_err(h, cudaGetLastError(), "heat product launch");
+  return cuda_err(h, launch(true, k, grid, HJ_THREADS, 0, s, a, cgroups), "heat product launch");
 }
 
 }  // namespace ocpg

@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "follow_on.cuh"
 #include "ocp_internal.h"
 
 namespace ocpg {
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(KKT_THREADS) k_kkt_values(const __grid_constan
     }
     __syncthreads();
   }
+  start_follow_on();   // (the plan read so far is older than any launch)
   switch (R.kind) {  // (CTA-uniform)
     case KR_X: kkt_block<KR_X>(a, R, s0, s_src, s_a, s_diag); break;
     case KR_U: kkt_block<KR_U>(a, R, s0, s_src, s_a, s_diag); break;
@@ -346,8 +348,7 @@ ocp_status ocp_kkt_values(ocp_t* h, const double* hvals, const double* jvals, co
   KktArgs a;
   if (kkt_fill(h, a) != OCP_OK) return set_err(h, OCP_EDIM, "KKT matrix too large for the int32 interface");
   a.hv = hvals; a.jv = jvals; a.sx = sigma_x; a.out = kvals; a.dw = delta_w; a.dc = delta_c;
-  k_kkt_values<<<a.nblocks, KKT_THREADS, 0, (cudaStream_t)stream>>>(a);
-  return cuda_err(h, cudaGetLastError(), "KKT values launch");
+  return cuda_err(h, launch(true, k_kkt_values, a.nblocks, KKT_THREADS, 0, (cudaStream_t)stream, a), "KKT values launch");
 }
 
 }  // extern "C"

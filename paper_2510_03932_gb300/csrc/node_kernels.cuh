@@ -24,6 +24,7 @@
 #include <stdint.h>
 
 #include "model_base.cuh"
+#include "follow_on.cuh"
 #include "ocp_internal.h"
 
 namespace ocpg {
@@ -740,6 +741,7 @@ __device__ __forceinline__ void node_eval_kernel_body(const NodeArgs<M>& a) {
   constexpr bool WF = OUT & O_F;
   extern __shared__ __align__(16) double sm[];
   __shared__ double sEdge[2 * (TILE / 32 + 1) * M::NX];
+  start_follow_on();
   const ModelConst K = launch_consts<M, PAR>(a);
   for (int64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x)
     node_eval_tile<M, TILE, NPT, OUT, IP>(a, K, tile, sm, sEdge, a.partials + tile);
@@ -763,6 +765,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, TILE, O_JV, IP>()) k_node_jp
   constexpr unsigned SOFT = soft_kernel<M, O_JV, IP>();
   __shared__ double sEdge[(TILE / 32 + 1) * NX];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  start_follow_on();
   const ModelConst K0 = launch_consts<M, PAR>(a);
   double pd = 0.0;
   if (PDIR) pd = a.pdir_dev ? __ldg(a.pdir_dev) : a.pdir;
@@ -832,6 +835,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, TILE, O_JTV, IP>()) k_node_j
   constexpr int NP = M::NP, NPA = (NP > 0) ? NP : 1;
   constexpr unsigned SOFT = soft_kernel<M, O_JTV, IP>();
   __shared__ double red[TILE * NPA];
+  start_follow_on();
   const ModelConst K0 = launch_consts<M, PAR>(a);
   const int64_t nchunks = (a.E - a.B + TILE - 1) / TILE;   // the nodes [B, E) in chunks of TILE
   for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
@@ -894,6 +898,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, TILE, O_HV, IP>()) k_node_hp
   constexpr int NHD = (M::NHD > 0) ? M::NHD : 1;
   constexpr unsigned SOFT = soft_kernel<M, O_HV, IP && !MIX>();
   __shared__ double red[TILE];
+  start_follow_on();
   const ModelConst K0 = launch_consts<M, PAR>(a);
   double ms = 0.0;
   if (MIX) ms = a.mixs ? __ldg(a.mixs) : 0.0;
@@ -1004,8 +1009,7 @@ ocp_status launch_eval_ip(ocp* h, const EvalCall& c, NodeArgs<M>& a, cudaStream_
     attr_done |= 1u << (h->device & 31);
   }
   const int grid = occupancy_grid(h, (const void*)kern, TILE, S::bytes, a.ntiles);
-  kern<<<grid, TILE, S::bytes, s>>>(a);
-  return cuda_err(h, cudaGetLastError(), "k_node_eval launch");
+  return cuda_err(h, launch(true, kern, grid, TILE, S::bytes, s, a), "k_node_eval launch");
 }
 
 template <class M, int TILE, int NPT, unsigned OUT, bool PAR>
@@ -1067,6 +1071,7 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, TILE, OUT, IP, true>()) k_eu
   const bool doH = sH || WHV;
   constexpr unsigned SOFT = soft_kernel<M, OUT, IP>();
   const int t = threadIdx.x;
+  start_follow_on();
   const ModelConst K0 = launch_consts<M, PAR>(a);
   const int64_t N = a.N;
   const int64_t xN = (int64_t)NX * N;  // first entry of X_N
@@ -1231,8 +1236,7 @@ ocp_status launch_euler_ip(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_err(h, e, "cudaFuncSetAttribute(euler)");
   }
-  kern<<<(int)a.ntiles, TILE, smem, s>>>(a);
-  return cuda_err(h, cudaGetLastError(), "k_euler launch");
+  return cuda_err(h, launch(true, kern, a.ntiles, TILE, smem, s, a), "k_euler launch");
 }
 
 template <class M, int TILE, unsigned OUT, bool PAR>
@@ -1317,9 +1321,10 @@ ocp_status node_eval_tiles(ocp* h, unsigned out, const EvalCall& c, cudaStream_t
 
 template <class M, int TILE, bool PAR, bool IP>
 cudaError_t node_prod_launch_ip(ocp* h, const ProdCall& c, const NodeArgs<M>& a, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
   auto go = [&](auto kern, int64_t units) {
     const int grid = occupancy_grid(h, (const void*)kern, TILE, 0, units);
-    kern<<<grid, TILE, 0, s>>>(a);
+    e = launch(true, kern, grid, TILE, 0, s, a);
   };
   // the parameter-direction and mixed terms of the double backward exist for the Van der Pol
   // model alone (the C-ABI rejects them for the others)
@@ -1336,7 +1341,7 @@ cudaError_t node_prod_launch_ip(ocp* h, const ProdCall& c, const NodeArgs<M>& a,
     if (VDP && c.mixw && c.mixs) go(k_node_hprod<M, TILE, VDP, PAR, false>, blocks);
     else go(k_node_hprod<M, TILE, false, PAR, IP>, blocks);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 template <class M, int TILE, bool PAR>

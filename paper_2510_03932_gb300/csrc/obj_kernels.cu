@@ -45,6 +45,7 @@ constexpr int OBJ_PER = 8, OBJ_CHUNK = OBJ_THREADS * OBJ_PER;
 
 __global__ void __launch_bounds__(OBJ_THREADS) k_obj_grad(const __grid_constant__ ObjArgs a, int64_t xblocks) {
   __shared__ double s_in[OBJ_MAXV], s_end[OBJ_MAXV];
+  start_follow_on();
   const double s = __ldg(a.s);
   for (int v = threadIdx.x; v < a.nx + a.nu; v += OBJ_THREADS) {
     s_in[v] = fma(s, a.gq_in[v], a.mz);
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(OBJ_THREADS) k_obj_grad(const __grid_constant_
 // out = s * Hess F v, dot = grad F . v
 __global__ void __launch_bounds__(OBJ_THREADS) k_obj_hvp(const __grid_constant__ ObjArgs a) {
   __shared__ double red[OBJ_THREADS];
+  start_follow_on();
   const double s = __ldg(a.s);
   const int nz = a.nx + a.nu;
   const int64_t nchunks = (a.N + OBJ_THREADS) / OBJ_THREADS;
@@ -144,15 +146,16 @@ ocp_status obj_launch(ocp* h, bool hvp, const double* x, const double* s, const 
     a.gq_end[v2] = h->h * w;
     a.ref[v2] = v2 < h->nx ? h->xref[v2] : h->uref[v2 - h->nx];
   }
+  cudaError_t e;
   if (hvp) {
     const int64_t nchunks = (h->N + OBJ_THREADS) / OBJ_THREADS;
-    k_obj_hvp<<<occupancy_grid(h, nullptr, OBJ_THREADS, 0, nchunks), OBJ_THREADS, 0, st>>>(a);
+    e = launch(true, k_obj_hvp, occupancy_grid(h, nullptr, OBJ_THREADS, 0, nchunks), OBJ_THREADS, 0, st, a);
   } else {
     auto blocks = [&](int w) { return ((int64_t)w * (h->N + 1) + OBJ_CHUNK - 1) / OBJ_CHUNK; };
     const int64_t xb = blocks(h->nx);
-    k_obj_grad<<<(int)(xb + blocks(h->nu)), OBJ_THREADS, 0, st>>>(a, xb);
+    e = launch(true, k_obj_grad, xb + blocks(h->nu), OBJ_THREADS, 0, st, a, xb);
   }
-  return cuda_err(h, cudaGetLastError(), "objective kernel launch");
+  return cuda_err(h, e, "objective kernel launch");
 }
 
 }  // namespace ocpg

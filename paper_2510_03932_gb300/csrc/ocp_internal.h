@@ -193,6 +193,7 @@ struct EvalCall {
   double *ojv = nullptr, *ojtv = nullptr, *ohv = nullptr;
   int64_t B = 0, E = 0;  // owned node range [B, E)
   bool range = false;    // f receives the partial sum of this range
+  bool products_beside = false;  // heat's fused step: launched in the ordinary way, the products beside its end
 };
 
 enum ProdKind { P_JPROD = 0, P_JTPROD = 1, P_HPROD = 2 };

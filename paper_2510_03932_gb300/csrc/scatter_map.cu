@@ -18,6 +18,7 @@
 #include <cstring>
 #include <vector>
 
+#include "follow_on.cuh"
 #include "ocp_internal.h"
 
 namespace ocpg {
@@ -276,6 +277,7 @@ static ocp_status map_ready(ocp* h, cudaStream_t s) {
 __global__ void __launch_bounds__(256) k_jtprod_coo(const int32_t* __restrict__ ptr, const int32_t* __restrict__ rows,
                                                     const int32_t* __restrict__ slots, const double* __restrict__ jv,
                                                     const double* __restrict__ w, double* out, int64_t ncols) {
+  start_follow_on();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncols; c += stride) {
     double acc = 0.0;
@@ -291,6 +293,7 @@ __global__ void __launch_bounds__(1024) k_jtprod_coo_long(const int32_t* __restr
                                                           const double* __restrict__ jv,
                                                           const double* __restrict__ w, double* out, int64_t c) {
   __shared__ double s[1024];
+  start_follow_on();
   const int32_t t0 = ptr[c], t1 = ptr[c + 1];
   double acc = 0.0;
   for (int32_t t = t0 + threadIdx.x; t < t1; t += 1024) acc = fma(jv[slots[t]], w[rows[t]], acc);
@@ -329,9 +332,10 @@ ocp_status ocp_jtprod_coo(ocp_t* h, const double* jvals, const double* w, double
   const ScatterMap* m = h->smap;
   const int64_t ncols = h->pat.n - h->pat.free_tf;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((ncols + 255) / 256, (int64_t)h->num_sms * 16));
-  k_jtprod_coo<<<grid, 256, 0, s>>>(m->ptr, m->rows, m->slots, jvals, w, Jtw, ncols);
-  if (h->pat.free_tf) k_jtprod_coo_long<<<1, 1024, 0, s>>>(m->ptr, m->rows, m->slots, jvals, w, Jtw, ncols);
-  return cuda_err(h, cudaGetLastError(), "k_jtprod_coo launch");
+  cudaError_t e = launch(true, k_jtprod_coo, grid, 256, 0, s, m->ptr, m->rows, m->slots, jvals, w, Jtw, ncols);
+  if (e == cudaSuccess && h->pat.free_tf)
+    e = launch(true, k_jtprod_coo_long, 1, 1024, 0, s, m->ptr, m->rows, m->slots, jvals, w, Jtw, ncols);
+  return cuda_err(h, e, "k_jtprod_coo launch");
 }
 
 }  // extern "C"
