@@ -139,6 +139,8 @@ class _Objective(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gF):
         (x,) = ctx.saved_tensors
+        if not torch.is_grad_enabled():
+            return None, ctx.H.eval_grad_scaled(x, gF.reshape(1).contiguous())
         return None, _ObjGrad.apply(ctx.H, x, gF.reshape(1))
 
 

@@ -188,13 +188,30 @@ def sum_ordered(parts, out, stream=None):
     return out
 
 
+_F64 = torch.float64
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _first_device():
+    global _device
+    d = torch.cuda.current_device()   # starts CUDA if it has to, and checks for a forked process
+    _device = getattr(torch._C, "_cuda_getDevice", _first_device)
+    return d
+
+
+def _forked():
+    global _device
+    _device = _first_device
+
+
+_device = _first_device
+os.register_at_fork(after_in_child=_forked)
 
 
 def _stream(stream):
     if stream is None:
         if _raw_stream is not None:   # the current stream's handle without a Stream object
-            return _raw_stream(torch.cuda.current_device())
+            return _raw_stream(_device())
         stream = torch.cuda.current_stream()
     return C.c_void_p(stream.cuda_stream)
 
@@ -206,7 +223,7 @@ def _check(st, h=None):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()   # (ctypes converts by the declared argument types)
 
 
 class OCP:
@@ -304,6 +321,9 @@ class OCP:
 
     # ---- argument checks --------------------------------------------------------------
     def _vec(self, t, size, name):
+        # (the calls on small problems are bound by this module: the good case is one test)
+        if t is not None and t.dtype is _F64 and t.is_cuda and t.is_contiguous() and t.numel() == size:
+            return t
         if t is None:
             raise ValueError("%s is required" % name)
         if t.dtype != torch.float64 or not t.is_cuda or not t.is_contiguous():
@@ -328,19 +348,25 @@ class OCP:
     def eval_obj(self, x, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         out = self._out(out, 1, "f")
-        _check(lib().eval_obj(self.h, _ptr(x), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.eval_obj(self.h, _ptr(x), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def eval_cons(self, x, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         out = self._out(out, self.m, "c")
-        _check(lib().eval_cons(self.h, _ptr(x), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.eval_cons(self.h, _ptr(x), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def eval_grad(self, x, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         out = self._out(out, self.n, "g")
-        _check(lib().eval_grad(self.h, _ptr(x), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.eval_grad(self.h, _ptr(x), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def jac_coo_structure(self, stream=None):
@@ -374,35 +400,45 @@ class OCP:
         if sigma_x is not None:
             sigma_x = self._vec(sigma_x, self.n, "sigma_x")
         out = self._out(out, self.kkt_nnz(), "kvals")
-        _check(lib().ocp_kkt_values(self.h, _ptr(hvals), _ptr(jvals), _ptr(sigma_x), float(delta_w), float(delta_c),
-                                    _ptr(out), _stream(stream)), self.h)
+        st = self._lib.ocp_kkt_values(self.h, _ptr(hvals), _ptr(jvals), _ptr(sigma_x), float(delta_w), float(delta_c),
+                                      _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def jac_coo_values(self, x, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         out = self._out(out, self.nnzj, "vals")
-        _check(lib().jac_coo_values(self.h, _ptr(x), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.jac_coo_values(self.h, _ptr(x), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def hess_coo_values(self, x, y, sigma, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         y = self._vec(y, self.m, "y")
         out = self._out(out, self.nnzh, "vals")
-        _check(lib().hess_coo_values(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.hess_coo_values(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def jprod(self, x, v, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         v = self._vec(v, self.n, "v")
         out = self._out(out, self.m, "Jv")
-        _check(lib().jprod(self.h, _ptr(x), _ptr(v), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.jprod(self.h, _ptr(x), _ptr(v), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def jtprod(self, x, v, out=None, stream=None):
         x = self._vec(x, self.n, "x")
         v = self._vec(v, self.m, "v")
         out = self._out(out, self.n, "Jtv")
-        _check(lib().jtprod(self.h, _ptr(x), _ptr(v), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.jtprod(self.h, _ptr(x), _ptr(v), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def hprod(self, x, y, sigma, v, out=None, stream=None):
@@ -410,7 +446,9 @@ class OCP:
         y = self._vec(y, self.m, "y")
         v = self._vec(v, self.n, "v")
         out = self._out(out, self.n, "Hv")
-        _check(lib().hprod(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(v), _ptr(out), _stream(stream)), self.h)
+        st = self._lib.hprod(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(v), _ptr(out), _stream(stream))
+        if st:
+            _check(st, self.h)
         return out
 
     def eval_all(self, x, y, sigma, f=None, c=None, g=None, jvals=None, hvals=None, stream=None, alloc=True):
@@ -421,8 +459,10 @@ class OCP:
         if alloc:
             f = self._out(f, 1, "f"); c = self._out(c, self.m, "c"); g = self._out(g, self.n, "g")
             jvals = self._out(jvals, self.nnzj, "jvals"); hvals = self._out(hvals, self.nnzh, "hvals")
-        _check(lib().ocp_eval_all(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(f), _ptr(c), _ptr(g), _ptr(jvals),
-                                  _ptr(hvals), _stream(stream)), self.h)
+        st = self._lib.ocp_eval_all(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(f), _ptr(c), _ptr(g), _ptr(jvals),
+                                    _ptr(hvals), _stream(stream))
+        if st:
+            _check(st, self.h)
         return f, c, g, jvals, hvals
 
     def eval_step(self, x, y, sigma, vn, vm, outs=None, stream=None):
@@ -433,8 +473,10 @@ class OCP:
             outs = (self._out(None, 1, "f"), self._out(None, self.m, "c"), self._out(None, self.n, "g"),
                     self._out(None, self.nnzj, "jvals"), self._out(None, self.nnzh, "hvals"),
                     self._out(None, self.m, "Jv"), self._out(None, self.n, "Jtv"), self._out(None, self.n, "Hv"))
-        _check(lib().ocp_eval_step(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(vn), _ptr(vm),
-                                   *[_ptr(t) for t in outs], _stream(stream)), self.h)
+        st = self._lib.ocp_eval_step(self.h, _ptr(x), _ptr(y), float(sigma), _ptr(vn), _ptr(vm),
+                                     *[_ptr(t) for t in outs], _stream(stream))
+        if st:
+            _check(st, self.h)
         return outs
 
     def eval_step_range(self, node_begin, node_end, x, y, sigma, vn, vm, outs, stream=None):
