@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(TILE, batch_ctas<M, TILE, IP>()) k_batch_eval(
     __syncthreads();
     if (threadIdx.x == 0) {
       sa.x = b.x + __ldg(b.xoff + i);
-      sa.y = b.y ? b.y + __ldg(b.coff + i) : nullptr;
+      sa.y = b.y ? b.y + __ldg(b.coff + i) : any_multipliers(sa.x, sa.nb);
       sa.f = b.f;
       sa.c = b.c ? b.c + __ldg(b.coff + i) : nullptr;
       sa.g = b.g ? b.g + __ldg(b.xoff + i) : nullptr;

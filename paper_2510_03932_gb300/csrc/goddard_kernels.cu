@@ -61,7 +61,8 @@ struct GodArgs {
   int many, small;                   // large_launch, small_launch
 };
 
-// The inputs of node j's work that its products multiply (see soft_mul.cuh).
+// The inputs of node j's work that its products multiply (see soft_mul.cuh); no multipliers when H is not
+// asked for.
 template <bool Y, bool YALL, bool V, bool W>
 __device__ __forceinline__ bool soft_god(const GodArgs& a, int64_t j) {
   const int64_t jl = max(j - 1, (int64_t)0), jr = min(j, a.N - 1);   // (as in soft_node)
@@ -72,7 +73,7 @@ __device__ __forceinline__ bool soft_god(const GodArgs& a, int64_t j) {
     ok &= soft_input(a.x + 3 * j + k);
     if (V) ok &= soft_input(a.vn + 3 * j + k);
     const int64_t row = a.nb + (int64_t)k * a.N;
-    if (Y && (YALL || k == 1)) ok &= soft_input(a.y + row + jl) & soft_input(a.y + row + jr);
+    if (Y && (YALL || k == 1) && a.y) ok &= soft_input(a.y + row + jl) & soft_input(a.y + row + jr);
     if (W) ok &= soft_input(a.vm + row + jl) & soft_input(a.vm + row + jr);
   }
   return ok;

@@ -453,13 +453,13 @@ __device__ __forceinline__ bool soft_node(const NodeArgs<M>& a, const double* y,
   return ok;
 }
 
-// The same for a node of the Euler scheme (its own rows' multipliers).
+// The same for a node of the Euler scheme (its own rows' multipliers; none when H is not asked for).
 template <class M, bool Y, bool V, bool W>
 __device__ __forceinline__ bool soft_euler(const NodeArgs<M>& a, const double* y, const double* v, const double* w, int64_t j) {
   bool ok = soft_node<M, false, V, false>(a, nullptr, v, nullptr, j);
 #pragma unroll
   for (int k = 0; k < M::NX; ++k) {
-    if (Y && M::HK(k)) ok &= soft_input(y + a.nb + (int64_t)k * a.N + j);
+    if (Y && M::HK(k) && y) ok &= soft_input(y + a.nb + (int64_t)k * a.N + j);
     if (W) ok &= soft_input(w + a.nb + (int64_t)k * a.N + j);
   }
   return ok;
@@ -980,6 +980,10 @@ void fill_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   for (int i = 0; i < h->ntrk; ++i) a.trk[h->trk_comp[i]] = (int8_t)i;
 }
 
+// The kernel of all outputs forms H whether it is stored or not.  For a caller without multipliers
+// (y = NULL, no H) it reads the rows nb + k N + j < nb + nx N of y from the states, which are in range.
+__host__ __device__ inline const double* any_multipliers(const double* x, int64_t nb) { return x - nb; }
+
 // Tiles that large launches use (the quadrotor's products have tiles of TILE_SMALL in every launch).
 template <class M, int TILE>
 constexpr bool ip_tile() { return TILE != TILE_SMALL || TILE == M::PROD_TILE; }
@@ -991,7 +995,8 @@ bool soft_choice(const NodeArgs<M>& a) { return M::template SOFT<OUT> != 0 && (P
 
 template <class M, int TILE, int NPT, unsigned OUT, bool PAR, bool IP>
 ocp_status launch_eval_ip(ocp* h, const EvalCall& c, NodeArgs<M>& a, cudaStream_t s) {
-  a.x = c.x; a.y = c.y; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
+  a.x = c.x; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
+  a.y = c.y ? c.y : any_multipliers(c.x, a.nb);
   a.v = c.vn; a.wv = c.vm; a.ojv = c.ojv; a.ojtv = c.ojtv; a.ohv = c.ohv;
   a.B = c.B; a.E = c.E;
   a.range = c.range ? 1 : 0;
