@@ -24,17 +24,17 @@ __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.
 constexpr unsigned FEW_CTAS = 76;   // half of the SMs: two such grids fit one CTA to an SM
 __device__ __forceinline__ void start_follow_on() {
   wait_for_previous();
-  if (gridDim.x <= FEW_CTAS) let_next_start();
+  if (gridDim.x * gridDim.y <= FEW_CTAS) let_next_start();
 }
 
 // The launch of `kernel`: beside the end of the launch before it, or in the ordinary way.
-inline cudaError_t launch_args(bool follow_on, const void* kernel, int64_t grid, int threads, size_t smem, cudaStream_t s,
+inline cudaError_t launch_args(bool follow_on, const void* kernel, dim3 grid, int threads, size_t smem, cudaStream_t s,
                                void** args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -45,7 +45,7 @@ inline cudaError_t launch_args(bool follow_on, const void* kernel, int64_t grid,
 }
 template <class T> struct Same { using type = T; };   // (arguments convert to the kernel's parameters)
 template <class... P>
-inline cudaError_t launch(bool follow_on, void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s,
+inline cudaError_t launch(bool follow_on, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
                           typename Same<P>::type... args) {
   void* p[] = {&args...};
   return launch_args(follow_on, (const void*)kernel, grid, threads, smem, s, p);

@@ -43,6 +43,7 @@ struct CartPole {
   template <unsigned OUT> static constexpr int CTAS_FP64 = OUT == O_G ? 6 : 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
   static constexpr int PROD_TILE = TILE_CARTPOLE;
+  static constexpr bool SPLIT = true;   // k_node_eval_split in the smallest launches
   static constexpr int EVAL_TILE = TILE_CARTPOLE;
   static constexpr int NC = 15;  // leading constants c[] that products use
   static constexpr int NX = 4, NU = 1, NZ = 5;

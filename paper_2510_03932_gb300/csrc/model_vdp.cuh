@@ -26,6 +26,7 @@ struct VdP {
   template <unsigned OUT> static constexpr int CTAS_FP64 = 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
   static constexpr int PROD_TILE = TILE_VDP;
+  static constexpr bool SPLIT = false;  // (a node's work is short)
   static constexpr int EVAL_TILE = TILE_VDP;
   static constexpr int NC = 3;  // leading constants c[] that products use
   static constexpr int NX = 2, NU = 1, NZ = 3;

@@ -753,6 +753,34 @@ __global__ void __launch_bounds__(TILE, min_ctas<M, TILE, OUT, IP>()) k_node_eva
   node_eval_kernel_body<M, TILE, NPT, OUT, PAR, IP>(a);
 }
 
+// The same for launches so small that most FP64 pipes would idle.  A warp of the fused kernels holds its
+// pipe for every instruction of every output (15 us of the quadrotor's step, 9 of its evaluation), so the
+// outputs go to groups of CTAs (blockIdx.y) on pipes of their own, which each form the dynamics for
+// themselves.  N = 1000: quadrotor step 22.4 -> 11.6 us, evaluation and KKT values 21.5 -> 16.4, cart-pole
+// step 10.5 -> 7.5, evaluation and KKT values 13.7 -> 12.1.
+constexpr unsigned split_group(int g) {
+  return g == 0 ? O_C | O_J : g == 1 ? O_F | O_G | O_H : g == 2 ? O_JV | O_JTV : O_HV;
+}
+template <class M, int TILE, unsigned OUT>
+__global__ void __launch_bounds__(TILE, 1) k_node_eval_split(const __grid_constant__ NodeArgs<M> a) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double sEdge[2 * (TILE / 32 + 1) * M::NX];
+  start_follow_on();
+  const ModelConst K = launch_consts<M, false>(a);
+  const int64_t tile = blockIdx.x;
+  auto group = [&](auto g) __attribute__((always_inline)) {
+    constexpr unsigned G = split_group(decltype(g)::value) & OUT;
+    if constexpr (G != 0) node_eval_tile<M, TILE, 1, G, false>(a, K, tile, sm, sEdge, a.partials + tile);
+    if (G & O_F && a.f) finish_tiles<TILE>(a.partials, a.ntiles, a.counter, a.f, 0.5, sm);
+  };
+  switch (blockIdx.y) {
+    case 0: if (a.c || a.jv) group(std::integral_constant<int, 0>{}); break;
+    case 1: if (a.f || a.g || a.hv) group(std::integral_constant<int, 1>{}); break;
+    case 2: group(std::integral_constant<int, 2>{}); break;
+    default: group(std::integral_constant<int, 3>{}); break;
+  }
+}
+
 // ======================================================================================
 // Jv.  Row (k,j) = (p_k(j) - v_{X_j,k}) + (p_k(j+1) + v_{X_{j+1},k}),  (B(j) + A(j+1)),
 // p_k(j) = -hh grad f_k(z_j) . v_{z_j}  (+ -hh df_k/dmu(z_j) * pdir for the parameter).
@@ -993,6 +1021,14 @@ constexpr bool ip_tile() { return TILE != TILE_SMALL || TILE == M::PROD_TILE; }
 template <class M, unsigned OUT, bool PAR>
 bool soft_choice(const NodeArgs<M>& a) { return M::template SOFT<OUT> != 0 && (PAR ? a.K.many : a.K.soft); }
 
+// Models and outputs with a split kernel, and the nodes per SM up to which it is launched: half a warp of
+// nodes per sub-partition, so that the four groups make two warps (N = 9000: quadrotor step 23.1 -> 17.0 us,
+// evaluation and KKT values 23.3 -> 19.1, cart-pole 11.1 -> 10.0 and 14.4 -> 12.8; N = 12000: 25.4 -> 21.7 and
+// 24.8 -> 21.3, but 11.8 -> 12.8 and 15.1 -> 14.5; N = 15000: 26.6 -> 25.6 and 25.7 -> 24.7, 11.5 -> 13.7 and 15.4 -> 16.0).
+template <class M, int TILE, unsigned OUT>
+constexpr bool split_kernel() { return TILE == TILE_SMALL && M::SPLIT && (OUT == O_ALL || OUT == O_STEP); }
+constexpr int SPLIT_NODES = 64;
+
 template <class M, int TILE, int NPT, unsigned OUT, bool PAR, bool IP>
 ocp_status launch_eval_ip(ocp* h, const EvalCall& c, NodeArgs<M>& a, cudaStream_t s) {
   a.x = c.x; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
@@ -1011,7 +1047,18 @@ ocp_status launch_eval_ip(ocp* h, const EvalCall& c, NodeArgs<M>& a, cudaStream_
   if (!(attr_done & (1u << (h->device & 31)))) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::bytes);
     if (e != cudaSuccess) return cuda_err(h, e, "cudaFuncSetAttribute(eval)");
+    if constexpr (split_kernel<M, TILE, OUT>()) {
+      e = cudaFuncSetAttribute(k_node_eval_split<M, TILE, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::bytes);
+      if (e != cudaSuccess) return cuda_err(h, e, "cudaFuncSetAttribute(eval)");
+    }
     attr_done |= 1u << (h->device & 31);
+  }
+  if constexpr (split_kernel<M, TILE, OUT>()) {
+    if (nodes <= (int64_t)SPLIT_NODES * h->num_sms) {
+      cudaError_t e = launch(true, k_node_eval_split<M, TILE, OUT>, dim3((unsigned)a.ntiles, OUT == O_STEP ? 4 : 2),
+                             TILE, S::bytes, s, a);
+      return cuda_err(h, e, "k_node_eval_split launch");
+    }
   }
   const int grid = occupancy_grid(h, (const void*)kern, TILE, S::bytes, a.ntiles);
   return cuda_err(h, launch(true, kern, grid, TILE, S::bytes, s, a), "k_node_eval launch");

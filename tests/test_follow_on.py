@@ -21,7 +21,7 @@ def test_every_overlapping_kernel_waits():
                 waits.add(k.group(1))
             else:
                 ordinary.add(k.group(1))
-    assert waits == {"k_node_eval", "k_node_jprod", "k_node_jtprod", "k_node_hprod", "k_euler", "k_god", "k_extra",
+    assert waits == {"k_node_eval", "k_node_eval_split", "k_node_jprod", "k_node_jtprod", "k_node_hprod", "k_euler", "k_god", "k_extra",
                      "k_heat_eval", "k_heat_jh", "k_heat_hprod", "k_heat_prod_unit", "k_kkt_values", "k_obj_grad",
                      "k_obj_hvp", "k_jtprod_coo", "k_jtprod_coo_long", "k_batch_eval"}
     assert not waits & ordinary
