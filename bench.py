@@ -88,7 +88,7 @@ FP64_OPS_PER_NODE = {("vdp", "eval_all"): 18.6, ("vdp", "jh"): 10.0, ("vdp", "jp
                      ("cartpole", "jtprod"): 45.0, ("cartpole", "hprod"): 50.0, ("cartpole", "step"): 101.6,
                      ("quadrotor", "eval_all"): 232.4, ("quadrotor", "jh"): 160.2, ("quadrotor", "jprod"): 95.3,
                      ("quadrotor", "jtprod"): 90.0, ("quadrotor", "hprod"): 104.0, ("quadrotor", "step"): 385.8,
-                     ("goddard", "eval_all"): 52.2, ("goddard", "jh"): 44.2, ("goddard", "jprod"): 41.2,
+                     ("goddard", "eval_all"): 56.2, ("goddard", "jh"): 44.2, ("goddard", "jprod"): 41.2,
                      ("goddard", "jtprod"): 42.2, ("goddard", "hprod"): 51.2, ("goddard", "step"): 97.3,
                      ("vdp:euler", "eval_all"): 13.5, ("vdp:euler", "jh"): 8.0, ("vdp:euler", "jprod"): 8.0,
                      ("vdp:euler", "jtprod"): 7.0, ("vdp:euler", "hprod"): 5.0, ("vdp:euler", "step"): 26.5,
@@ -110,7 +110,7 @@ KERNEL_SOURCES = {
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
 FP64_OPS_SRC = {"vdp": "3d06204e3134", "vdp:euler": "3d06204e3134", "cartpole": "83609fa71199",
-                "quadrotor": "3a5f809c5bc6", "goddard": "5cbd0c17e1b1", "heat64": "eb23ea47d260"}
+                "quadrotor": "3a5f809c5bc6", "goddard": "5cbd0c17e1b1", "heat64": "754c291ae75b"}
 
 
 def kernel_source_tag(key):
@@ -159,7 +159,7 @@ def named_workload(name):
 # DRAM bytes (read + write) of one launch at a workload, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; writes still dirty in L2 when the kernel ends
 # are not counted), with the source tag of the kernel it was captured on (see traffic()).
-TRAFFIC = {("vdp_mu_n1e6", "step"): (226.79e6, "3d06204e3134")}
+TRAFFIC = {("vdp_mu_n1e6", "step"): (226.52e6, "3d06204e3134")}
 # Each SM's FP64 pipe completes 2 FP64 instructions (one lane each) per clock: the recipe's
 # nominal 1.25 TFLOP/s FP64 of GB300 is 6.25e11 FMA/s = 1.99 per clock per SM at 152 SMs and
 # 2070 MHz.  bench.py measures the rate live (measure_fp64_rate) and reports it beside the peak.

@@ -764,12 +764,20 @@ ocp_status heat_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
 // Whether the fused step's products may run beside the evaluation's last CTAs.  They read nothing
 // that the evaluation writes and write nothing that it touches, unless the caller's arrays share
 // memory; then (and with path or boundary terms, whose launch comes between) they come after it.
-// 64 cells, N = 2e4: the evaluation's 646 CTAs leave SMs idle at their end, and the step takes
-// 80.1 us with the overlap, 97.1 without.
+// An SM holds HJ_CTAS of the products' CTAs, and it may be given all of them.  So they have to fill the chip
+// in any case (64 cells, N = 2e4: 2584 CTAs, the step 92.9 us in order, 79.3 so; 128 cells, N = 1e4: 103.4
+// and 93.6), or the SMs that the evaluation leaves without a CTA have to have room for them (64 cells, N = 3000:
+// 33.6 and 23.9; 8 cells, N = 3000: 25.6 and 16.7).  In between they crowd SMs beside the evaluation's CTAs and
+// slow these down: 14 cells, N = 9041: 28.6 us in order, 59.6 beside each other; 37 cells, N = 20000: 63.0 and 69.8 (but
+// 64 cells, N = 1e4: 57.2 and 46.8; limiting the CTAs per SM by their shared memory gained nothing: 63.8).
+constexpr int HJ_CTAS = 18;   // (the register cap of k_heat_prod_unit)
 bool heat_step_overlaps(const ocp* h, const EvalCall& e, const double* vn, const double* vm, const double* Jv,
                         const double* Jtv, const double* Hv) {
   const Pattern& P = h->pat;
   if (P.npath > 0 || P.nbin > 0 || h->has_bol) return false;
+  const int64_t tiles = (h->N + 1 + (HT_LANES - 2)) / (HT_LANES - 1), ctas = tiles * ((h->nx + HJ_CELLS - 1) / HJ_CELLS);
+  const int64_t free_sms = h->num_sms - tiles;
+  if (ctas < (int64_t)(HJ_CTAS - 2) * h->num_sms && ctas > HJ_CTAS * free_sms) return false;
   struct Range { const double* p; int64_t n; };
   const Range eval_in[] = {{e.x, P.n}, {e.y, P.m}};
   const Range eval_out[] = {{e.f, 1}, {e.c, P.m}, {e.g, P.n}, {e.jv, P.nnzj}, {e.hv, P.nnzh}};

@@ -35,7 +35,7 @@ def _separate(H, x, y, vn, vm):
     return [f, c, g, jv, hv, o1, o2, o3]
 
 
-@pytest.mark.parametrize("cells,N", [(2, 3), (17, 30), (64, 31 * 152), (37, 7003), (64, 20000)])
+@pytest.mark.parametrize("cells,N", [(2, 3), (17, 30), (64, 3000), (64, 31 * 152), (37, 7003), (64, 20000)])
 def test_heat_step_products_beside_the_evaluation(cells, N):
     H = _heat(cells, N)
     outs = _empty(H)
