@@ -29,6 +29,8 @@
  *     DEVICE pointers; the handle owns only its pattern tables and a small scratch area.
  *   - Calls are asynchronous on the given stream (a cudaStream_t passed as void*; NULL is
  *     the legacy default stream).  The status reports argument and launch errors only.
+ *     A kernel may be set up while the launch before it on the stream still runs; the stream's
+ *     order of reads and writes holds.
  *   - Calls on one handle must not overlap on the GPU (they share the handle's scratch);
  *     use one handle per concurrent stream.
  *   - No call aborts the process.  On failure the status is non-zero and
@@ -150,8 +152,8 @@ ocp_status ocp_set_scheme(ocp_t* h, int scheme);
  * come after the defects: row nb + nx N + p nun + i (nun = N+1, or N for Euler), bounds
  * (-inf, 0] in ocp_bounds.  Row (p, i) has one Jacobian entry per variable with a or l non-zero
  * (columns ascending); the squared terms add 2 a y on the Hessian diagonal of node i (the
- * entry becomes structural if it was not).  Every evaluation and product includes them (a
- * kernel after the model's on the same stream).  Rebuilds the pattern.  Not in the batched
+ * entry becomes structural if it was not).  Every evaluation and product includes them (one
+ * launch with the boundary terms, after the model's on the same stream).  Rebuilds the pattern.  Not in the batched
  * form.  Errors: OCP_EINVAL (bad counts, NULL or non-finite arrays, an empty row). */
 ocp_status ocp_set_path_constraints(ocp_t* h, int npath, const double* a, const double* b, const double* l,
                                     const double* r);
@@ -166,7 +168,7 @@ ocp_status ocp_set_path_constraints(ocp_t* h, int npath, const double* a, const 
  * entries); a squared term on component k adds 2 a y_q to the (k, k) Hessian entry of node 0
  * or node N, and (k, k) becomes structural in every node's block (the node blocks share one
  * template; the entry is zero at the other nodes).  Every evaluation, product and the KKT
- * assembly include them (one small kernel after the model's and the path rows' on the same
+ * assembly include them (in the path rows' launch, after the model's on the same
  * stream).  Trapezoidal scheme only (OCP_EMODEL with Euler, here or in ocp_set_scheme); not in
  * node ranges or the batched form (OCP_EMODEL).  Rebuilds the pattern.  Errors: OCP_EINVAL (bad
  * count, NULL or non-finite arrays, a row without variables). */
@@ -196,7 +198,7 @@ ocp_status ocp_set_final_components(ocp_t* h, int count, const int32_t* comps, c
  * nx + v is X_{N,v}); all three NULL remove it.  The gradient gains dg/dz at X_0 and X_N; the
  * Hessian gains sigma 2 a[v] on the (k, k) entry of node 0 or node N, and (k, k) becomes
  * structural in every node's block (zero at the other nodes).  Every evaluation, hprod and the
- * KKT assembly include it (one small kernel after the others on the same stream).  With the
+ * KKT assembly include it (in the launch of the path and boundary rows).  With the
  * Euler scheme the X_N terms must be linear (node N has no Hessian block): OCP_EMODEL here or
  * in ocp_set_scheme otherwise.  Not in node ranges, the batched form or the objective-only
  * kernels of the differentiation form (OCP_EMODEL).  Rebuilds the pattern.  Errors: OCP_EINVAL
@@ -281,7 +283,8 @@ ocp_status ocp_eval_all(ocp_t* h, const double* x, const double* y, double sigma
 /* The whole per-iteration evaluation in one pass over the nodes: everything of ocp_eval_all
  * plus the products Jv = J vn, Jtv = J^T vm and Hv = H(y, sigma) vn at the same x, sharing the
  * per-node derivative work and the loads of x and y (one launch for the node models; the heat
- * model runs two: its evaluation, then its three products in one).  vn has length n, vm length
+ * model runs two: its evaluation, and its three products in one that may run beside the evaluation's
+ * end).  vn has length n, vm length
  * m.  All arguments are
  * required.  Values are bit-identical to the separate calls. */
 ocp_status ocp_eval_step(ocp_t* h, const double* x, const double* y, double sigma, const double* vn,
