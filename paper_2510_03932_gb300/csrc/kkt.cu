@@ -50,7 +50,7 @@ struct KktArgs {
   const int32_t* boff;     // their supports: bv[boff[q] .. boff[q+1]) (local indices of (X_0, X_N))
   const int32_t* bv;
   int64_t N, n, m, nb, uoff, hbase_u, hbase_t, kb_xn, kb_u, kb_t, kb_c, nnzk;
-  double dw, dc;
+  double dw, ndc;
   int nx, nu, hx, hu, tx, tu, kx, ku, free_tf, euler, npath, nbin;
   int64_t nun, prow0;
   int16_t ksrc[2 * KKT_TMAX];  // X template then U template: source position or -1
@@ -85,7 +85,9 @@ __device__ __forceinline__ int kkt_comp(const KktArgs& a, int64_t s) {
 // first store: the gather is latency-bound otherwise.  Loads and stores are coalesced; the period of a
 // slot comes from a single-precision product (see kkt_div) instead of an integer division, and
 // the X / U templates sit in shared memory.  Moved values are copied bit for bit; the (1,1)
-// diagonal gets sigma_x + delta_w, the constraint diagonal is -delta_c.
+// diagonal gets sigma_x + delta_w, the constraint diagonal is -delta_c, negated on the host: in
+// the kernel every slot of the defect rows paid for the negation on the FP64 pipe (iteration of the quadrotor at
+// N = 1e5 94.0 us so, 92.1 now).
 constexpr int KKT_THREADS = 256, KKT_PER = 8;
 constexpr uint32_t KKT_SLOTS = KKT_THREADS * KKT_PER;
 enum { KR_X = 0, KR_U = 1, KR_TF = 2, KR_BND = 3, KR_DEF = 4, KR_XN = 5 };
@@ -116,7 +118,7 @@ __device__ __forceinline__ void kkt_block(const KktArgs& a, const KRegion& R, ui
     if (i >= n) continue;
     if constexpr (KIND == KR_DEF) {
       const uint32_t u = i + o0, jl = kkt_div(u, invP);
-      v[q] = (u - jl * P + 1 == P) ? -a.dc : __ldg(src + (u - jl));   // u - jl: the diagonals before this slot
+      v[q] = (u - jl * P + 1 == P) ? a.ndc : __ldg(src + (u - jl));   // u - jl: the diagonals before this slot
     } else if constexpr (ROWS) {
       const uint32_t u = i + o0, jl = kkt_div(u, invP), e = u - jl * P;
       const int sp = s_src[e];
@@ -132,7 +134,7 @@ __device__ __forceinline__ void kkt_block(const KktArgs& a, const KRegion& R, ui
     } else if constexpr (KIND == KR_XN) {   // Euler: the X rows of node N hold only their diagonal
       v[q] = (a.sx ? __ldg(a.sx + (int64_t)a.nx * a.N + s0 + i) : 0.0) + a.dw;
     } else {                                // boundary rows: the unit entry, then the diagonal
-      v[q] = ((s0 + i) & 1) ? -a.dc : __ldg(src + ((s0 + i) >> 1));
+      v[q] = ((s0 + i) & 1) ? a.ndc : __ldg(src + ((s0 + i) >> 1));
     }
   }
 #pragma unroll
@@ -347,7 +349,7 @@ ocp_status ocp_kkt_values(ocp_t* h, const double* hvals, const double* jvals, co
     return set_err(h, OCP_EINVAL, "arrays must be 8-byte aligned");
   KktArgs a;
   if (kkt_fill(h, a) != OCP_OK) return set_err(h, OCP_EDIM, "KKT matrix too large for the int32 interface");
-  a.hv = hvals; a.jv = jvals; a.sx = sigma_x; a.out = kvals; a.dw = delta_w; a.dc = delta_c;
+  a.hv = hvals; a.jv = jvals; a.sx = sigma_x; a.out = kvals; a.dw = delta_w; a.ndc = -delta_c;
   return cuda_err(h, launch(true, k_kkt_values, a.nblocks, KKT_THREADS, 0, (cudaStream_t)stream, a), "KKT values launch");
 }
 
