@@ -109,8 +109,8 @@ KERNEL_SOURCES = {
     "heat64": _COMMON + ["heat_kernels.cu"],
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
-FP64_OPS_SRC = {"vdp": "3d06204e3134", "vdp:euler": "3d06204e3134", "cartpole": "83609fa71199",
-                "quadrotor": "3a5f809c5bc6", "goddard": "5cbd0c17e1b1", "heat64": "754c291ae75b"}
+FP64_OPS_SRC = {"vdp": "1ae4d0001865", "vdp:euler": "1ae4d0001865", "cartpole": "7b7a5dd3ffae",
+                "quadrotor": "94ea9140168c", "goddard": "04ebb286082d", "heat64": "121b3eb2dbf3"}
 
 
 def kernel_source_tag(key):
@@ -159,7 +159,7 @@ def named_workload(name):
 # DRAM bytes (read + write) of one launch at a workload, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; writes still dirty in L2 when the kernel ends
 # are not counted), with the source tag of the kernel it was captured on (see traffic()).
-TRAFFIC = {("vdp_mu_n1e6", "step"): (226.52e6, "3d06204e3134")}
+TRAFFIC = {("vdp_mu_n1e6", "step"): (226.52e6, "1ae4d0001865")}
 # Each SM's FP64 pipe completes 2 FP64 instructions (one lane each) per clock: the recipe's
 # nominal 1.25 TFLOP/s FP64 of GB300 is 6.25e11 FMA/s = 1.99 per clock per SM at 152 SMs and
 # 2070 MHz.  bench.py measures the rate live (measure_fp64_rate) and reports it beside the peak.

@@ -1313,7 +1313,7 @@ template <class M>
 void fill_euler_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   fill_args<M>(h, sigma, a);
   M::host_consts(h->params.data(), h->h, a.K);   // the scheme's step is h (not h/2)
-  a.K.soft = soft_consts(a.K, M::NC);
+  a.K.soft = a.K.many && soft_consts(a.K, M::NC);
   a.B = 0;
   a.E = h->N + 1;
 }
