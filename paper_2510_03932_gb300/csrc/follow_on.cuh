@@ -18,14 +18,11 @@ __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.
 // Its launch, its CTAs' start and its parameters' loads run beside the end of the launch before it: about 2 us
 // of each short one (five callbacks of the cart-pole at N = 1e5 51.3 -> 41.8 us, three heat products of
 // 37 cells at N = 7003 30.8 -> 24.6, an iteration of the constrained quadrotor at N = 33333 55.5 -> 48.8).
-// A grid of few CTAs lets the next one in at once (Van der Pol step at N = 1000 8.0 -> 7.7 us); from
-// a larger one the next one's CTAs would crowd the SMs that this one leaves free, and FP64 work is
-// bound by the fullest SM (the callbacks above 56.1 us, the iteration 61.0).
-constexpr unsigned FEW_CTAS = 76;   // half of the SMs: two such grids fit one CTA to an SM
-__device__ __forceinline__ void start_follow_on() {
-  wait_for_previous();
-  if (gridDim.x * gridDim.y <= FEW_CTAS) let_next_start();
-}
+// A kernel lets the next one in by ending.  Let in from its start on, the next one's CTAs crowd the SMs that
+// it leaves free, and FP64 work is bound by the fullest SM (the callbacks above 56.1 us, the iteration
+// 61.0); from grids of at most 76 CTAs alone it gained nothing either (N = 1000: cart-pole callbacks 18.2 us
+// without and 19.2 with it, step 7.1 and 7.4, Van der Pol step 6.5 and 6.8).
+__device__ __forceinline__ void start_follow_on() { wait_for_previous(); }
 
 // The launch of `kernel`: beside the end of the launch before it, or in the ordinary way.
 inline cudaError_t launch_args(bool follow_on, const void* kernel, dim3 grid, int threads, size_t smem, cudaStream_t s,
