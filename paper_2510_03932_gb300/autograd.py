@@ -24,6 +24,7 @@ pointers.
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 
 from .ocp import OCP, _check, _raw_stream
 
@@ -139,7 +140,8 @@ class _Objective(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gF):
         (x,) = ctx.saved_tensors
-        if not torch.is_grad_enabled():
+        # (a cotangent with a forward-mode tangent goes through the function, which refuses it)
+        if not torch.is_grad_enabled() and forward_ad.unpack_dual(gF).tangent is None:
             return None, ctx.H.eval_grad_scaled(x, gF.reshape(1).contiguous())
         return None, _ObjGrad.apply(ctx.H, x, gF.reshape(1))
 
