@@ -61,8 +61,8 @@ struct GodArgs {
   int many, small;                   // large_launch, small_launch
 };
 
-// The inputs of node j's work that its products multiply (see soft_mul.cuh); no multipliers when H is not
-// asked for.
+// The inputs of node j's work that its products multiply (see soft_mul.cuh); no multipliers (NULL) when H
+// is not asked for.
 template <bool Y, bool YALL, bool V, bool W>
 __device__ __forceinline__ bool soft_god(const GodArgs& a, int64_t j) {
   const int64_t jl = max(j - 1, (int64_t)0), jr = min(j, a.N - 1);   // (as in soft_node)
@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(GT, god_ctas<OUT, IP, GT>()) k_god(const __gri
     if constexpr (SOFT != 0) {
       if (K0.soft && act) ok = soft_god<(WH || WHV), FREE, (WJV || WHV), WJTV>(a, j);
     }
-    with_products<SOFT>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
+    using Pipe = std::conditional_t<SOFT != 0 && (OUT & O_J) && (OUT & O_H), PipeConst, ModelConst>;
+    with_products<SOFT, Pipe>(K0, act, ok, [&](const auto& K) __attribute__((always_inline)) {
       const double r = __ldg(a.x + 3 * j), v = __ldg(a.x + 3 * j + 1), m = __ldg(a.x + 3 * j + 2);
       const double u = __ldg(a.x + a.uoff + j);
       if constexpr (NEEDF) {
@@ -504,7 +505,8 @@ ocp_status goddard_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s)
   GodArgs a;
   fill_god(h, a);
   if (2 * a.ntiles > h->max_partials) return set_err(h, OCP_EDIM, "too many tiles for the reduction scratch");
-  a.x = c.x; a.y = c.y; a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
+  a.x = c.x; a.y = (c.hv || c.ohv) ? c.y : nullptr;   // (not looked at without H)
+  a.f = c.f; a.c = c.c; a.g = c.g; a.jv = c.jv; a.hv = c.hv;
   a.vn = c.vn; a.vm = c.vm; a.ojv = c.ojv; a.ojtv = c.ojtv; a.ohv = c.ohv;
   cudaError_t e;
   if (a.p_dev) {  // device parameters: the constraints alone

@@ -55,6 +55,17 @@ struct SoftConst : ModelConst {
   __device__ __forceinline__ explicit SoftConst(const ModelConst& k) : ModelConst(k), worst(0u) {}
 };
 
+// The constants of a node's work on the FP64 pipe beside the integer products' body in one kernel, with
+// sums and products that the compiler cannot form a second time: for the Goddard model's fused kernels,
+// whose register caps had it repeat some FMAs (all outputs 107.7 instead of 98.6 a node).  N = 2e5 with a
+// zero in every warp, plain FMAs and these: step 81.3 and 77.5 us, all outputs 47.8 and 45.1, those without
+// H 34.6 and 31.5, J + H 39.5 and 39.0 (ordinary inputs 63.7 and 62.6, 34.7 and 33.9, 25.5 and 24.6, 29.7 and
+// 28.7).  The kernels of one output repeat none (J^T w, zeros, 31.4 and 32.0; quadrotor J^T w, N = 1e5, 24.1
+// and 25.4).
+struct PipeConst : ModelConst {
+  __device__ __forceinline__ explicit PipeConst(const ModelConst& k) : ModelConst(k) {}
+};
+
 // h/2 and the first n model constants: non-zero and of moderate size
 __host__ __device__ __forceinline__ bool soft_consts(const ModelConst& K, int n) {
   auto hi = [](const double& v) {
@@ -88,6 +99,15 @@ __device__ __forceinline__ double fmul(const SoftConst<MASK>& K, double a, doubl
   K.worst = max(K.worst, x - SOFT_BASE);   // (unsigned: sums below the range wrap to large values)
   return r;
 }
+__device__ __forceinline__ double pipe_fma(double a, double b, double c) {
+  double r;
+  asm("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(c));
+  return r;
+}
+__device__ __forceinline__ double fadd(const PipeConst& K, double a, double b) { return pipe_fma(a, K.one, b); }
+__device__ __forceinline__ double fsub(const PipeConst& K, double a, double b) { return pipe_fma(-b, K.one, a); }
+template <unsigned C = MUL_P>
+__device__ __forceinline__ double fmul(const PipeConst& K, double a, double b) { return pipe_fma(a, b, K.mz); }
 // c * v, c a cost weight or diagonal that may be zero for the whole launch (a zero with the product's sign)
 template <unsigned C>
 __device__ __forceinline__ double fmul_w(const ModelConst& K, double c, double v) { return fmul<C>(K, c, v); }

@@ -23,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "model_base.cuh"
 #include "follow_on.cuh"
 #include "ocp_internal.h"
@@ -482,9 +484,9 @@ __device__ __forceinline__ void prefetch_node(const NodeArgs<M>& a, const double
 }
 
 // Runs work(K) for the lanes with `act`, with the products of SoftConst where the warp's inputs
-// (ok) allow it and none came out of range, else (or again) with ModelConst: the same values, bit
+// (ok) allow it and none came out of range, else (or again) with PIPE, a ModelConst: the same values, bit
 // for bit.  Called by whole warps.
-template <unsigned SOFT, class F>
+template <unsigned SOFT, class PIPE = ModelConst, class F>
 __device__ __forceinline__ void with_products(const ModelConst& K, bool act, bool ok, F&& work) {
   bool done = false;
   if constexpr (SOFT != 0) {
@@ -494,7 +496,14 @@ __device__ __forceinline__ void with_products(const ModelConst& K, bool act, boo
       done = __all_sync(0xffffffffu, KS.worst <= SOFT_SPAN);
     }
   }
-  if (!done && act) work(K);
+  if (!done && act) {
+    if constexpr (std::is_same_v<PIPE, ModelConst>) {
+      work(K);
+    } else {
+      const PIPE KP(K);
+      work(KP);
+    }
+  }
 }
 
 // One tile of the fused evaluation.  The CTA's TILE threads cover NPT*TILE consecutive
