@@ -264,7 +264,7 @@ static ocp_status batch_upload_inst(ocp_batch* b) {
   std::vector<NodeArgs<M>> inst(b->count);
   for (int i = 0; i < b->count; ++i) {
     fill_args<M>(b->items[i], 1.0, inst[i]);
-    inst[i].K.many = b->many;   // (the instances share one launch)
+    inst[i].K.many = b->many && finite_cost(b->items[i]);   // (the instances share one launch)
     inst[i].K.soft = inst[i].K.many && soft_consts(inst[i].K, M::NC);
     inst[i].B = 0;
     inst[i].E = b->items[i]->N + 1;

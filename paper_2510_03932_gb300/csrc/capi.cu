@@ -44,6 +44,13 @@ int occupancy_grid(ocp* h, const void* kernel, int threads, size_t smem, int64_t
   return (int)work_tiles;
 }
 
+bool finite_cost(const ocp* h) {
+  for (const auto* v : {&h->q, &h->r, &h->xref, &h->uref})
+    for (double e : *v)
+      if (!std::isfinite(e)) return false;
+  return true;
+}
+
 int64_t objective_tiles(int model, int64_t nodes) {
   int owned = 0;
   switch (model) {

@@ -694,7 +694,7 @@ static void heat_fill(const ocp* h, double sigma, HeatArgs& a) {
   a.counter = h->d_counter;
   // (a thread takes eight cells of a node, so a node counts n / 8 times)
   auto fits = [](double v) { return v >= 0x1p-64 && v < 0x1p64; };
-  a.soft = large_launch((h->N + 1) * (int64_t)n / 8, h->num_sms) && fits(a.h6);
+  a.soft = large_launch((h->N + 1) * (int64_t)n / 8, h->num_sms) && fits(a.h6) && finite_cost(h);
 }
 
 // Calls fn with the number of warps as a compile-time constant.

@@ -37,8 +37,8 @@ struct ModelConst {
   double one;      // 1.0 and -0.0, passed at run time (see fadd / fmul below)
   double mz;
   double c[16];    // model-specific precomputed constants (see each model)
-  int soft;        // this launch uses integer products (large_launch and soft_consts)
-  int many;        // large_launch alone (for parameters that are read on the device)
+  int soft;        // this launch uses integer products (many and soft_consts)
+  int many;        // large_launch and finite_cost (for parameters that are read on the device)
 };
 
 // Classes of a node's plain products: intermediates of the dynamics, entries of the Jacobian, of

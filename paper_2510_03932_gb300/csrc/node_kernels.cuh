@@ -993,7 +993,7 @@ void fill_args(const ocp* h, double sigma, NodeArgs<M>& a) {
   a.has_final = h->has_final ? 1 : 0;
   a.has_ref = h->has_ref ? 1 : 0;
   M::host_consts(h->params.data(), h->hh, a.K);
-  a.K.many = large_launch(h->N + 1, h->num_sms);
+  a.K.many = large_launch(h->N + 1, h->num_sms) && finite_cost(h);
   a.K.soft = a.K.many && soft_consts(a.K, M::NC);
   for (int v = 0; v < M::NZ; ++v) {
     const double w = v < M::NX ? h->q[v] : h->r[v - M::NX];

@@ -175,6 +175,9 @@ ocp_status cuda_err(ocp* h, cudaError_t e, const char* what);
 // more nodes they only make more CTAs and partial sums (N = 30000: Van der Pol 10.9 -> 11.9).
 inline bool large_launch(int64_t nodes, int num_sms) { return nodes >= (int64_t)256 * num_sms; }
 inline bool small_launch(int64_t nodes, int num_sms) { return nodes <= (int64_t)128 * num_sms; }
+// Whether the cost's weights and references are finite: a zero weight on a NaN or infinite difference, or
+// the other way round, gives NaN only from the FP64 pipe's products.
+bool finite_cost(const ocp* h);
 int occupancy_grid(ocp* h, const void* kernel, int threads, size_t smem, int64_t work_tiles);
 
 // Host pattern compiler.
