@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import concurrent.futures as cf
 import glob
+import hashlib
 import os
 import subprocess
 import sys
@@ -41,9 +42,22 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(d) <= t for d in _deps())
 
 
+def kernels_tag(extra=()) -> str:
+    """Tag of the kernels that a batch runs: their sources and flags.  Part of the key of the batch autotuning
+    cache, so that timings of other kernels are not taken for these."""
+    h = hashlib.sha256(" ".join(ARCH + list(extra)).encode())
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) +
+                       [os.path.join(CSRC, "batch.cu"), os.path.abspath(__file__)]):
+        with open(path, "rb") as fh:
+            h.update(os.path.basename(path).encode() + b"\0" + fh.read() + b"\0")
+    return h.hexdigest()[:12]
+
+
 def _compile(src: str, extra: list[str], objdir: str = OUT) -> str:
     obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
     cmd = [NVCC] + FLAGS + extra + ["-c", src, "-o", obj]
+    if os.path.basename(src) == "batch.cu":
+        cmd.append('-DOCP_KERNELS_TAG="%s"' % kernels_tag(extra))
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))

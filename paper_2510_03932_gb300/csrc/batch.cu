@@ -208,9 +208,13 @@ struct ocp_batch : ocp_batch_impl {};
 
 // Autotuning cache (OCP_AUTOTUNE_CACHE = path of a text file): one line per tuned batch shape,
 // "key<TAB>threads npt ctas_per_sm ms", the key naming the model, the instance count, the total
-// and the largest horizon, the requested outputs and the GPU (SM count, compute capability).
+// and the largest horizon, the requested outputs, the GPU (SM count, compute capability) and the kernels
+// (build.py's tag of their sources: a time taken with others says nothing about these).
 // A batch of a shape already in the file takes the stored configuration without timing; the
 // last line of a key wins.  Lines that do not parse are ignored.
+#ifndef OCP_KERNELS_TAG
+#define OCP_KERNELS_TAG __DATE__ "," __TIME__
+#endif
 static std::mutex g_tune_mu;
 
 static std::string tune_key(const ocp_batch* b, unsigned outs) {
@@ -220,8 +224,8 @@ static std::string tune_key(const ocp_batch* b, unsigned outs) {
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, b->device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, b->device);
   char buf[256];
-  std::snprintf(buf, sizeof(buf), "model=%d count=%d nodes=%lld maxnodes=%lld outputs=%u sms=%d cc=%d.%d", b->model,
-                b->count, (long long)nodes, (long long)maxn, outs, b->num_sms, major, minor);
+  std::snprintf(buf, sizeof(buf), "model=%d count=%d nodes=%lld maxnodes=%lld outputs=%u sms=%d cc=%d.%d kernels=%s",
+                b->model, b->count, (long long)nodes, (long long)maxn, outs, b->num_sms, major, minor, OCP_KERNELS_TAG);
   return buf;
 }
 
