@@ -1026,9 +1026,12 @@ template <class M, int TILE>
 constexpr bool ip_tile() { return TILE != TILE_SMALL || TILE == M::PROD_TILE; }
 
 // Whether the launch takes the integer-product instance of its kernel (the device reads the parameters
-// itself with PAR, and tests the constants made of them there).
+// itself with PAR, and tests the constants made of them there).  A gradient written over x (each entry
+// needs only its own variable) keeps the FP64 pipe's: a warp could not do such nodes again.
 template <class M, unsigned OUT, bool PAR>
-bool soft_choice(const NodeArgs<M>& a) { return M::template SOFT<OUT> != 0 && (PAR ? a.K.many : a.K.soft); }
+bool soft_choice(const NodeArgs<M>& a, const double* x = nullptr, const double* g = nullptr) {
+  return M::template SOFT<OUT> != 0 && (PAR ? a.K.many : a.K.soft) && !(OUT == O_G && x == g);
+}
 
 // Models and outputs with a split kernel, and the nodes per SM up to which it is launched: half a warp of
 // nodes per sub-partition, so that the four groups make two warps (N = 9000: quadrotor step 23.1 -> 17.0 us,
@@ -1078,7 +1081,7 @@ ocp_status launch_eval_k(ocp* h, const EvalCall& c, cudaStream_t s) {
   NodeArgs<M> a;
   fill_args<M>(h, c.sigma, a);
   if constexpr (ip_tile<M, TILE>() && M::template SOFT<OUT> != 0) {
-    if (soft_choice<M, OUT, PAR>(a)) return launch_eval_ip<M, TILE, NPT, OUT, PAR, true>(h, c, a, s);
+    if (soft_choice<M, OUT, PAR>(a, c.x, c.g)) return launch_eval_ip<M, TILE, NPT, OUT, PAR, true>(h, c, a, s);
   }
   return launch_eval_ip<M, TILE, NPT, OUT, PAR, false>(h, c, a, s);
 }
@@ -1305,7 +1308,7 @@ ocp_status launch_euler_ip(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
 template <class M, int TILE, unsigned OUT, bool PAR>
 ocp_status launch_euler_k(ocp* h, NodeArgs<M>& a, cudaStream_t s) {
   if constexpr (ip_tile<M, TILE>() && M::template SOFT<OUT> != 0) {
-    if (soft_choice<M, OUT, PAR>(a)) return launch_euler_ip<M, TILE, OUT, PAR, true>(h, a, s);
+    if (soft_choice<M, OUT, PAR>(a, a.x, a.g)) return launch_euler_ip<M, TILE, OUT, PAR, true>(h, a, s);
   }
   return launch_euler_ip<M, TILE, OUT, PAR, false>(h, a, s);
 }
