@@ -59,6 +59,14 @@ ocp_status ocp_probe_sincos_table(const double* x, double* s, double* c, double*
  * asynchronous on `stream`).  Errors: OCP_EINVAL, OCP_ECUDA (ocp_last_error(NULL)). */
 ocp_status ocp_probe_exp_table(const double* x, double* e, double* e_lib, int64_t n, void* stream);
 
+/* The kernels' FP64 product on the integer pipes: r[i] = a[i] b[i] so, r64[i] by the FP64 pipe, and
+ * in_range[i] = 1 where the kernels take the former (the operands' exponents add up to at most 400 in
+ * magnitude; a zero, subnormal, infinite or NaN operand beside one below 2^600 and above 2^-600
+ * comes out of that range).  n device entries each; asynchronous on `stream`.  Errors: OCP_EINVAL,
+ * OCP_ECUDA (ocp_last_error(NULL)). */
+ocp_status ocp_probe_product(const double* a, const double* b, double* r, double* r64, double* in_range, int64_t n,
+                             void* stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -89,7 +89,30 @@ __global__ void k_probe_exp(const double* x, double* e, double* el, int64_t n,
   }
 }
 
+// The integer pipes' product of a[i] and b[i], the FP64 pipe's, and whether the former is in its range.
+__global__ void k_probe_product(const double* a, const double* b, double* r, double* r64, double* in_range, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    uint32_t x;
+    r[i] = ocpg::soft_product(a[i], b[i], x);
+    in_range[i] = x - ocpg::SOFT_BASE <= ocpg::SOFT_SPAN ? 1.0 : 0.0;
+    r64[i] = a[i] * b[i];
+  }
+}
+
 }  // namespace
+
+extern "C" ocp_status ocp_probe_product(const double* a, const double* b, double* r, double* r64, double* in_range, int64_t n,
+                                        void* stream) {
+  OCP_RANGE();
+  const double* p[5] = {a, b, r, r64, in_range};
+  for (const double* q : p)
+    if (!q || ((uintptr_t)q & 7u)) return ocpg::set_err(nullptr, OCP_EINVAL, "ocp_probe_product: bad pointer");
+  if (n < 0) return ocpg::set_err(nullptr, OCP_EINVAL, "ocp_probe_product: n < 0");
+  if (n == 0) return OCP_OK;
+  const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
+  k_probe_product<<<grid, 256, 0, (cudaStream_t)stream>>>(a, b, r, r64, in_range, n);
+  return ocpg::cuda_err(nullptr, cudaGetLastError(), "ocp_probe_product launch");
+}
 
 extern "C" ocp_status ocp_probe_exp_table(const double* x, double* e, double* e_lib, int64_t n, void* stream) {
   OCP_RANGE();

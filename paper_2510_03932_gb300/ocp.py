@@ -101,6 +101,7 @@ _SIGS = {
     "ocp_probe_sincos": [_P, _P, _P, _P, _P, _I64, _P],
     "ocp_probe_sincos_table": [_P, _P, _P, _P, _P, _I64, _P],
     "ocp_probe_exp_table": [_P, _P, _P, _I64, _P],
+    "ocp_probe_product": [_P, _P, _P, _P, _P, _I64, _P],
     "ocp_set_fault": [C.c_char_p],
     "ocp_last_error": [_P],
 }
@@ -175,6 +176,18 @@ def probe_exp(x, stream=None):
     _check(lib().ocp_probe_exp_table(*[C.c_void_p(t.data_ptr()) for t in [x] + outs], int(x.numel()),
                                      _stream(stream)))
     return tuple(outs)
+
+
+def probe_product(a, b, stream=None):
+    """ocp_probe_product: the integer pipes' products of the CUDA float64 tensors a and b, the FP64
+    pipe's, and 1.0 where the former are in their range."""
+    for t in (a, b):
+        if t.dtype != torch.float64 or not t.is_cuda or not t.is_contiguous() or t.numel() != a.numel():
+            raise TypeError("a and b must be contiguous float64 CUDA tensors of one size")
+    outs = [torch.empty_like(a) for _ in range(3)]
+    _check(lib().ocp_probe_product(*[C.c_void_p(t.data_ptr()) for t in [a, b] + outs], int(a.numel()),
+                                   _stream(stream)))
+    return outs
 
 
 def sum_ordered(parts, out, stream=None):
