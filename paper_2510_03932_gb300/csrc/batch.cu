@@ -58,10 +58,10 @@ struct BatchArgs {
   int count;
 };
 
-// Resident CTAs that the registers are capped for: as many threads as the plain evaluation's (the
-// cart-pole batch of 6.5e6 nodes 1042 us at 72 registers, 1433 at the allocator's 126).
+// Resident CTAs that the registers are capped for, with integer products (each model's threads per SM from
+// measurements of its own).
 template <class M, int TILE, bool IP>
-constexpr int batch_ctas() { return soft_kernel<M, O_ALL, IP>() ? M::template CTAS<O_ALL> * M::EVAL_TILE / TILE : 0; }
+constexpr int batch_ctas() { return soft_kernel<M, O_ALL, IP>() ? M::BATCH_THREADS / TILE : 0; }
 
 template <class M, int TILE, int NPT, bool IP>
 __global__ void __launch_bounds__(TILE, batch_ctas<M, TILE, IP>()) k_batch_eval(const __grid_constant__ BatchArgs<M> b) {

@@ -42,6 +42,9 @@ struct CartPole {
       OUT == O_STEP ? 5 : (OUT == O_ALL || OUT == (O_J | O_H) || OUT == O_H) ? 7 : (OUT == O_JTV || OUT == O_HV) ? 6 : 0;
   template <unsigned OUT> static constexpr int CTAS_FP64 = OUT == O_G ? 6 : 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  // threads per SM that the batch kernel's registers are capped for: 72 registers (6.5e6 nodes: 1042 us; 1433 at the
+  // allocator's 126)
+  static constexpr int BATCH_THREADS = 7 * 128;
   static constexpr int PROD_TILE = TILE_CARTPOLE;
   static constexpr bool SPLIT = true;   // k_node_eval_split in the smallest launches
   static constexpr int EVAL_TILE = TILE_CARTPOLE;

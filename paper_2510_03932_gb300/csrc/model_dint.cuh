@@ -14,6 +14,7 @@ struct Dint {
   template <unsigned OUT> static constexpr unsigned SOFT = 0u;  // (see soft_kernel)
   template <unsigned OUT> static constexpr int CTAS_FP64 = 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  static constexpr int BATCH_THREADS = 0;  // (no integer products in its evaluation)
   static constexpr int PROD_TILE = TILE_DINT;
   static constexpr bool SPLIT = false;  // (a node's work is short)
   static constexpr int EVAL_TILE = TILE_DINT;

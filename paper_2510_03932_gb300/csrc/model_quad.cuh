@@ -44,6 +44,7 @@ struct Quadrotor {
       (OUT == O_JV || OUT == O_JTV || OUT == O_HV) ? 8 : OUT == O_H ? 4 : 0;
   template <unsigned OUT> static constexpr int CTAS_FP64 = (OUT == O_JV || OUT == O_JTV || OUT == O_HV) ? 0 : 3;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = OUT == O_STEP ? 3 : 0;  // (N = 50000: 69.2 us uncapped, 51.5)
+  static constexpr int BATCH_THREADS = 0;  // (no integer products in its evaluation)
   static constexpr int PROD_TILE = TILE_QUAD;
   static constexpr bool SPLIT = true;   // k_node_eval_split in the smallest launches
   static constexpr int EVAL_TILE = TILE_QUAD_EVAL;

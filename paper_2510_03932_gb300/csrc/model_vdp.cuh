@@ -25,6 +25,10 @@ struct VdP {
   template <unsigned OUT> static constexpr int CTAS = OUT == O_STEP ? 5 : (OUT == O_ALL || OUT == O_F) ? 8 : 0;
   template <unsigned OUT> static constexpr int CTAS_FP64 = 0;   // without integer products
   template <unsigned OUT> static constexpr int CTAS_EULER = 0;
+  // threads per SM that the batch kernel's registers are capped for: 40 registers (256 problems, 6.46e6 nodes:
+  // 334 us; 393 at the plain evaluation's 32, 327 at 48, 343 at the allocator's choice; with y = 0, F and
+  // c 310, 312, 321 and 331; 16 problems, 48000 nodes: 10.5, 13.0, 10.1 and 10.1)
+  static constexpr int BATCH_THREADS = 6 * 256;
   static constexpr int PROD_TILE = TILE_VDP;
   static constexpr bool SPLIT = false;  // (a node's work is short)
   static constexpr int EVAL_TILE = TILE_VDP;
