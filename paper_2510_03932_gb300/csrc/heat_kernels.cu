@@ -708,6 +708,8 @@ static cudaError_t with_warps(int w, Fn&& fn) {
   }
 }
 
+constexpr int HEAT_STEP_CARVEOUT = 81;   // percent of 228 KB: 18 CTAs of the products, 9 KB and 1 KB of the system's each
+
 template <unsigned OUT>
 static ocp_status heat_eval_t(ocp* h, const EvalCall& c, cudaStream_t s) {
   HeatArgs a;
@@ -726,6 +728,15 @@ static ocp_status heat_eval_t(ocp* h, const EvalCall& c, cudaStream_t s) {
     constexpr int W = decltype(w)::value;
     auto kern = (MUL && a.soft) ? k_heat_eval<OUT, MUL, W> : k_heat_eval<OUT, false, W>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if constexpr (OUT == O_ALL) {
+      // An SM splits its memory between L1 and shared memory for the kernel that it runs, and takes CTAs that
+      // need another split only when it is empty.  The products' CTAs ask for 18 x 10 KB, and beside an
+      // evaluation of fewer than 64 cells, which gets less, they all went to the SMs without one (16
+      // cells, N = 4300: 36.9 us, 27.8 in order, 20.5 with this split).
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 c.products_beside && a.ntiles <= h->num_sms ? HEAT_STEP_CARVEOUT : cudaSharedmemCarveoutDefault);
+    }
     if (e != cudaSuccess) return e;
     return launch(!c.products_beside, kern, occupancy_grid(h, (const void*)kern, 32 * W, smem, a.ntiles), 32 * W, smem, s, a);
   };
@@ -764,20 +775,21 @@ ocp_status heat_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
 // Whether the fused step's products may run beside the evaluation's last CTAs.  They read nothing
 // that the evaluation writes and write nothing that it touches, unless the caller's arrays share
 // memory; then (and with path or boundary terms, whose launch comes between) they come after it.
-// An SM holds HJ_CTAS of the products' CTAs, and it may be given all of them.  So they have to fill the chip
-// in any case (64 cells, N = 2e4: 2584 CTAs, the step 92.9 us in order, 79.3 so; 128 cells, N = 1e4: 103.4
-// and 93.6), or the SMs that the evaluation leaves without a CTA have to have room for them (64 cells, N = 3000:
-// 33.6 and 23.9; 8 cells, N = 3000: 25.6 and 16.7).  In between they crowd SMs beside the evaluation's CTAs and
-// slow these down: 14 cells, N = 9041: 28.6 us in order, 59.6 beside each other; 37 cells, N = 20000: 63.0 and 69.8 (but
-// 64 cells, N = 1e4: 57.2 and 46.8; limiting the CTAs per SM by their shared memory gained nothing: 63.8).
+// With at most one evaluation CTA per SM they always do: heat_eval_t splits those SMs' memory so that the
+// products' CTAs find room on all of them (2 to 128 cells, N = 60 to 4650, 119 sizes: 0.48 to 0.89 of
+// the time in order; 64 cells, N = 3000: 33.6 and 22.7 us).  With more, FP64 work is bound by the fullest
+// SM, and the products' CTAs crowd some of them (14 cells, N = 9041: 28.6 us in order, 59.6 beside each other; 37
+// cells, N = 20000: 63.0 and 69.8; but 64 cells, N = 1e4: 57.2 and 46.8), unless they fill the chip in any
+// case, HJ_CTAS on every SM or nearly so: at 16 to 24 per SM 0.76 to 1.05 of the time in order (64 cells,
+// N = 2e4, 17 per SM: 92.9 us in order, 79.3 so; 128 cells, N = 1e4: 103.4 and 93.6; 33 cells, N = 28000: 83.0 and
+// 86.1), at 14 and 15 0.88 to 1.07 (50 cells, N = 16500).
 constexpr int HJ_CTAS = 18;   // (the register cap of k_heat_prod_unit)
 bool heat_step_overlaps(const ocp* h, const EvalCall& e, const double* vn, const double* vm, const double* Jv,
                         const double* Jtv, const double* Hv) {
   const Pattern& P = h->pat;
   if (P.npath > 0 || P.nbin > 0 || h->has_bol) return false;
   const int64_t tiles = (h->N + 1 + (HT_LANES - 2)) / (HT_LANES - 1), ctas = tiles * ((h->nx + HJ_CELLS - 1) / HJ_CELLS);
-  const int64_t free_sms = h->num_sms - tiles;
-  if (ctas < (int64_t)(HJ_CTAS - 2) * h->num_sms && ctas > HJ_CTAS * free_sms) return false;
+  if (tiles > h->num_sms && ctas < (int64_t)(HJ_CTAS - 2) * h->num_sms) return false;
   struct Range { const double* p; int64_t n; };
   const Range eval_in[] = {{e.x, P.n}, {e.y, P.m}};
   const Range eval_out[] = {{e.f, 1}, {e.c, P.m}, {e.g, P.n}, {e.jv, P.nnzj}, {e.hv, P.nnzh}};
