@@ -349,7 +349,9 @@ __global__ void __launch_bounds__(GT, god_ctas<OUT, IP, GT>()) k_god(const __gri
           a.g[a.uoff + j] = 0.0;
           if (FREE && j == 0) a.g[a.tau] = 0.0;
         }
-        if (sF && bnd && j == N) *a.f = fma(a.mayer[0], r, fma(a.mayer[1], v, fmul(K, a.mayer[2], m)));
+        // (by the FP64 pipe: a weight is often zero, and an integer product of it would come out of range and have
+        // the last node's warp work twice, 4 us on the end of the launch)
+        if (sF && bnd && j == N) *a.f = fma(a.mayer[0], r, fma(a.mayer[1], v, fma(a.mayer[2], m, a.mz)));
         if (j == 0) {
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
