@@ -51,6 +51,8 @@ bool finite_cost(const ocp* h) {
   return true;
 }
 
+// Objective tiles of a launch that is not small (small launches have tiles of TILE_SMALL nodes, a few hundred at
+// most): what ocp_eval_obj_noalloc holds its scratch against.
 int64_t objective_tiles(int model, int64_t nodes) {
   int owned = 0;
   switch (model) {

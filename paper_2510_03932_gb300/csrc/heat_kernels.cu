@@ -8,9 +8,9 @@
 // each side, plus the control for k = 0, so 6 entries per row except the last cell's 4.
 //
 // Work decomposition: a CTA covers 32 consecutive nodes (one per lane); in the evaluation and
-// H v its 8 warps take the cells in groups of 8, while the J + H values, Jv and J^T w run two
-// warps per CTA on units of 16 cells of a tile (four times as many CTAs, the same number on
-// every SM).  Row-coupled outputs (defects, Jacobian rows) use tiles that overlap by one node
+// H v its one, two, four or eight warps (heat_warps) take the cells in groups of 8, while the
+// J + H values, Jv and J^T w run two warps per CTA on units of 16 cells of a tile (at 64 cells four
+// times as many CTAs, the same number on every SM).  Row-coupled outputs (defects, Jacobian rows) use tiles that overlap by one node
 // (the CTA owns 31 of its 32 nodes); node-local products use disjoint tiles.
 // The states of the tile's nodes are staged in shared memory with a padded row (n+1 doubles)
 // so that lanes reading different nodes hit different banks; node-major outputs (Hessian

@@ -6,7 +6,7 @@ namespace ocpg {
 
 // Threads (= nodes) per CTA of the node-model kernels; a tile owns TILE-1 nodes.
 constexpr int TILE_VDP = 256, TILE_CARTPOLE = 128, TILE_DINT = 256, TILE_QUAD = 64;
-// ... and in small launches (large_launch): two warps per CTA.
+// ... and in small launches (small_launch): two warps per CTA.
 constexpr int TILE_SMALL = 64;
 // The quadrotor's evaluation kernels (F, c, g, J, H and the fused step) run 128-node tiles with
 // three CTAs per SM at its register cap, its product kernels 64-node tiles (measured at N = 1e6:

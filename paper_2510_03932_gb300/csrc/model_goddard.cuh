@@ -13,7 +13,6 @@ namespace ocpg {
 // the dedicated free-final-time kernels (goddard_kernels.cu).
 // ------------------------------------------------------------------------------------
 struct Goddard {
-  static constexpr int EVAL_MIN_CTAS = 0;
   static constexpr int NX = 3, NU = 1, NZ = 4;
   static constexpr int MAXRX = 3, MAXRU = 1;
   OCP_TABLE1(RX, int, NX, {2, 3, 1})

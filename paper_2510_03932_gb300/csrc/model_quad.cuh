@@ -42,7 +42,7 @@ struct Quadrotor {
   // spill), H alone 4 (188 us; 203 at 3); of 64 for the products: 8
   template <unsigned OUT> static constexpr int CTAS =
       (OUT == O_JV || OUT == O_JTV || OUT == O_HV) ? 8 : OUT == O_H ? 4 : 0;
-  template <unsigned OUT> static constexpr int CTAS_FP64 = (OUT == O_JV || OUT == O_JTV || OUT == O_HV) ? 0 : 3;   // without integer products
+  template <unsigned OUT> static constexpr int CTAS_FP64 = 3;   // without integer products (evaluation kernels)
   template <unsigned OUT> static constexpr int CTAS_EULER = OUT == O_STEP ? 3 : 0;  // (N = 50000: 69.2 us uncapped, 51.5)
   static constexpr int BATCH_THREADS = 0;  // (no integer products in its evaluation)
   static constexpr int PROD_TILE = TILE_QUAD;

@@ -418,7 +418,8 @@ template <class M, unsigned OUT, bool IP>
 constexpr unsigned soft_kernel() { return IP ? M::template SOFT<OUT> : 0u; }
 
 // Resident CTAs per SM that a kernel's registers are capped for (0: the allocator's own choice).
-// (The two-warp CTAs of small launches may take every register they ask for.)
+// (Two-warp CTAs with FP64 products alone, those of small launches and the quadrotor's product kernels in
+// middle ones, may take every register they ask for.)
 template <class M, int TILE, unsigned OUT, bool IP, bool EULER = false>
 constexpr int min_ctas() {
   if (soft_kernel<M, OUT, IP>()) return M::template CTAS<OUT>;

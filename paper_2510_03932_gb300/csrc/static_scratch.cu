@@ -21,7 +21,8 @@
 
 using namespace ocpg;
 
-// Maximum number of reduction tiles: 65536 tiles of 31 (heat) to 255 (Van der Pol) nodes.
+// Maximum number of reduction tiles: 65536 tiles of 31 (heat) to 255 (Van der Pol) nodes.  (Small launches have
+// tiles of 63, a few hundred at most.)
 // The array holds the ticket in its first 256 bytes and one partial sum per tile after it.
 #define OCP_NOALLOC_MAX_TILES 65536
 static __device__ __align__(256) double g_noalloc_scratch[32 + OCP_NOALLOC_MAX_TILES];
