@@ -196,9 +196,11 @@ __device__ __forceinline__ void heat_finish(const HeatArgs& a, double* red) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  // a warp takes the places of HT_WARPS / W warps at once, sixteen loads before the first sum (a lone warp that
+  // a warp takes the places of HT_WARPS / W warps at once, eight or sixteen loads before the first sum (a lone warp that
   // took them in turn, a load at a time, was the longest part of eval_obj: 5 cells, N = 1e5, 25.0 us so, 16.8 now)
-  constexpr int PER = HT_WARPS / W, DEPTH = 16 / PER;
+  // (eight warps, also those of launches with few tiles, take one load at a time: each further sum of zeros costs them
+  // 64 cycles)
+  constexpr int PER = HT_WARPS / W, DEPTH = PER == 1 ? 1 : PER > 4 ? 16 / PER : 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double s[PER] = {};
   for (int64_t i0 = 32 * warp + lane; i0 < a.ntiles; i0 += DEPTH * HT_THREADS) {
