@@ -93,8 +93,8 @@ FP64_OPS_PER_NODE = {("vdp", "eval_all"): 18.6, ("vdp", "jh"): 10.0, ("vdp", "jp
                      ("vdp:euler", "eval_all"): 13.5, ("vdp:euler", "jh"): 8.0, ("vdp:euler", "jprod"): 8.0,
                      ("vdp:euler", "jtprod"): 7.0, ("vdp:euler", "hprod"): 5.0, ("vdp:euler", "step"): 26.5,
                      # heat, 64 cells: the step is its evaluation and one launch of Jv, J^T w and H v
-                     ("heat64", "eval_all"): 866.0, ("heat64", "jh"): 262.4, ("heat64", "jprod"): 391.5,
-                     ("heat64", "jtprod"): 463.0, ("heat64", "hprod"): 129.1, ("heat64", "step"): 1723.7}
+                     ("heat64", "eval_all"): 865.8, ("heat64", "jh"): 262.4, ("heat64", "jprod"): 391.5,
+                     ("heat64", "jtprod"): 463.0, ("heat64", "hprod"): 129.1, ("heat64", "step"): 1723.5}
 
 # The kernel sources of each model key (paths under the package's csrc/): the tile body and
 # the helpers it includes, the model's device functor, the translation unit that instantiates
@@ -110,7 +110,7 @@ KERNEL_SOURCES = {
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
 FP64_OPS_SRC = {"vdp": "8da4dac21ad1", "vdp:euler": "8da4dac21ad1", "cartpole": "12bc1e221f01",
-                "quadrotor": "5314f1a415b6", "goddard": "3f9fb0d0770d", "heat64": "8e28a3a4cb08"}
+                "quadrotor": "5314f1a415b6", "goddard": "3f9fb0d0770d", "heat64": "c39638c045d5"}
 
 
 def kernel_source_tag(key):
@@ -159,7 +159,7 @@ def named_workload(name):
 # DRAM bytes (read + write) of one launch at a workload, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; writes still dirty in L2 when the kernel ends
 # are not counted), with the source tag of the kernel it was captured on (see traffic()).
-TRAFFIC = {("vdp_mu_n1e6", "step"): (226.64e6, "8da4dac21ad1")}
+TRAFFIC = {("vdp_mu_n1e6", "step"): (226.60e6, "8da4dac21ad1")}
 # Each SM's FP64 pipe completes 2 FP64 instructions (one lane each) per clock: the recipe's
 # nominal 1.25 TFLOP/s FP64 of GB300 is 6.25e11 FMA/s = 1.99 per clock per SM at 152 SMs and
 # 2070 MHz.  bench.py measures the rate live (measure_fp64_rate) and reports it beside the peak.

@@ -750,11 +750,12 @@ static ocp_status heat_eval_t(ocp* h, const EvalCall& c, cudaStream_t s) {
     if constexpr (OUT == O_ALL) {
       // An SM splits its memory between L1 and shared memory for the kernel that it runs, and takes CTAs that
       // need another split only when it is empty.  The products' CTAs ask for 18 x 10 KB, and beside an
-      // evaluation of fewer than 64 cells, which gets less, they all went to the SMs without one (16
-      // cells, N = 4300: 36.9 us, 27.8 in order, 20.5 with this split).
+      // evaluation of fewer than 64 cells, whose five CTAs fit in a split of 164 KB, they all went to the SMs
+      // without one (16 cells, N = 4300: 36.9 us, 27.8 in order, 20.5 with their split).
+      const bool ask = c.products_beside && a.ntiles <= h->num_sms && 5 * (smem + 1024) <= 164 * 1024;
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 c.products_beside && a.ntiles <= h->num_sms ? HEAT_STEP_CARVEOUT : cudaSharedmemCarveoutDefault);
+                                 ask ? HEAT_STEP_CARVEOUT : cudaSharedmemCarveoutDefault);
     }
     if (e != cudaSuccess) return e;
     return launch(!c.products_beside, kern, occupancy_grid(h, (const void*)kern, 32 * W, smem, a.ntiles), 32 * W, smem, s, a);
@@ -794,7 +795,7 @@ ocp_status heat_eval(ocp* h, unsigned out, const EvalCall& c, cudaStream_t s) {
 // Whether the fused step's products may run beside the evaluation's last CTAs.  They read nothing
 // that the evaluation writes and write nothing that it touches, unless the caller's arrays share
 // memory; then (and with path or boundary terms, whose launch comes between) they come after it.
-// With at most one evaluation CTA per SM they always do: heat_eval_t splits those SMs' memory so that the
+// With at most one evaluation CTA per SM they always do: heat_eval_t has those SMs' memory split so that the
 // products' CTAs find room on all of them (2 to 128 cells, N = 60 to 4650, 119 sizes: 0.48 to 0.89 of
 // the time in order; 64 cells, N = 3000: 33.6 and 22.7 us).  With more, FP64 work is bound by the fullest
 // SM, and the products' CTAs crowd some of them (14 cells, N = 9041: 28.6 us in order, 59.6 beside each other; 37
