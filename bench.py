@@ -88,8 +88,8 @@ FP64_OPS_PER_NODE = {("vdp", "eval_all"): 18.6, ("vdp", "jh"): 10.0, ("vdp", "jp
                      ("cartpole", "jtprod"): 45.0, ("cartpole", "hprod"): 50.0, ("cartpole", "step"): 101.6,
                      ("quadrotor", "eval_all"): 232.4, ("quadrotor", "jh"): 160.2, ("quadrotor", "jprod"): 95.3,
                      ("quadrotor", "jtprod"): 90.0, ("quadrotor", "hprod"): 104.0, ("quadrotor", "step"): 385.8,
-                     ("goddard", "eval_all"): 55.2, ("goddard", "jh"): 42.1, ("goddard", "jprod"): 41.2,
-                     ("goddard", "jtprod"): 42.2, ("goddard", "hprod"): 51.2, ("goddard", "step"): 96.3,
+                     ("goddard", "eval_all"): 55.3, ("goddard", "jh"): 42.2, ("goddard", "jprod"): 41.2,
+                     ("goddard", "jtprod"): 42.2, ("goddard", "hprod"): 51.2, ("goddard", "step"): 96.4,
                      ("vdp:euler", "eval_all"): 13.5, ("vdp:euler", "jh"): 8.0, ("vdp:euler", "jprod"): 8.0,
                      ("vdp:euler", "jtprod"): 7.0, ("vdp:euler", "hprod"): 5.0, ("vdp:euler", "step"): 26.5,
                      # heat, 64 cells: the step is its evaluation and one launch of Jv, J^T w and H v
@@ -110,7 +110,7 @@ KERNEL_SOURCES = {
 }
 # Tags of the sources the FP64_OPS_PER_NODE counts (and TRAFFIC) were measured on.
 FP64_OPS_SRC = {"vdp": "8da4dac21ad1", "vdp:euler": "8da4dac21ad1", "cartpole": "12bc1e221f01",
-                "quadrotor": "5314f1a415b6", "goddard": "3f9fb0d0770d", "heat64": "c39638c045d5"}
+                "quadrotor": "5314f1a415b6", "goddard": "3228eccf23b8", "heat64": "c39638c045d5"}
 
 
 def kernel_source_tag(key):
@@ -159,7 +159,7 @@ def named_workload(name):
 # DRAM bytes (read + write) of one launch at a workload, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum; writes still dirty in L2 when the kernel ends
 # are not counted), with the source tag of the kernel it was captured on (see traffic()).
-TRAFFIC = {("vdp_mu_n1e6", "step"): (226.60e6, "8da4dac21ad1")}
+TRAFFIC = {("vdp_mu_n1e6", "step"): (226.64e6, "8da4dac21ad1")}
 # Each SM's FP64 pipe completes 2 FP64 instructions (one lane each) per clock: the recipe's
 # nominal 1.25 TFLOP/s FP64 of GB300 is 6.25e11 FMA/s = 1.99 per clock per SM at 152 SMs and
 # 2070 MHz.  bench.py measures the rate live (measure_fp64_rate) and reports it beside the peak.

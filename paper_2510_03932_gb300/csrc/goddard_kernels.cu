@@ -68,8 +68,8 @@ __device__ __forceinline__ bool soft_god(const GodArgs& a, int64_t j) {
   const int64_t jl = max(j - 1, (int64_t)0), jr = min(j, a.N - 1);   // (as in soft_node)
   bool ok = soft_input(a.x + a.uoff + j);
   if (V) ok &= soft_input(a.vn + a.uoff + j);
-  // (r = 1: the drag's exponent is zero and exp_tab squares its remainder)
-  ok &= __double_as_longlong(__ldg(a.x + 3 * j)) != 0x3ff0000000000000ll;
+  // (r = 1, by the high word: within 2^-20 above: the drag's exponent is zero and exp_tab squares its remainder)
+  ok &= __ldg(reinterpret_cast<const uint32_t*>(a.x + 3 * j) + 1) != 0x3ff00000u;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     ok &= soft_input(a.x + 3 * j + k);
